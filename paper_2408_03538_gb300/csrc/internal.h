@@ -48,6 +48,7 @@ int sh_table(int S, int order, const float* dirs, float* Y, cudaStream_t stream)
 struct TraceArgs;
 // packet.cu
 int launch_packet(const TraceArgs& a, float* V, bool bounce, int sms, cudaStream_t stream);
+size_t packet_search_bytes(int64_t batch, int S);
 
 size_t transfer_backward_workspace(int64_t n, const prtgs_transfer_params* p);
 // dP [n,C] and dV [n,S] (extra dLoss/dV per ray, e.g. from the glossy matrices) are both nullable

@@ -5,16 +5,26 @@
 // of the scene. One warp takes such a packet: the lanes walk the LBVH together, testing up to
 // 32 nodes per step against the packet's beam (the rectangle the packet's origins span in the
 // plane orthogonal to the direction, and the depth range along it that the lanes still need),
-// and collect the leaves the beam meets in a shared-memory chunk. Each leaf of a chunk is then
-// tested by every lane whose own ray can meet its box, with the same per-ray hit test and the
-// same visitors as the per-ray walks in transfer.cu, so every hit decision, product and
-// index-matrix rule is that of a single ray; only the traversal is shared.
+// and collect the leaves the beam meets in a shared-memory chunk. The leaves of a chunk are staged 32
+// at a time, those whose own ellipse misses the beam are dropped, every lane takes a cheap conservative
+// test of the rest, and only what passes it is tested exactly; every hit decision, product and
+// index-matrix rule is that of a single ray, only the traversal is shared.
+//
+// What bounds it: issue slots and the latency of the node steps (about 40 % of the time), with L2 serving
+// the tree; a walk of surface-100k meets 1,300 nodes and 820 boxes of leaves, of which 560 leaves are
+// tested and 270 are hit by one of the 30 rays (9 of them each). Measured against testing every leaf
+// exactly, in step: surface-100k with bounces 77.4 -> 60.2 ms, a 60k volume 30.2 -> 24.1 ms, the million
+// splats with bounces and glossy matrices 1.037 -> 0.908 s. Tried and left out: the tree projected once
+// per direction (surface-100k 62.8 -> 62.8 ms before the search had its own kernel, but the million
+// splats 1.17 s: a direction's tree no longer fits the L2, and a launch per few directions ends with a
+// millisecond of few busy warps).
 //
 //  k_packet<B>    visibility V_is of every (receiver, direction) of a receiver batch into
 //                 V[s][i] (Eq. 4 along a ray, Eq. 27 read as the Gaussian's maximum); with B
-//                 (bounce) also the index matrix of Sec. 4.4: the visibility walk finds the
-//                 horizon and the nearest front-facing hit, then search rounds walk the hits
-//                 from there in key order until the argmax of W_j (Eq. 26) is settled.
+//                 (bounce) also the horizon, the nearest front-facing hit and, where that settles
+//                 it, the index matrix of Sec. 4.4.
+//  k_search       the rest of the index matrix: rounds over the hits in key order until the argmax
+//                 of W_j (Eq. 26) is settled.
 //  k_project      P_i = sum_s (4 pi / S) V_is max(0, n_i.w_s) Y(w_s) (Eq. 29 with Eq. 9),
 //                 one lane per receiver, compensated sums; also copies V of glossy receivers.
 #include "trace.cuh"
@@ -25,27 +35,21 @@ constexpr int kPacketWarps = 4;
 constexpr int kPacketThreads = 32 * kPacketWarps;
 constexpr int kPStack = 384;     // node stack of a warp (ints)
 #ifndef PRTGS_PACKET_ROUND_HITS
-#define PRTGS_PACKET_ROUND_HITS 14  // 14 keeps the bounce kernel at 4 blocks per SM (16: 3 blocks)
+// k_search at 4 blocks per SM: surface-100k transfer 60.3 ms at 14 hits, 58.1 at 18, 57.3 at 20, 61.2 at 24
+#define PRTGS_PACKET_ROUND_HITS 20
 #endif
 constexpr int kPacketRoundHits = PRTGS_PACKET_ROUND_HITS;  // hits per index-matrix search round
 #ifndef PRTGS_PACKET_LEAVES
 #define PRTGS_PACKET_LEAVES 224
 #endif
 #ifndef PRTGS_PACKET_MIN_BLOCKS
-#define PRTGS_PACKET_MIN_BLOCKS 4  // the visibility-only kernel fits 4 blocks per SM without spills
+#define PRTGS_PACKET_MIN_BLOCKS 5  // visibility only: a 60k volume at 128 directions 24.6 ms at 4, 24.1 at 5, 24.7 at 6
 #endif
 // leaf chunk of a warp (> 64: a step appends up to 64 leaves; flushed past kPLeaves - 64). Longer
-// chunks flush less often: 1M bounce transfer 1.085 s at 96, 0.988 s at 128, 0.970 s at 160,
-// 0.962 s at 192, 0.957 s at 224 (4 blocks per SM still fit at S = 256)
+// chunks flush less often: 1M bounce transfer 1.085 s at 96, 0.988 s at 128, 0.957 s at 224 (as measured
+// when the index search still ran in the same kernel; now surface-100k 57.8 ms at 160, 57.3 at 224).
+// The chunk also sets when the beam shrinks, and with it the order in which hits are met.
 constexpr int kPLeaves = PRTGS_PACKET_LEAVES;
-#ifndef PRTGS_PACKET_UNROLL
-#define PRTGS_PACKET_UNROLL 0
-#endif
-#ifndef PRTGS_PACKET_BOUNCE_UNROLL
-#define PRTGS_PACKET_BOUNCE_UNROLL 8
-#endif
-constexpr int kPUnrollVis = PRTGS_PACKET_UNROLL;            // leaves tested together (0: one by one): visibility walk
-constexpr int kPUnrollBounce = PRTGS_PACKET_BOUNCE_UNROLL;  // ... bounce and index-search walks
 // wide pops (32 nodes) only while the stack keeps room for their pushes plus a full one-node-
 // at-a-time descent of the deepest possible tree (64 levels)
 constexpr int kPHeadroom = 64 + 64 + 4;
@@ -57,16 +61,21 @@ constexpr int kPacketDirs = 1;
 struct PacketSmem {
   int stack[kPStack];
   int lpos[kPLeaves];      // the chunk's leaves (sorted positions)
-  float4 stage[32][4];     // a group of leaves, staged: the exact-test terms of stage_leaf
-  // the work item's window of 64 receivers: record row 0 (mean, opacity), scene root, Gaussian
-  // index; and, per direction, the window slots of the receivers that face it
-  float4 wq0[64];
-  int wroot[64], wgid[64];
-  int rlist[64];
+  float4 stage[4][32];     // a group of leaves, staged: the exact-test terms of stage_leaf, term-major (the
+                           // lanes of a drain read different leaves: 16-byte stride, few bank conflicts)
+  float4 quick[2][32];     // ... and the terms of the quick test
+  // the window slots of the receivers that face the direction
+  unsigned char rlist[64];
 };
-// Bounce mode, per warp after the PacketSmem array: the search round's nearest hits of each lane,
-// hits[k][lane] = (t*, position, alpha, m).
-using RoundHits = float4[kPacketRoundHits][32];
+
+// k_search, per warp after the PacketSmem array: the search round's nearest hits of each lane,
+// t*, position, and alpha with the sign bit set for a front-facing hit (m > 0; m itself is formed
+// again from the record by the few hits that need it: 12 bytes a hit leave room for 20 of them).
+struct RoundHits {
+  float t[kPacketRoundHits][32];
+  int pos[kPacketRoundHits][32];
+  float sal[kPacketRoundHits][32];
+};
 
 // Orthonormal frame (e1, e2, w) around a unit direction w (Duff et al. 2017, "Building an
 // orthonormal basis, revisited": the branchless form).
@@ -97,15 +106,16 @@ struct Beam {
   float xlo, xhi, ylo, yhi, zlo, zhi;
 };
 
+// Over the full warp, one instruction each (NaN inputs are ignored).
 __device__ __forceinline__ float warp_min(float v) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, off));
-  return v;
+  float r;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
 }
 __device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
-  return v;
+  float r;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+  return r;
 }
 
 __device__ __forceinline__ Beam make_beam(bool need, float xl, float yl, float zlo, float zhi) {
@@ -135,6 +145,7 @@ __device__ __forceinline__ Beam make_beam(bool need, float xl, float yl, float z
 // play in the per-ray test.
 struct Rel {
   float Rx, Ry, Rz;        // reference point (warp-uniform)
+  float Rxl, Ryl, Rzl;     // ... and its place on the frame
   float xr, xr_lo, yr, yr_lo;  // this lane's origin minus R on e1, e2, each as an unevaluated sum hi + lo
   float zr;                // ... and on w
 };
@@ -164,6 +175,9 @@ __device__ __forceinline__ Rel make_rel(const Frame& f, float ox0, float oy0, fl
   rel.Rx = Rx;
   rel.Ry = Ry;
   rel.Rz = Rz;
+  rel.Rxl = fmaf(f.e1x, Rx, fmaf(f.e1y, Ry, f.e1z * Rz));
+  rel.Ryl = fmaf(f.e2x, Rx, fmaf(f.e2y, Ry, f.e2z * Rz));
+  rel.Rzl = fmaf(f.wx, Rx, fmaf(f.wy, Ry, f.wz * Rz));
   float ox, oy, oz, lox, loy, loz;
   two_sum(ox0, -Rx, ox, lox);
   two_sum(oy0, -Ry, oy, loy);
@@ -179,12 +193,19 @@ __device__ __forceinline__ Rel make_rel(const Frame& f, float ox0, float oy0, fl
   return rel;
 }
 
-// Stage one leaf for the packet: (p on e1, e2 (high parts), R - mu on w; opacity), (A e1 x a; m1),
-// (A e2 x a; m2), (facing term max(-w.n_j, 0); sorted position; p on e1, e2 (low parts)).
-__device__ __forceinline__ void stage_leaf(const float4* __restrict__ recs, int pos, const Frame& f, const Rel& rel,
-                                           float4* out) {
-  const float4 q0 = __ldg(recs + 4 * pos), q1 = __ldg(recs + 4 * pos + 1), q2 = __ldg(recs + 4 * pos + 2),
-               q3 = __ldg(recs + 4 * pos + 3);
+__device__ __forceinline__ float facing(const Frame& f, const float4& q3) {
+  return fmaxf(-fmaf(f.wx, q3.y, fmaf(f.wy, q3.z, f.wz * q3.w)), 0.0f);
+}
+
+// Stage 32 leaves for the packet, one per lane (pos < 0: none), and return how many were kept: a leaf
+// whose own 3-sigma ellipse misses the beam is dropped (of the leaves whose box meets it, two in five).
+// Per leaf: (p on e1, e2 (high parts), R - mu on w; opacity), (A e1 x a; m1), (A e2 x a; m2), (facing term
+// max(-w.n_j, 0); sorted position; p on e1, e2 (low parts)), and the quick test's terms (quick_mask), for
+// which X, Y bound the lanes' |xr|, |yr|. et: the largest error bound of the quick t.
+__device__ __forceinline__ int stage_leaves(const float4* __restrict__ recs, int pos, const Frame& f, const Rel& rel,
+                                            const Beam& bm, float X, float Y, PacketSmem& sm, float& et) {
+  const float4* rec = recs + 4 * (int64_t)max(pos, 0);
+  const float4 q0 = __ldg(rec), q1 = __ldg(rec + 1), q2 = __ldg(rec + 2), q3 = __ldg(rec + 3);
   // R - mu = h + l exactly; p = R - mu + t_ref w, the offset of mu from the point of the reference
   // ray nearest to it, formed with one rounding per component (the product t_ref w is exact inside
   // the FMA): D^2 does not change along w, so the lanes use p in place of R - mu, and its projections
@@ -228,12 +249,51 @@ __device__ __forceinline__ void stage_leaf(const float4* __restrict__ recs, int 
   const float id = 1.0f / sqrtf(dd);
   const float ax = adx * id, ay = ady * id, az = adz * id;
   const float idd = 1.0f / dd;
-  out[0] = make_float4(cx, cy, cz, q0.w);
-  out[1] = make_float4(diff_prod(b1y, az, b1z, ay), diff_prod(b1z, ax, b1x, az), diff_prod(b1x, ay, b1y, ax),
-                       fmaf(b1x, adx, fmaf(b1y, ady, b1z * adz)) * idd);
-  out[2] = make_float4(diff_prod(b2y, az, b2z, ay), diff_prod(b2z, ax, b2x, az), diff_prod(b2x, ay, b2y, ax),
-                       fmaf(b2x, adx, fmaf(b2y, ady, b2z * adz)) * idd);
-  out[3] = make_float4(fmaxf(-fmaf(f.wx, q3.y, fmaf(f.wy, q3.z, f.wz * q3.w)), 0.0f), __int_as_float(pos), cxl, cyl);
+  const float4 s1 = make_float4(diff_prod(b1y, az, b1z, ay), diff_prod(b1z, ax, b1x, az), diff_prod(b1x, ay, b1y, ax),
+                                fmaf(b1x, adx, fmaf(b1y, ady, b1z * adz)) * idd);
+  const float4 s2 = make_float4(diff_prod(b2y, az, b2z, ay), diff_prod(b2z, ax, b2x, az), diff_prod(b2x, ay, b2y, ax),
+                                fmaf(b2x, adx, fmaf(b2y, ady, b2z * adz)) * idd);
+  // quick test: D^2 = |dx B1 + dy B2|^2 = u^2 + v^2, u = l11 dx + l21 dy, v = l22 dy (Cholesky of the
+  // Gram matrix of B1, B2; both are orthogonal to a, so l22 |B1| = |(B1 x B2) . a|). Every coefficient
+  // is off by a few ulp of |B1| or |B2|, so u and v are off by at most e below; a leaf that meets
+  // D^2 <= 9 then has u^2 + v^2 <= 9 + 12 e + 2 e^2. All are scaled so that this bound is 1.
+  const float g11 = fmaf(s1.x, s1.x, fmaf(s1.y, s1.y, s1.z * s1.z));
+  const float g12 = fmaf(s1.x, s2.x, fmaf(s1.y, s2.y, s1.z * s2.z));
+  const float cr = fmaf(s1.y * s2.z - s1.z * s2.y, ax, fmaf(s1.z * s2.x - s1.x * s2.z, ay, (s1.x * s2.y - s1.y * s2.x) * az));
+  const float rl = rsqrtf(g11);
+  const float c11 = g11 * rl, c21 = g12 * rl, c22 = fabsf(cr) * rl;
+  const float Xc = X + fabsf(cx), Yc = Y + fabsf(cy);
+  const float e = 2e-6f * fmaf(c11, Xc, (fabsf(c21) + c22) * Yc);
+  const float sc = rsqrtf(9.01f + fmaf(12.0f, e, 2.0f * e * e));
+  const float l11 = c11 * sc, l21 = c21 * sc, l22 = c22 * sc;
+  // t* + zr = -cz - dx m1 - dy m2, off by at most et (widened by it: a hit ahead of the origin stays so)
+  const float ter = 2e-6f * (fabsf(cz) + fmaf(fabsf(s1.w), Xc, fabsf(s2.w) * Yc));
+  // the ellipse u^2 + v^2 <= 1 holds |dy| <= 1 / l22, |dx| <= |(l21, l22)| / (l11 l22) and
+  // |dx m1 + dy m2| <= |L^-1 m|; its centre is at (-cx, -cy, -cz) from R. A NaN keeps the leaf.
+  bool keep = pos >= 0;
+  {
+    const float i11 = __fdividef(1.0f, l11), i22 = __fdividef(1.0f, l22);
+    const float k21 = l21 * i22, w1 = s1.w * i11, w2 = (s2.w - l21 * w1) * i22;
+    const float m = 3e-5f * (1.0f + fabsf(rel.Rx) + fabsf(rel.Ry) + fabsf(rel.Rz) + fabsf(cx) + fabsf(cy) + fabsf(cz));
+    const float rx = 1.001f * i11 * sqrtf(fmaf(k21, k21, 1.0f)) + m, ry = 1.001f * i22 + m;
+    const float rz = 1.001f * sqrtf(fmaf(w1, w1, w2 * w2)) + 1e-3f * (fabsf(s1.w) * rx + fabsf(s2.w) * ry) + m;
+    const float ox = rel.Rxl - cx, oy = rel.Ryl - cy, oz = rel.Rzl - cz;  // the centre on the frame
+    keep = keep && !(ox + rx < bm.xlo) && !(ox - rx > bm.xhi) && !(oy + ry < bm.ylo) && !(oy - ry > bm.yhi) &&
+           !(oz + rz < bm.zlo) && !(oz - rz > bm.zhi);
+  }
+  const unsigned m = __ballot_sync(0xffffffffu, keep);
+  const int slot = __popc(m & ((1u << (threadIdx.x & 31)) - 1u));
+  if (keep) {
+    sm.stage[0][slot] = make_float4(cx, cy, cz, q0.w);
+    sm.stage[1][slot] = s1;
+    sm.stage[2][slot] = s2;
+    sm.stage[3][slot] = make_float4(facing(f, q3), __int_as_float(pos), cxl, cyl);
+    sm.quick[0][slot] = make_float4(l11, l21, fmaf(l11, cx, l21 * cy), ter - cz - fmaf(cx, s1.w, cy * s2.w));
+    sm.quick[1][slot] = make_float4(l22, l22 * cy, s1.w, s2.w);
+  }
+  et = warp_max(keep ? ter : 0.0f);
+  __syncwarp();
+  return __popc(m);
 }
 
 // Projection of a box [lo, hi] on the frame: centre and half-width along e1, e2 and w, widened
@@ -263,34 +323,47 @@ __device__ __forceinline__ bool beam_meets(const Beam& b, const float4& A, const
 // The exact test of one staged leaf for the lane: D^2 and t* (see Rel). The high parts of dx
 // cancel without rounding error of their own beyond eps |dx| (exactly where they nearly cancel);
 // the low parts carry the roundings of both.
-__device__ __forceinline__ void leaf_test(const Rel& rel, const float4* e, float& d2, float& t) {
-  const float4 s0 = e[0], s1 = e[1], s2 = e[2], s3 = e[3];
+__device__ __forceinline__ void leaf_test(const Rel& rel, const PacketSmem& sm, int j, float& d2, float& t) {
+  const float4 s0 = sm.stage[0][j], s1 = sm.stage[1][j], s2 = sm.stage[2][j], s3 = sm.stage[3][j];
   const float dx = (rel.xr + s0.x) + (rel.xr_lo + s3.z), dy = (rel.yr + s0.y) + (rel.yr_lo + s3.w);
   const float wx = fmaf(dx, s1.x, dy * s2.x), wy = fmaf(dx, s1.y, dy * s2.y), wz = fmaf(dx, s1.z, dy * s2.z);
   d2 = fmaf(wx, wx, fmaf(wy, wy, wz * wz));
   t = -(rel.zr + s0.z) - fmaf(dx, s1.w, dy * s2.w);
 }
 
-// Hand one passing leaf test over to the visitor (the receiver's own Gaussian excepted).
-template <class Vis>
-__device__ __forceinline__ bool hand_over(const float4* e, int self, float d2, float t, Vis& vis, RayStats& st) {
-  const float4 s3 = e[3];
-  const int pos = __float_as_int(s3.y);
-  if (pos == self) return false;
-  ++st.hits;
-  vis.hit(pos, t, e[0].w * expf(-0.5f * d2), s3.x);
-  return true;
+// Quick test of the staged leaves for the lane: bit j of the result is set for every leaf j < cnt whose
+// exact test can pass (and for a few more). Two 16-byte loads, seven FMAs and three comparisons per
+// leaf, no branch; a NaN passes on to the exact test. zlo: tlo + zr, zhi: thn + zr, both widened.
+__device__ __forceinline__ unsigned quick_mask(const PacketSmem& sm, int cnt, float x, float y, float zlo, float zhi) {
+  unsigned pass = 0u;
+#pragma unroll 1
+  for (int j0 = 0; j0 < cnt; j0 += 8) {
+    unsigned m = 0u;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const float4 a = sm.quick[0][j0 + k], b = sm.quick[1][j0 + k];
+      const float u = fmaf(a.x, x, fmaf(a.y, y, a.z));
+      const float v = fmaf(b.x, y, b.y);
+      const float d = fmaf(u, u, v * v);
+      const float t = fmaf(-b.z, x, fmaf(-b.w, y, a.w));
+      if (!(d > 1.0f) && !(t <= zlo) && !(t > zhi)) m |= 1u << k;
+    }
+    pass |= m << j0;
+  }
+  return cnt < 32 ? pass & ((1u << cnt) - 1u) : pass;
 }
 
 // One packet walk. Lane state: `active` (this lane's ray takes part), its projected origin
 // (xl, yl) and depth zl (for the beam), its offset from the packet's reference point (rel, for the
 // exact test), the lower bound t_lo of the hits it wants (0: all hits ahead) and its visitor, whose
 // t_hi() bounds the hits it still wants and stop() ends its ray. The leaves of a chunk are staged
-// 32 at a time (one record load and the per-Gaussian terms of the exact test per lane), then every
-// lane tests its ray against each of them (the test of Rel above) and hands the hits to
-// vis.hit(), in chunk order.
-template <int UNROLL, class Vis>
-__device__ void packet_walk(const TraceArgs& a, const Frame& f, const Ray& r, const Rel& rel, int self, int root,
+// 32 at a time (one record load and the per-Gaussian terms of the tests per lane). Every lane then
+// takes the quick test of all of them into a 32-bit mask, without a branch, and drains its mask: the
+// exact test (of Rel above) and, for the hits, vis.hit(), in chunk order. A leaf is hit by about a
+// tenth of the lanes, so walking the leaves in step and branching to the visitor would run it with
+// three lanes of 32; in the drain every lane is at a hit of its own.
+template <class Vis>
+__device__ void packet_walk(const TraceArgs& a, const Frame& f, const Rel& rel, int self, int root,
                             bool active, float xl, float yl, float zl, float t_lo, Vis& vis, PacketSmem& sm,
                             RayStats& st, unsigned& node_count) {
   const int lane = threadIdx.x & 31;
@@ -302,12 +375,11 @@ __device__ void packet_walk(const TraceArgs& a, const Frame& f, const Ray& r, co
   const float zlo_l = t_lo > 0.f ? zl + (t_lo * (1.0f - 1e-5f) - 1e-6f) : zl;
   bool need = active && !vis.stop();
   if (!__any_sync(0xffffffffu, need) || root == INT32_MIN) return;
-  if (root < 0) {  // a one-Gaussian scene
-    if (need) vis.leaf(~root);
-    return;
-  }
+  if (root < 0) return;  // a one-Gaussian scene: the receiver alone
   float th = vis.t_hi();
   Beam bm = make_beam(need, xl, yl, zlo_l, th == FLT_MAX ? FLT_MAX : zl + th);
+  const float X = warp_max(need ? fabsf(rel.xr) : 0.0f), Y = warp_max(need ? fabsf(rel.yr) : 0.0f);
+  const float zlo_q = (tlo + rel.zr) - 2e-6f * (tlo + fabsf(rel.zr));
   int sp = 1, nl = 0;
   if (lane == 0) sm.stack[0] = root;
   __syncwarp();
@@ -325,11 +397,10 @@ __device__ void packet_walk(const TraceArgs& a, const Frame& f, const Ray& r, co
       if (lane == 0) node_count += npop;
       bool push0 = false, push1 = false, leaf0 = false, leaf1 = false;
       int c0 = 0, c1 = 0;
-      float4 A0, A1;
-      float2 Z0, Z1;
       bool near0 = true;
       if (node >= 0) {
-        float4 n0, n1, n2;
+        float4 n0, n1, n2, A0, A1;
+        float2 Z0, Z1;
         load_node(a.nodes, node, n0, n1, n2, c0, c1);
         project_box(f, n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, A0, Z0);
         project_box(f, n1.z, n1.w, n2.x, n2.y, n2.z, n2.w, A1, Z1);
@@ -365,53 +436,42 @@ __device__ void packet_walk(const TraceArgs& a, const Frame& f, const Ray& r, co
     }
     if (nl > kPLeaves - 64 || (sp == 0 && nl > 0)) {
       for (int g = 0; g < nl; g += 32) {
-        // stage: lane j forms the exact-test terms of leaf g + j
-        if (g + lane < nl) stage_leaf(a.recs, sm.lpos[g + lane], f, rel, sm.stage[lane]);
-        __syncwarp();
-        const int cnt = min(32, nl - g);
+        float et;
+        const int cnt = stage_leaves(a.recs, g + lane < nl ? sm.lpos[g + lane] : -1, f, rel, bm, X, Y, sm, et);
         if (lane == 0) st.entries += cnt;
-        // per leaf only the test itself; the bookkeeping (the receiver's own Gaussian, the
-        // visitor's bound th, whether the lane still wants hits) waits for a passing test, which
-        // is rare (a few percent of the leaves); th only falls, and changes only at a hand-over.
-        // UNROLL > 0 tests UNROLL leaves at a time (independent chains) and hands the passing
-        // ones over in order, each test taken again by the same arithmetic (bit-identical)
-        // against the current th: one copy of the visitor's code serves the whole block, which
-        // pays where that code is long (the bounce and index-search visitors).
         if (need) st.leaves += cnt;  // leaf tests of the lane (its own Gaussian included)
         float thn = need ? th : -FLT_MAX;  // a lane that wants no hits passes no test
-        if constexpr (UNROLL == 0) {
-          for (int j = 0; j < cnt; ++j) {
+        const float zhi_q = need ? (thn + rel.zr) + (2.0f * et + 2e-6f * (fabsf(thn) + fabsf(rel.zr))) : -FLT_MAX;
+        unsigned pass = need ? quick_mask(sm, cnt, rel.xr, rel.yr, zlo_q, zhi_q) : 0u;
+        if constexpr (Vis::kInStep) {
+          unsigned any = __reduce_or_sync(0xffffffffu, pass);
+          while (any) {
+            const int j = __ffs(any) - 1;
+            any &= any - 1u;
             float d2, t;
-            leaf_test(rel, sm.stage[j], d2, t);
-            if (d2 <= 9.0f && t > tlo && t <= thn) {
-              if (hand_over(sm.stage[j], self, d2, t, vis, st)) {
-                need = !vis.stop();
-                th = vis.t_hi();
-                thn = need ? th : -FLT_MAX;
-              }
-            }
+            leaf_test(rel, sm, j, d2, t);
+            const int pos = __float_as_int(sm.stage[3][j].y);
+            const bool h = d2 <= 9.0f && t > tlo && t <= thn && pos != self;
+            if (vis.step(h, pos, t, sm.stage[0][j].w * expf(-0.5f * d2), sm.stage[3][j].x)) ++st.hits;
           }
-        } else {
-          for (int j0 = 0; j0 < cnt; j0 += UNROLL) {
-            unsigned pass = 0u;
-#pragma unroll
-            for (int k = 0; k < UNROLL; ++k) {
-              float d2, t;
-              leaf_test(rel, sm.stage[min(j0 + k, 31)], d2, t);  // past cnt: a stale entry, masked below
-              if (d2 <= 9.0f && t > tlo && t <= thn) pass |= 1u << k;
-            }
-            if (cnt - j0 < UNROLL) pass &= (1u << (cnt - j0)) - 1u;
-            while (pass) {
-              const int j = j0 + __ffs(pass) - 1;
-              pass &= pass - 1u;
-              float d2, t;
-              leaf_test(rel, sm.stage[j], d2, t);
-              if (t <= thn && hand_over(sm.stage[j], self, d2, t, vis, st)) {
-                need = !vis.stop();
-                th = vis.t_hi();
-                thn = need ? th : -FLT_MAX;
-              }
-            }
+          need = need && !vis.stop();
+          th = vis.t_hi();
+          pass = 0u;
+        }
+        while (pass) {
+          const int j = __ffs(pass) - 1;
+          pass &= pass - 1u;
+          float d2, t;
+          leaf_test(rel, sm, j, d2, t);
+          const float4 s3 = sm.stage[3][j];
+          const int pos = __float_as_int(s3.y);
+          if (d2 <= 9.0f && t > tlo && t <= thn && pos != self) {
+            ++st.hits;
+            vis.hit(pos, t, sm.stage[0][j].w * expf(-0.5f * d2), s3.x);
+            th = vis.t_hi();  // th only falls
+            need = !vis.stop();
+            thn = th;
+            if (!need) pass = 0u;
           }
         }
         __syncwarp();
@@ -427,6 +487,23 @@ __device__ void packet_walk(const TraceArgs& a, const Frame& f, const Ray& r, co
   __syncwarp();
 }
 
+// Visibility: product of (1 - alpha) over every hit, in any order; stops below t_min. Its code is short
+// and the hits of a leaf fall on neighbouring rays (9 lanes of 30 per leaf that is hit at all), so the
+// lanes take the leaves in step, each factor a select: no divergence, and the staged terms are
+// broadcast reads.
+struct VisibilityVis {
+  static constexpr bool kInStep = true;
+  float t_min, T;
+  __device__ float t_hi() const { return FLT_MAX; }
+  __device__ bool stop() const { return T < t_min; }
+  __device__ bool step(bool h, int, float, float al, float) {
+    h = h && !(T < t_min);
+    T = h ? T * (1.0f - al) : T;
+    return h;
+  }
+  __device__ void hit(int, float, float, float) {}
+};
+
 // Visibility walk of the bounce mode. Until T < t_min it multiplies every hit into T (in any
 // order, as ShadowVis), records the largest alpha m of the front-facing hits and, at the cut-off,
 // the horizon: the largest t* met so far (a hit past it has prefix transmittance below t_min and
@@ -437,53 +514,46 @@ __device__ void packet_walk(const TraceArgs& a, const Frame& f, const Ray& r, co
 // stays exact while no hit it holds lies behind a nearer candidate found later (checked with the
 // largest key summed); when it holds, the index search needs no walk in front of the candidate.
 struct BounceVis {
-  const TraceArgs& a;
-  const Ray& r;
-  int self;
-  RayStats& st;
+  static constexpr bool kInStep = false;  // surface-100k transfer 60.3 ms drained, 61.8 in step
+  float t_min;
   float T;
   float t_seen;
   float t_hor;
-  float tf;  // nearest front-facing hit: t*, position, alpha, facing term
+  float tf;  // nearest front-facing hit: t*, position, alpha
   int pf;
-  float af, mf;
+  float af;
   float amax;  // largest alpha m of the front-facing hits multiplied into T
   float lpre;  // sum of log(1 - alpha) of the hits with key below (tf, pf)
   float ts;    // largest key summed into lpre: t*, position
   int ps;
   bool pre_ok;  // lpre is the prefix of (tf, pf)
-  __device__ float t_hi() const { return T < a.t_min ? fminf(slack_hi(t_hor), slack_hi(tf)) : FLT_MAX; }
+  __device__ float t_hi() const { return T < t_min ? fminf(slack_hi(t_hor), slack_hi(tf)) : FLT_MAX; }
   __device__ bool stop() const { return false; }
+  __device__ bool step(bool, int, float, float, float) { return false; }
+  // (a hit past t_hi() changes nothing here)
   __device__ void hit(int pos, float t, float al, float m) {
-    if (!(T < a.t_min)) {
+    const bool live = !(T < t_min);
+    if (live) {
       T *= 1.0f - al;
       t_seen = fmaxf(t_seen, t);
-      if (T < a.t_min) t_hor = t_seen;
+      if (T < t_min) t_hor = t_seen;
       if (m > 0.f) amax = fmaxf(amax, al * m);
-    } else if (t > t_hor) {
-      return;
     }
-    if (m > 0.f && key_less(t, pos, tf, pf)) {
-      if (ps != INT32_MIN && !key_less(ts, ps, t, pos)) pre_ok = false;  // a summed hit lies behind it
-      tf = t;
-      pf = pos;
-      af = al;
-      mf = m;
-    } else if (key_less(t, pos, tf, pf)) {
+    const bool closer = (live || !(t > t_hor)) && key_less(t, pos, tf, pf);
+    if (m > 0.f) {
+      if (closer) {
+        if (ps != INT32_MIN && !key_less(ts, ps, t, pos)) pre_ok = false;  // a summed hit lies behind it
+        tf = t;
+        pf = pos;
+        af = al;
+      }
+    } else if (closer) {
       lpre += log1pf(-al);
       if (ps == INT32_MIN || key_less(ts, ps, t, pos)) {
         ts = t;
         ps = pos;
       }
     }
-  }
-  __device__ void leaf(int pos) {
-    if (pos == self) return;
-    ++st.leaves;
-    float t, al, m;
-    if (!gauss_hit(a.recs, pos, r, t, al, m)) return;
-    ++st.hits;
-    hit(pos, t, al, m);
   }
 };
 
@@ -494,17 +564,15 @@ struct BounceVis {
 // the prefix transmittance in front of that candidate.
 template <int KR>
 struct SearchVis {
-  const TraceArgs& a;
-  const Ray& r;
-  int self;
-  RayStats& st;
+  static constexpr bool kInStep = false;
+  __device__ bool step(bool, int, float, float, float) { return false; }
   float t_last;
   int p_last;
   float t_hor;
   float tf;
   int pf;
   float lbase;
-  float4 (*buf)[32];  // buf[k][lane]
+  RoundHits& buf;
   int lane;
   int count;
   float t_max;  // key of the last kept hit once the buffer is full
@@ -521,46 +589,85 @@ struct SearchVis {
     // sorted insertion: shift the larger keys up by one (the last falls out when full)
     int k = count < KR ? count : KR - 1;
     while (k > 0) {
-      const float4 e = buf[k - 1][lane];
-      if (!key_less(t, pos, e.x, __float_as_int(e.y))) break;
-      buf[k][lane] = e;
+      const float te = buf.t[k - 1][lane];
+      const int pe = buf.pos[k - 1][lane];
+      if (!key_less(t, pos, te, pe)) break;
+      buf.t[k][lane] = te;
+      buf.pos[k][lane] = pe;
+      buf.sal[k][lane] = buf.sal[k - 1][lane];
       --k;
     }
-    buf[k][lane] = make_float4(t, __int_as_float(pos), al, m);
+    buf.t[k][lane] = t;
+    buf.pos[k][lane] = pos;
+    buf.sal[k][lane] = m > 0.f ? -al : al;
     if (count < KR) ++count;
     if (count == KR) {
-      const float4 e = buf[KR - 1][lane];
-      t_max = e.x;
-      p_max = __float_as_int(e.y);
+      t_max = buf.t[KR - 1][lane];
+      p_max = buf.pos[KR - 1][lane];
     }
-  }
-  __device__ void leaf(int pos) {
-    if (pos == self) return;
-    ++st.leaves;
-    float t, al, m;
-    if (!gauss_hit(a.recs, pos, r, t, al, m)) return;
-    ++st.hits;
-    hit(pos, t, al, m);
   }
 };
 
-// Visibility (and with BOUNCE the index matrix) of the rays of receiver batch [r0, r1):
+// A ray handed from the visibility walk to the index-matrix search (self < 0: none).
+struct __align__(16) SearchRec {
+  int self;
+  int ref;  // receiver whose origin is the reference point of the exact tests; sign bit: lpre is exact
+  float t_hor;
+  float tf;  // the nearest front-facing hit: t*, position, alpha
+  int pf;
+  float af;
+  float lamax;  // every later candidate has log W_j <= lamax + log T_j
+  float lpre;
+};
+
+// Index matrix (Sec. 4.4): argmax of W_j = alpha_j T_j m_j over the hits in key order, T_j the prefix
+// transmittance; candidates need T_j >= t_min and T_j <= filter_t. Every later candidate has
+// W_j <= amax T_j (amax covers every front-facing hit when no cut-off happened, else the trivial bound
+// 1). With an exact prefix of the first candidate, the candidate is taken here, as the rounds would
+// take it (same arithmetic), and the rounds start behind it, if they are still needed: often its
+// weight already settles the argmax.
+struct FirstCandidate {
+  bool searching;
+  float t_last, lt, lw_best;
+  int p_last, best;
+};
+
+__device__ __forceinline__ FirstCandidate first_candidate(const TraceArgs& a, const Frame& f, const SearchRec& r) {
+  FirstCandidate c{true, -FLT_MAX, 0.0f, -FLT_MAX, INT32_MIN, -1};
+  if (r.ref >= 0) return c;
+  const float lmin = a.t_min > 0.f ? logf(a.t_min) : -FLT_MAX;
+  c.lt = r.lpre;
+  if (c.lt < lmin) {
+    c.searching = false;
+    return c;
+  }
+  if (c.lt <= logf(a.filter_t)) {
+    const float lw = logf(r.af * facing(f, __ldg(a.recs + 4 * (int64_t)r.pf + 3))) + c.lt;
+    if (lw > c.lw_best) {
+      c.lw_best = lw;
+      c.best = r.pf;
+    }
+  }
+  c.lt += log1pf(-r.af);
+  if (c.lt < lmin || c.lt + r.lamax <= c.lw_best) c.searching = false;
+  c.t_last = r.tf;
+  c.p_last = r.pf;
+  return c;
+}
+
+// Visibility (and with BOUNCE the first index-matrix candidates) of the rays of receiver batch [r0, r1):
 // V[s * batch + (i - r0)] (0 where n.w <= 0), idx[gid * S + s].
 #ifndef PRTGS_PACKET_BOUNCE_MIN_BLOCKS
-#define PRTGS_PACKET_BOUNCE_MIN_BLOCKS 4  // 128 registers, no spills; 55.5 KB shared per block at S = 256
+#define PRTGS_PACKET_BOUNCE_MIN_BLOCKS 4  // surface-100k transfer 60.3 ms at 4, 61.8 at 5
 #endif
 template <bool BOUNCE>
 __global__ void __launch_bounds__(kPacketThreads, BOUNCE ? PRTGS_PACKET_BOUNCE_MIN_BLOCKS : PRTGS_PACKET_MIN_BLOCKS)
     k_packet(TraceArgs a, float* __restrict__ V, int dpi) {
   extern __shared__ float4 psmem4[];
-  float* sdir = reinterpret_cast<float*>(psmem4);  // [S*3]
-  PacketSmem* wsm = reinterpret_cast<PacketSmem*>(sdir + ((3 * a.S + 3) & ~3));
+  PacketSmem* wsm = reinterpret_cast<PacketSmem*>(psmem4);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   PacketSmem& sm = wsm[warp];
-  RoundHits& hbuf = reinterpret_cast<RoundHits*>(wsm + kPacketWarps)[warp];  // bounce mode only
   __shared__ unsigned int s_item[kPacketWarps];
-  for (int i = threadIdx.x; i < 3 * a.S; i += blockDim.x) sdir[i] = a.dirs[i];
-  __syncthreads();
   const int64_t batch = a.r1 - a.r0;
   const int64_t n_windows = (batch + 63) / 64;
   const int dblocks = (a.S + dpi - 1) / dpi;  // dpi directions per work item
@@ -580,23 +687,11 @@ __global__ void __launch_bounds__(kPacketThreads, BOUNCE ? PRTGS_PACKET_BOUNCE_M
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int j = lane + 32 * h;
-      const bool vj = base + j < a.r1;
-      const int sj = vj ? (int)(base + j) : (int)a.r0;
-      sm.wq0[j] = __ldg(a.recs + 4 * sj);
-      nq[h] = __ldg(a.recs + 4 * sj + 3);
-      int rt = INT32_MIN, gj = -1;
-      if (vj) {
-        gj = a.order[sj];
-        rt = a.roots[find_scene(a.offsets, a.n_scenes, gj)];
-        if (rt != INT32_MIN && !child_ok(rt, a.n, a.status)) rt = INT32_MIN;
-      }
-      sm.wroot[j] = rt;
-      sm.wgid[j] = gj;
+      nq[h] = __ldg(a.recs + 4 * (base + j < a.r1 ? base + j : a.r0) + 3);
     }
-    __syncwarp();
     const int s1 = min(a.S, s0 + dpi);
     for (int s = s0; s < s1; ++s) {
-      const float* d = sdir + 3 * s;
+      const float d[3] = {__ldg(a.dirs + 3 * s), __ldg(a.dirs + 3 * s + 1), __ldg(a.dirs + 3 * s + 2)};
       // the receivers of the window that face direction s, compacted into packets of 32 lanes
       // (a window whose receivers all face it gives the two packets of its halves)
       bool upj[2];
@@ -607,29 +702,34 @@ __global__ void __launch_bounds__(kPacketThreads, BOUNCE ? PRTGS_PACKET_BOUNCE_M
         upj[h] = vj && ray_cos(nq[h].y, nq[h].z, nq[h].w, d) > 0.0f;
         if (vj && !upj[h]) {  // untraced ray: no visibility, no index-matrix entry
           V[(int64_t)s * batch + (base + j - a.r0)] = 0.0f;
-          if (BOUNCE) a.idx[(int64_t)sm.wgid[j] * a.S + s] = -1;
+          if (BOUNCE) a.idx[(int64_t)__ldg(a.order + base + j) * a.S + s] = -1;
         }
       }
       const unsigned m0 = __ballot_sync(0xffffffffu, upj[0]), m1 = __ballot_sync(0xffffffffu, upj[1]);
       const int total = __popc(m0) + __popc(m1);
-      if (upj[0]) sm.rlist[__popc(m0 & below)] = lane;
-      if (upj[1]) sm.rlist[__popc(m0) + __popc(m1 & below)] = lane + 32;
+      if (upj[0]) sm.rlist[__popc(m0 & below)] = (unsigned char)lane;
+      if (upj[1]) sm.rlist[__popc(m0) + __popc(m1 & below)] = (unsigned char)(lane + 32);
       __syncwarp();
       for (int pass = 0; pass * 32 < total; ++pass) {
       const bool up = pass * 32 + lane < total;
       const int jw = up ? sm.rlist[pass * 32 + lane] : 0;
-      const float4 q0 = sm.wq0[jw];
-      const int root = up ? sm.wroot[jw] : INT32_MIN;
       const int self = (int)(base + jw);
+      const float4 q0 = __ldg(a.recs + 4 * (int64_t)self);
+      const int gid = __ldg(a.order + self);
+      int root = INT32_MIN;
+      if (up) {
+        root = a.roots[find_scene(a.offsets, a.n_scenes, gid)];
+        if (root != INT32_MIN && !child_ok(root, a.n, a.status)) root = INT32_MIN;
+      }
       float vis = up ? 1.0f : 0.0f;
       int best = -1;  // index-matrix entry (sorted position of the chosen hit)
+      SearchRec rec;
+      rec.self = -1;
       if ((a.flags & PRTGS_SHADOW) && __any_sync(0xffffffffu, up)) {
         const Frame f = make_frame(d[0], d[1], d[2]);
         const float xl = f.e1x * q0.x + f.e1y * q0.y + f.e1z * q0.z;
         const float yl = f.e2x * q0.x + f.e2y * q0.y + f.e2z * q0.z;
         const float zl = f.wx * q0.x + f.wy * q0.y + f.wz * q0.z;
-        Ray r;
-        make_ray(r, q0.x, q0.y, q0.z, d[0], d[1], d[2]);
         traced += up ? 1u : 0u;
         // lanes of different scenes walk their own subtrees, one group at a time
         unsigned todo = __ballot_sync(0xffffffffu, up);
@@ -639,86 +739,27 @@ __global__ void __launch_bounds__(kPacketThreads, BOUNCE ? PRTGS_PACKET_BOUNCE_M
           const unsigned grp = __ballot_sync(0xffffffffu, up && root == groot) & todo;
           const bool mine = (grp >> lane) & 1u;
           if (lane == 0) ++walks;
+          const int leader_self = __shfl_sync(0xffffffffu, self, leader);
           // reference point of the group's exact tests: its leader's ray origin
           const Rel rel = make_rel(f, q0.x, q0.y, q0.z, __shfl_sync(0xffffffffu, q0.x, leader),
                                    __shfl_sync(0xffffffffu, q0.y, leader), __shfl_sync(0xffffffffu, q0.z, leader));
           if (!BOUNCE) {
-            ShadowVis sv{a, r, self, rs, 1.0f};
-            packet_walk<kPUnrollVis>(a, f, r, rel, self, groot, mine, xl, yl, zl, 0.0f, sv, sm, rs, rs.nodes);
+            VisibilityVis sv{a.t_min, 1.0f};
+            packet_walk(a, f, rel, self, groot, mine, xl, yl, zl, 0.0f, sv, sm, rs, rs.nodes);
             if (mine) vis = sv.T;
           } else {
-            BounceVis bv{a,    r,    self, rs,   1.0f, 0.0f,      FLT_MAX, FLT_MAX,
-                         INT32_MAX, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, INT32_MIN, true};
-            packet_walk<kPUnrollBounce>(a, f, r, rel, self, groot, mine, xl, yl, zl, 0.0f, bv, sm, rs, rs.nodes);
+            BounceVis bv{a.t_min, 1.0f, 0.0f, FLT_MAX, FLT_MAX, INT32_MAX, 0.0f, 0.0f, 0.0f, 0.0f, INT32_MIN, true};
+            packet_walk(a, f, rel, self, groot, mine, xl, yl, zl, 0.0f, bv, sm, rs, rs.nodes);
             if (mine) vis = bv.T;
-            // index matrix (Sec. 4.4): argmax of W_j = alpha_j T_j m_j over the hits in key order,
-            // T_j the prefix transmittance; candidates need T_j >= t_min and T_j <= filter_t.
-            // Every later candidate has W_j <= amax T_j (amax covers every front-facing hit when
-            // no cut-off happened, else the trivial bound 1).
-            const float lfilter = logf(a.filter_t);
-            const float lmin = a.t_min > 0.f ? logf(a.t_min) : -FLT_MAX;
-            const float lamax = bv.T < a.t_min ? 0.0f : logf(bv.amax);
-            bool searching = mine && bv.tf != FLT_MAX;
-            float t_last = -FLT_MAX, lt = 0.0f, lw_best = -FLT_MAX;
-            int p_last = INT32_MIN;
-            // with an exact prefix of the first candidate, the candidate is taken here, as the
-            // rounds would take it (same arithmetic), and the rounds start behind it, if they are
-            // still needed: often its weight already settles the argmax
-            const bool pre = bv.pre_ok && bv.pf > INT32_MIN;
-            if (pre && searching) {
-              lt = bv.lpre;
-              if (lt < lmin) {
-                searching = false;
-              } else {
-                if (lt <= lfilter) {
-                  const float lw = logf(bv.af * bv.mf) + lt;
-                  if (lw > lw_best) {
-                    lw_best = lw;
-                    best = bv.pf;
-                  }
-                }
-                lt += log1pf(-bv.af);
-                if (lt < lmin || lt + lamax <= lw_best) searching = false;
-                t_last = bv.tf;
-                p_last = bv.pf;
-              }
-            }
-            for (int64_t round = 0; __any_sync(0xffffffffu, searching); ++round) {
-              if (round > a.n / kPacketRoundHits + 1) {
-                if (searching) set_status(a.status, PRTGS_STATUS_BAD_INDEX);
-                break;
-              }
-              SearchVis<kPacketRoundHits> sv{a,     r,      self, rs,      t_last, p_last, bv.t_hor, bv.tf,
-                                             bv.pf, 0.0f,   hbuf,   lane, 0,     FLT_MAX, INT32_MAX};
-              if (searching) ++rs.rounds;
-              packet_walk<kPUnrollBounce>(a, f, r, rel, self, groot, searching, xl, yl, zl, t_last > 0.f ? t_last : 0.0f, sv, sm, rs,
-                          rs.search_nodes);
-              if (searching) {
-                if (round == 0 && !pre) lt = sv.lbase;
-                const int nh = sv.count;
-                bool decided = false;
-                for (int k = 0; k < nh && !decided; ++k) {
-                  if (lt < lmin || lt + lamax <= lw_best) {
-                    decided = true;
-                  } else {
-                    const float4 e = hbuf[k][lane];  // t*, position, alpha, m
-                    if (e.w > 0.f && lt <= lfilter) {
-                      const float lw = logf(e.z * e.w) + lt;
-                      if (lw > lw_best) {
-                        lw_best = lw;
-                        best = __float_as_int(e.y);
-                      }
-                    }
-                    lt += log1pf(-e.z);
-                  }
-                }
-                if (decided || nh < kPacketRoundHits || lt < lmin || lt + lamax <= lw_best) {
-                  searching = false;
-                } else {
-                  t_last = sv.t_max;
-                  p_last = sv.p_max;
-                }
-              }
+            // the index-matrix search goes on in k_search, for the rays whose first candidate does not
+            // already settle the argmax
+            FirstCandidate fc;
+            if (mine && bv.tf != FLT_MAX) {
+              const float lamax = bv.T < a.t_min ? 0.0f : logf(bv.amax);
+              rec = SearchRec{self, leader_self | (bv.pre_ok ? INT32_MIN : 0), bv.t_hor, bv.tf, bv.pf, bv.af, lamax, bv.lpre};
+              fc = first_candidate(a, f, rec);
+              best = fc.best;
+              if (!fc.searching) rec.self = -1;
             }
           }
           todo &= ~grp;
@@ -726,7 +767,14 @@ __global__ void __launch_bounds__(kPacketThreads, BOUNCE ? PRTGS_PACKET_BOUNCE_M
       }
       if (up) {
         V[(int64_t)s * batch + (self - a.r0)] = vis;
-        if (BOUNCE) a.idx[(int64_t)sm.wgid[jw] * a.S + s] = best >= 0 ? a.order[best] : -1;
+        if (BOUNCE) a.idx[(int64_t)gid * a.S + s] = best >= 0 ? a.order[best] : -1;
+      }
+      if (BOUNCE && __any_sync(0xffffffffu, rec.self >= 0)) {  // a search item: the packet's rays that go on
+        unsigned e = 0;
+        if (lane == 0) e = atomicAdd(a.queue_count, 1u);
+        e = __shfl_sync(0xffffffffu, e, 0);
+        if (lane == 0) a.pending[e] = (uint32_t)s;
+        static_cast<SearchRec*>(a.queue)[(int64_t)e * 32 + lane] = rec;
       }
       __syncwarp();
       }  // pass
@@ -746,6 +794,108 @@ __global__ void __launch_bounds__(kPacketThreads, BOUNCE ? PRTGS_PACKET_BOUNCE_M
       atomicAdd(a.stats + 3, c3);
       atomicAdd(a.stats + 5, c5);
       atomicAdd(a.stats + 8, c8);
+      atomicAdd(a.stats + 9, c9);
+    }
+  }
+}
+
+// The index-matrix search of the packets that k_packet<true> left: one warp per item, rounds of 14 hits
+// in key order until every ray's argmax is settled. A kernel of its own: only a third of the packets
+// get here, and beside the visibility walk's code and registers both ran slower.
+#ifndef PRTGS_SEARCH_MIN_BLOCKS
+#define PRTGS_SEARCH_MIN_BLOCKS 4
+#endif
+__global__ void __launch_bounds__(kPacketThreads, PRTGS_SEARCH_MIN_BLOCKS) k_search(TraceArgs a) {
+  extern __shared__ float4 psmem4[];
+  PacketSmem* wsm = reinterpret_cast<PacketSmem*>(psmem4);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  PacketSmem& sm = wsm[warp];
+  RoundHits& hbuf = reinterpret_cast<RoundHits*>(wsm + kPacketWarps)[warp];
+  RayStats rs{0u, 0u, 0u, 0u, 0u, 0u};
+  const unsigned items = *a.queue_count;
+  for (;;) {
+    unsigned item = 0;
+    if (lane == 0) item = atomicAdd(a.work, 1u);
+    item = __shfl_sync(0xffffffffu, item, 0);
+    if (item >= items) break;
+    const int s = (int)a.pending[item];
+    const SearchRec rec = static_cast<const SearchRec*>(a.queue)[(int64_t)item * 32 + lane];
+    const bool mine = rec.self >= 0;
+    const int self = mine ? rec.self : (int)a.r0;
+    const float d[3] = {__ldg(a.dirs + 3 * s), __ldg(a.dirs + 3 * s + 1), __ldg(a.dirs + 3 * s + 2)};
+    const Frame f = make_frame(d[0], d[1], d[2]);
+    const float4 q0 = __ldg(a.recs + 4 * (int64_t)self);
+    const int gid = __ldg(a.order + self);
+    const int ref = rec.ref & INT32_MAX;
+    const int root = mine ? a.roots[find_scene(a.offsets, a.n_scenes, gid)] : INT32_MIN;
+    const float xl = f.e1x * q0.x + f.e1y * q0.y + f.e1z * q0.z;
+    const float yl = f.e2x * q0.x + f.e2y * q0.y + f.e2z * q0.z;
+    const float zl = f.wx * q0.x + f.wy * q0.y + f.wz * q0.z;
+    const float lfilter = logf(a.filter_t);
+    const float lmin = a.t_min > 0.f ? logf(a.t_min) : -FLT_MAX;
+    const bool pre = rec.ref < 0;
+    FirstCandidate c{false, -FLT_MAX, 0.0f, -FLT_MAX, INT32_MIN, -1};
+    if (mine) c = first_candidate(a, f, rec);
+    unsigned todo = __ballot_sync(0xffffffffu, mine);
+    while (todo) {  // rays of different scenes one group at a time
+      const int leader = __ffs(todo) - 1;
+      const int groot = __shfl_sync(0xffffffffu, root, leader);
+      const unsigned grp = __ballot_sync(0xffffffffu, mine && root == groot) & todo;
+      const int gref = __shfl_sync(0xffffffffu, ref, leader);
+      const float4 R = __ldg(a.recs + 4 * (int64_t)gref);
+      const Rel rel = make_rel(f, q0.x, q0.y, q0.z, R.x, R.y, R.z);
+      bool searching = ((grp >> lane) & 1u) && c.searching;
+      for (int64_t round = 0; __any_sync(0xffffffffu, searching); ++round) {
+        if (round > a.n / kPacketRoundHits + 1) {
+          if (searching) set_status(a.status, PRTGS_STATUS_BAD_INDEX);
+          break;
+        }
+        SearchVis<kPacketRoundHits> sv{c.t_last, c.p_last, rec.t_hor, rec.tf, rec.pf, 0.0f, hbuf, lane, 0, FLT_MAX, INT32_MAX};
+        if (searching) ++rs.rounds;
+        packet_walk(a, f, rel, self, groot, searching, xl, yl, zl, c.t_last > 0.f ? c.t_last : 0.0f, sv, sm, rs,
+                    rs.search_nodes);
+        if (searching) {
+          if (round == 0 && !pre) c.lt = sv.lbase;
+          const int nh = sv.count;
+          bool decided = false;
+          for (int k = 0; k < nh && !decided; ++k) {
+            if (c.lt < lmin || c.lt + rec.lamax <= c.lw_best) {
+              decided = true;
+            } else {
+              const float sal = hbuf.sal[k][lane], al = fabsf(sal);
+              if (signbit(sal) && c.lt <= lfilter) {  // front-facing
+                const int pos = hbuf.pos[k][lane];
+                const float lw = logf(al * facing(f, __ldg(a.recs + 4 * (int64_t)pos + 3))) + c.lt;
+                if (lw > c.lw_best) {
+                  c.lw_best = lw;
+                  c.best = pos;
+                }
+              }
+              c.lt += log1pf(-al);
+            }
+          }
+          if (decided || nh < kPacketRoundHits || c.lt < lmin || c.lt + rec.lamax <= c.lw_best) {
+            searching = false;
+          } else {
+            c.t_last = sv.t_max;
+            c.p_last = sv.p_max;
+          }
+        }
+        __syncwarp();
+      }
+      todo &= ~grp;
+    }
+    if (mine) a.idx[(int64_t)gid * a.S + s] = c.best >= 0 ? a.order[c.best] : -1;
+    __syncwarp();
+  }
+  if (a.stats) {
+    const unsigned long long c1 = warp_sum_u64(rs.search_nodes), c2 = warp_sum_u64(rs.leaves), c3 = warp_sum_u64(rs.hits),
+                             c4 = warp_sum_u64(rs.rounds), c9 = warp_sum_u64(rs.entries);
+    if (lane == 0) {
+      atomicAdd(a.stats + 1, c1);
+      atomicAdd(a.stats + 2, c2);
+      atomicAdd(a.stats + 3, c3);
+      atomicAdd(a.stats + 4, c4);
       atomicAdd(a.stats + 9, c9);
     }
   }
@@ -795,14 +945,16 @@ __global__ void __launch_bounds__(128) k_project(TraceArgs a, const float* __res
   }
 }
 
-static size_t packet_smem(int S, bool bounce) {
-  return sizeof(float) * ((3 * S + 3) & ~3) + sizeof(PacketSmem) * kPacketWarps +
-         (bounce ? sizeof(RoundHits) * kPacketWarps : 0);
+// Scratch of the index-matrix search of a batch: every packet (at most two per window and direction)
+// may need it.
+size_t packet_search_bytes(int64_t batch, int S) {
+  const size_t items = 2 * (size_t)((batch + 63) / 64) * S;
+  return align_up(sizeof(SearchRec) * 32 * items) + align_up(sizeof(uint32_t) * items);
 }
 
 template <bool BOUNCE>
 static int launch_packet_t(const TraceArgs& a, float* V, int sms, cudaStream_t stream) {
-  const size_t smem = packet_smem(a.S, BOUNCE);
+  const size_t smem = sizeof(PacketSmem) * kPacketWarps;
   cudaFuncSetAttribute(k_packet<BOUNCE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   cudaFuncSetAttribute(k_packet<BOUNCE>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   int per_sm = 0;
@@ -810,7 +962,16 @@ static int launch_packet_t(const TraceArgs& a, float* V, int sms, cudaStream_t s
   // work items: (window of 64 receivers, dpi directions); at most 2^26 / 64 of them per batch
   const int dpi = a.packet_dirs > 0 ? a.packet_dirs : kPacketDirs;
   cudaMemsetAsync(a.work, 0, sizeof(unsigned int), stream);
+  if (BOUNCE) cudaMemsetAsync(a.queue_count, 0, sizeof(unsigned int), stream);
   k_packet<BOUNCE><<<sms * (per_sm > 0 ? per_sm : 1), kPacketThreads, smem, counted(stream)>>>(a, V, dpi);
+  if (BOUNCE) {
+    const size_t ssmem = (sizeof(PacketSmem) + sizeof(RoundHits)) * kPacketWarps;
+    cudaFuncSetAttribute(k_search, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssmem);
+    cudaFuncSetAttribute(k_search, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_search, kPacketThreads, ssmem);
+    cudaMemsetAsync(a.work, 0, sizeof(unsigned int), stream);
+    k_search<<<sms * (per_sm > 0 ? per_sm : 1), kPacketThreads, ssmem, counted(stream)>>>(a);
+  }
   PRTGS_CHECK_LAUNCH();
   const int64_t batch = a.r1 - a.r0;
   k_project<<<(unsigned)((batch + 127) / 128), 128, sizeof(float) * 3 * a.S, counted(stream)>>>(a, V);

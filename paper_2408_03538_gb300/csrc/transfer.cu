@@ -1046,12 +1046,25 @@ static int64_t packet_batch(int64_t n, int S) {
   return b < n ? b : n;
 }
 
+// ... and per launch inside a batch, in whole windows: with bounces half of that, whose search records
+// (32 B a ray at most) then take at most 1 GB.
+static int64_t packet_part(int64_t n, int S, bool bounce) {
+  const int64_t batch = packet_batch(n, S);
+  int64_t b = ((int64_t(1) << 25) / (S > 0 ? S : 1)) / 64 * 64;
+  if (b < 64) b = 64;
+  return bounce && b < batch ? b : batch;
+}
+
 static bool use_packets(const prtgs_transfer_params* p) { return p->walk == 0; }
 
 size_t transfer_workspace(int64_t n, int64_t n_glossy, const prtgs_transfer_params* p, bool want_V) {
   size_t b = 2 * align_up(sizeof(unsigned int));
   if (want_V) b += align_up(sizeof(int32_t) * (size_t)n);
-  if (use_packets(p)) b += align_up(sizeof(float) * (size_t)packet_batch(n, p->n_dirs) * p->n_dirs);
+  if (use_packets(p)) {
+    const bool bounce = (p->flags & PRTGS_BOUNCE) != 0;
+    const int64_t batch = packet_part(n, p->n_dirs, bounce);
+    b += align_up(sizeof(float) * (size_t)batch * p->n_dirs) + (bounce ? packet_search_bytes(batch, p->n_dirs) : 0);
+  }
   if (sh_count(p->sh_order) > kMaxC) b += align_up(sizeof(float) * (size_t)p->n_dirs * sh_count(p->sh_order));
   if (p->flags & PRTGS_BOUNCE) {
     if (!use_packets(p)) {  // the per-ray walk's candidate records and rounds queue
@@ -1131,7 +1144,13 @@ int precompute_transfer(const prtgs_gaussians* g, const prtgs_bvh* bvh, const pr
   unsigned int* more_count = rayq ? c.take<unsigned int>(1) : nullptr;
   float* ytab = C > kMaxC ? c.take<float>((size_t)S * C) : nullptr;
   const bool packets = use_packets(p);
-  float* vbuf = packets ? c.take<float>((size_t)packet_batch(n, S) * S) : nullptr;
+  const int64_t pb = packet_part(n, S, bounce);
+  float* vbuf = packets ? c.take<float>((size_t)pb * S) : nullptr;
+  if (packets && bounce) {
+    const size_t items = 2 * (size_t)((pb + 63) / 64) * S;
+    queue = c.take<char>(packet_search_bytes(pb, S) - align_up(sizeof(uint32_t) * items));
+    pending = c.take<uint32_t>(items);
+  }
   float* tb[2] = {nullptr, nullptr};  // ping-pong bounce buffers [n,3,C] for n_bounces > 1
   if (bounce && n_bounces_of(p) > 1) tb[0] = c.take<float>((size_t)n * 3 * C);
   if (bounce && n_bounces_of(p) > 2) tb[1] = c.take<float>((size_t)n * 3 * C);
@@ -1192,11 +1211,14 @@ int precompute_transfer(const prtgs_gaussians* g, const prtgs_bvh* bvh, const pr
   int rct;
   if (packets) {
     rct = PRTGS_OK;
-    const int64_t pb = packet_batch(n, S);
-    for (int64_t r0 = 0; r0 < n && rct == PRTGS_OK; r0 += pb) {
-      a.r0 = r0;
-      a.r1 = r0 + pb < n ? r0 + pb : n;
-      rct = launch_packet(a, vbuf, bounce, sms, stream);
+    const int64_t whole = packet_batch(n, S);
+    for (int64_t b0 = 0; b0 < n; b0 += whole) {
+      const int64_t b1 = b0 + whole < n ? b0 + whole : n;
+      for (int64_t r0 = b0; r0 < b1 && rct == PRTGS_OK; r0 += pb) {
+        a.r0 = r0;
+        a.r1 = r0 + pb < b1 ? r0 + pb : b1;
+        rct = launch_packet(a, vbuf, bounce, sms, stream);
+      }
     }
   } else if (!bounce) {
     rct = launch_trace<false, 1>(a, smem, sms, batch, incl, rlist, rscan_ws, more, more_count, stream);

@@ -1,0 +1,66 @@
+"""The packet walk's staging, quick test and index search at the sizes where they can go wrong: windows
+and packets that are just full or one over, several scenes inside a window, needle-thin splats (the
+quick test's margin), many hits on a ray (more rounds than one buffer holds).
+
+Tolerances as in test_gpu_transfer.py: 1e-4 norm-wise per receiver plus the oracle's allowance; the
+index matrix bit-exact on unflagged rays.
+"""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2408_03538_gb300 import api, scenes as S
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(sc, offs, dirs, order, sizes):
+    g = api.GaussianTensors.from_scene(sc)
+    st = api.Status()
+    bvh = api.build_bvh(g, torch.from_numpy(offs).cuda(), status=st)
+    d = torch.from_numpy(dirs).cuda()
+    out = api.precompute_transfer(g, bvh, d, order, bounce=True, status=st)
+    P0 = api.precompute_transfer(g, bvh, d, order, status=st)["P"]
+    torch.cuda.synchronize()
+    assert st.read() == 0
+    floor = 1e-3 * oracle.unoccluded_norm(order)
+    for b, n in enumerate(sizes):
+        at = np.arange(offs[b], offs[b + 1])
+        ref = oracle.transfer(sc.subset(at), dirs, order, np.arange(n), bounce=True)
+        lim = 1e-4 * np.maximum(np.linalg.norm(ref["P"], axis=1), floor) + ref["allow_P"]
+        for P in (out["P"], P0):
+            assert np.all(np.linalg.norm(P.cpu().numpy()[at] - ref["P"], axis=1) <= lim)
+        T = out["T"].cpu().numpy()[at]
+        lim = 1e-4 * np.maximum(np.linalg.norm(ref["T"].reshape(n, -1), axis=1), floor)
+        lim = lim + np.linalg.norm(ref["allow_T"], axis=1)
+        assert np.all(np.linalg.norm((T - ref["T"]).reshape(n, -1), axis=1) <= lim)
+        clean = (ref["flags"] & (oracle.RF_AMBIG_HIT | oracle.RF_AMBIG_ARGMAX)) == 0
+        idx = out["idx"].cpu().numpy()[at]
+        np.testing.assert_array_equal(np.where(idx >= 0, idx - offs[b], idx)[clean], ref["idx"][clean])
+
+
+@pytest.mark.parametrize("sizes", [[31], [64], [65], [129], [40, 1, 30, 90], [500]])
+def test_packet_windows_against_oracle(sizes):
+    parts = [S.surface_scene(n, 300 + n) for n in sizes]
+    for p in parts:
+        p.means *= 0.25  # crowded: hits in the tens per ray
+    sc, offs = S.concat_scenes(parts)
+    _check(sc, offs, S.direction_set(37, 5), 2, sizes)
+
+
+@pytest.mark.parametrize("thin", [1.0, 30.0, 300.0])
+def test_packet_thin_splats_against_oracle(thin):
+    sc = S.surface_scene(900, 41)
+    sc.means *= 0.3
+    sc.scales[:, 2] = sc.scales[:, :2].min(axis=1) / np.float32(thin)
+    sc.scales[::3, 0] /= np.float32(thin)
+    _check(sc, np.array([0, sc.n], np.int64), S.direction_set(48, 6), 3, [sc.n])
+
+
+def test_packet_many_hits_per_ray():
+    """Faint splats: rays pass tens of them before the index matrix is settled."""
+    sc = S.surface_scene(1500, 42)
+    sc.means *= 0.2
+    sc.opacity *= np.float32(0.1)
+    _check(sc, np.array([0, sc.n], np.int64), S.direction_set(24, 7), 1, [sc.n])
