@@ -220,9 +220,9 @@ int prtgs_precompute_transfer(const prtgs_gaussians* g, const prtgs_bvh* bvh, co
 /*
  * Transfer backward: gradients of a loss through P (the shadowed diffuse transfer of Eq. 29
  * projected by Eq. 9) to the Gaussians, for optimising geometry against relit images
- * (Sec. 4.4). Each traced ray is walked again twice in the forward's order -- once for
- * V_is, once pushing dL/dalpha_j = -g V_is / (1 - alpha_j) to every occluder up to the same
- * early exit -- so no per-ray hit list is stored. The hit set (t* > 0, D^2 <= 9) and the
+ * (Sec. 4.4). Each traced ray is walked again for V_is, as part of its packet, and pushes
+ * dL/dalpha_j = -g V_is / (1 - alpha_j) to every occluder up to the same early exit; a packet's
+ * hit leaves are listed while it is in flight, no per-ray hit list is stored. The hit set (t* > 0, D^2 <= 9) and the
  * hemisphere test are held fixed (non-differentiable boundaries); the gradient flows through
  * opacity_j exp(-D^2/2), D^2 at the closest approach (to mu_j, s_j, q_j and, via the ray
  * origin, mu_i) and the cosine max(0, n_i.w) (to the raw normal n_i).

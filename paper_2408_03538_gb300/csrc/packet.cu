@@ -323,12 +323,48 @@ __device__ __forceinline__ bool beam_meets(const Beam& b, const float4& A, const
 // The exact test of one staged leaf for the lane: D^2 and t* (see Rel). The high parts of dx
 // cancel without rounding error of their own beyond eps |dx| (exactly where they nearly cancel);
 // the low parts carry the roundings of both.
-__device__ __forceinline__ void leaf_test(const Rel& rel, const PacketSmem& sm, int j, float& d2, float& t) {
+__device__ __forceinline__ void leaf_offset(const Rel& rel, const PacketSmem& sm, int j, float& wx, float& wy, float& wz,
+                                            float& t) {
   const float4 s0 = sm.stage[0][j], s1 = sm.stage[1][j], s2 = sm.stage[2][j], s3 = sm.stage[3][j];
   const float dx = (rel.xr + s0.x) + (rel.xr_lo + s3.z), dy = (rel.yr + s0.y) + (rel.yr_lo + s3.w);
-  const float wx = fmaf(dx, s1.x, dy * s2.x), wy = fmaf(dx, s1.y, dy * s2.y), wz = fmaf(dx, s1.z, dy * s2.z);
-  d2 = fmaf(wx, wx, fmaf(wy, wy, wz * wz));
+  wx = fmaf(dx, s1.x, dy * s2.x);
+  wy = fmaf(dx, s1.y, dy * s2.y);
+  wz = fmaf(dx, s1.z, dy * s2.z);
   t = -(rel.zr + s0.z) - fmaf(dx, s1.w, dy * s2.w);
+}
+
+__device__ __forceinline__ void leaf_test(const Rel& rel, const PacketSmem& sm, int j, float& d2, float& t) {
+  float wx, wy, wz;
+  leaf_offset(rel, sm, j, wx, wy, wz, t);
+  d2 = fmaf(wx, wx, fmaf(wy, wy, wz * wz));
+}
+
+// Hit decision of a leaf by the single ray's own test (the transfer backward decides as the per-ray
+// walk does): only where the planar test is near a boundary, D^2 = 9 or t* = 0, can the two differ.
+// The band is some ten times the largest difference of their roundings.
+__device__ __noinline__ bool ray_hit(const float4* __restrict__ recs, int pos, float ox, float oy, float oz, float dx,
+                                     float dy, float dz) {
+  Ray r{};
+  r.ox = ox;
+  r.oy = oy;
+  r.oz = oz;
+  r.dx = dx;
+  r.dy = dy;
+  r.dz = dz;
+  float t, al, m;
+  return gauss_hit(recs, pos, r, t, al, m);
+}
+
+__device__ __forceinline__ bool ray_decides(const float4* __restrict__ recs, const Frame& f, float ox, float oy, float oz,
+                                            const Rel& rel, const PacketSmem& sm, int j, int pos, float d2, float t,
+                                            bool planar) {
+  const float4 s0 = sm.stage[0][j];
+  const float dx = rel.xr + s0.x, dy = rel.yr + s0.y;
+  const float band = 1e-4f * (fabsf(rel.zr) + fabsf(s0.z) + fabsf(dx) * (1.0f + fabsf(sm.stage[1][j].w)) +
+                              fabsf(dy) * (1.0f + fabsf(sm.stage[2][j].w)));
+  if (!(d2 > 9.02f) && !(t < -band) && (!(d2 < 8.98f) || !(t > band)))
+    return ray_hit(recs, pos, ox, oy, oz, f.wx, f.wy, f.wz);
+  return planar;
 }
 
 // Quick test of the staged leaves for the lane: bit j of the result is set for every leaf j < cnt whose
@@ -442,7 +478,8 @@ __device__ void packet_walk(const TraceArgs& a, const Frame& f, const Rel& rel, 
         if (need) st.leaves += cnt;  // leaf tests of the lane (its own Gaussian included)
         float thn = need ? th : -FLT_MAX;  // a lane that wants no hits passes no test
         const float zhi_q = need ? (thn + rel.zr) + (2.0f * et + 2e-6f * (fabsf(thn) + fabsf(rel.zr))) : -FLT_MAX;
-        unsigned pass = need ? quick_mask(sm, cnt, rel.xr, rel.yr, zlo_q, zhi_q) : 0u;
+        const float zlo_g = Vis::kRayDecides ? zlo_q - 50.0f * et : zlo_q;  // the band of ray_decides
+        unsigned pass = need ? quick_mask(sm, cnt, rel.xr, rel.yr, zlo_g, zhi_q) : 0u;
         if constexpr (Vis::kInStep) {
           unsigned any = __reduce_or_sync(0xffffffffu, pass);
           while (any) {
@@ -451,7 +488,10 @@ __device__ void packet_walk(const TraceArgs& a, const Frame& f, const Rel& rel, 
             float d2, t;
             leaf_test(rel, sm, j, d2, t);
             const int pos = __float_as_int(sm.stage[3][j].y);
-            const bool h = d2 <= 9.0f && t > tlo && t <= thn && pos != self;
+            bool h = d2 <= 9.0f && t > tlo && t <= thn && pos != self;
+            if constexpr (Vis::kRayDecides) {
+              if (need && pos != self) h = ray_decides(a.recs, f, vis.ox, vis.oy, vis.oz, rel, sm, j, pos, d2, t, h);
+            }
             if (vis.step(h, pos, t, sm.stage[0][j].w * expf(-0.5f * d2), sm.stage[3][j].x)) ++st.hits;
           }
           need = need && !vis.stop();
@@ -492,6 +532,7 @@ __device__ void packet_walk(const TraceArgs& a, const Frame& f, const Rel& rel, 
 // lanes take the leaves in step, each factor a select: no divergence, and the staged terms are
 // broadcast reads.
 struct VisibilityVis {
+  static constexpr bool kRayDecides = false;
   static constexpr bool kInStep = true;
   float t_min, T;
   __device__ float t_hi() const { return FLT_MAX; }
@@ -514,6 +555,7 @@ struct VisibilityVis {
 // stays exact while no hit it holds lies behind a nearer candidate found later (checked with the
 // largest key summed); when it holds, the index search needs no walk in front of the candidate.
 struct BounceVis {
+  static constexpr bool kRayDecides = false;
   static constexpr bool kInStep = false;  // surface-100k transfer 60.3 ms drained, 61.8 in step
   float t_min;
   float T;
@@ -564,6 +606,7 @@ struct BounceVis {
 // the prefix transmittance in front of that candidate.
 template <int KR>
 struct SearchVis {
+  static constexpr bool kRayDecides = false;
   static constexpr bool kInStep = false;
   __device__ bool step(bool, int, float, float, float) { return false; }
   float t_last;
@@ -899,6 +942,368 @@ __global__ void __launch_bounds__(kPacketThreads, PRTGS_SEARCH_MIN_BLOCKS) k_sea
       atomicAdd(a.stats + 9, c9);
     }
   }
+}
+
+// ---- backward of the shadowed transfer ---------------------------------------------------------------
+// Per ray V = prod (1 - alpha_j); with g_V its gradient, dL/dalpha_j = -g_V V / (1 - alpha_j), and with
+// x the whitened offset at the closest approach (D^2 = |x|^2), g = dL/dD^2 = -alpha/2 dL/dalpha:
+//   d opacity_j += dL/dalpha exp(-D^2/2),  d mu_j -= 2 g A^T x,  d o += 2 g A^T x,
+//   d s_k -= 2 g x_k^2 / s_k,  d R_jk += 2 g x_k w_j / s_k with w = R diag(s) x.
+// So a Gaussian needs only sum g_alpha exp(-D^2/2), sum g x and sum g x x^T over its hits, ten numbers
+// that do not depend on the direction. k_packet_bwd walks each packet once for V, noting the leaves that
+// any of its rays hit, then goes through that list: every lane forms its g and the offset w' = x cross a
+// (two coordinates in a plane of the leaf), the six moments are summed over the packet's rays through
+// shared memory, and one lane per leaf turns them into the ten sums and adds them with three vector
+// reductions. k_bwd_finish forms the gradients, once per Gaussian.
+// Walking each ray alone and twice, with twelve atomics per hit, took 843 ms for a 100k volume at 128
+// directions and 147 ms for 40k surface splats at 256; this takes 80 and 14 ms, bound by issue slots.
+// Hits are decided as by the ray's own test (ray_decides, a tenth of that time): on a surface, splats in
+// the receiver's own plane have t* = 0 up to rounding and a large alpha.
+
+// Hits of the packet's rays, as VisibilityVis, and the list of the leaves hit by any of them from the
+// skip-th on (a list that overflows is continued by another walk: the same leaves in the same order).
+struct HitListVis {
+  static constexpr bool kInStep = true, kRayDecides = true;
+  float t_min, T;
+  float ox, oy, oz;  // the ray's origin
+  int* list;
+  int skip, cap, total;
+  __device__ float t_hi() const { return FLT_MAX; }
+  __device__ bool stop() const { return T < t_min; }
+  __device__ bool step(bool h, int pos, float, float al, float) {
+    h = h && !(T < t_min);
+    T = h ? T * (1.0f - al) : T;
+    if (__any_sync(0xffffffffu, h)) {
+      const int k = total - skip;
+      if ((threadIdx.x & 31) == 0 && k >= 0 && k < cap) list[k] = pos;
+      ++total;
+    }
+    return h;
+  }
+  __device__ void hit(int, float, float, float) {}
+};
+
+constexpr int kBwdBlocks = 4;      // per SM
+constexpr int kBwdList = 2048;     // hit leaves of a packet kept at a time
+constexpr int kBwdBatch = 5;       // leaves whose six moments are summed together (30 lanes, one sum each)
+constexpr int kBwdRow = 36;        // 32 lanes' values and padding: 16-byte reads of 30 rows without conflicts
+
+struct BwdSmem {
+  float row[6 * kBwdBatch][kBwdRow];
+  float sum[32][8];
+};
+
+__device__ __forceinline__ void red_add4(float* p, float a, float b, float c, float d) {
+  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d)
+               : "memory");
+}
+
+// G, GV: [S][batch] gradients of each ray's c V (for the normal) and of its V; acc: [n][12] sums per
+// Gaussian, ray: [n][8] (d o, d n) per receiver, both in sorted order; lists: kBwdList ints per warp.
+__global__ void __launch_bounds__(kPacketThreads, kBwdBlocks)
+    k_packet_bwd(TraceArgs a, const float* __restrict__ G, const float* __restrict__ GV, float* __restrict__ acc,
+                 float* __restrict__ rayacc, int* __restrict__ lists) {
+  extern __shared__ float4 psmem4[];
+  PacketSmem* wsm = reinterpret_cast<PacketSmem*>(psmem4);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  PacketSmem& sm = wsm[warp];
+  BwdSmem& bs = reinterpret_cast<BwdSmem*>(wsm + kPacketWarps)[warp];
+  int* list = lists + ((int64_t)blockIdx.x * kPacketWarps + warp) * kBwdList;
+  const int64_t batch = a.r1 - a.r0;
+  const int64_t n_windows = (batch + 63) / 64;
+  const unsigned below = (1u << lane) - 1u;
+  RayStats rs{0u, 0u, 0u, 0u, 0u, 0u};
+  for (;;) {
+    unsigned item = 0;
+    if (lane == 0) item = atomicAdd(a.work, 1u);
+    item = __shfl_sync(0xffffffffu, item, 0);
+    if ((int64_t)item >= n_windows * a.S) break;
+    const int64_t base = a.r0 + 64 * (item / a.S);
+    const int s = (int)(item % a.S);
+    const float d[3] = {__ldg(a.dirs + 3 * s), __ldg(a.dirs + 3 * s + 1), __ldg(a.dirs + 3 * s + 2)};
+    const Frame f = make_frame(d[0], d[1], d[2]);
+    bool upj[2];  // k_ray_grad left zeros for the directions below a receiver's horizon
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int64_t j = base + lane + 32 * h;
+      const int64_t o = (int64_t)s * batch + (j - a.r0);
+      upj[h] = j < a.r1 && (G[o] != 0.0f || GV[o] != 0.0f);
+    }
+    const unsigned m0 = __ballot_sync(0xffffffffu, upj[0]), m1 = __ballot_sync(0xffffffffu, upj[1]);
+    const int total = __popc(m0) + __popc(m1);
+    if (upj[0]) sm.rlist[__popc(m0 & below)] = (unsigned char)lane;
+    if (upj[1]) sm.rlist[__popc(m0) + __popc(m1 & below)] = (unsigned char)(lane + 32);
+    __syncwarp();
+    for (int pass = 0; pass * 32 < total; ++pass) {
+      const bool up = pass * 32 + lane < total;
+      const int self = (int)(base + (up ? sm.rlist[pass * 32 + lane] : 0));
+      const float4 q0 = __ldg(a.recs + 4 * (int64_t)self);
+      const int64_t o = (int64_t)s * batch + (self - a.r0);
+      const float gc = up ? G[o] : 0.0f, gV = up ? GV[o] : 0.0f;
+      float V = up ? 1.0f : 0.0f, go1 = 0.0f, go2 = 0.0f;
+      if (a.flags & PRTGS_SHADOW) {
+        int root = INT32_MIN;
+        if (up) {
+          root = a.roots[find_scene(a.offsets, a.n_scenes, __ldg(a.order + self))];
+          if (root != INT32_MIN && !child_ok(root, a.n, a.status)) root = INT32_MIN;
+        }
+        const float xl = f.e1x * q0.x + f.e1y * q0.y + f.e1z * q0.z;
+        const float yl = f.e2x * q0.x + f.e2y * q0.y + f.e2z * q0.z;
+        const float zl = f.wx * q0.x + f.wy * q0.y + f.wz * q0.z;
+        unsigned todo = __ballot_sync(0xffffffffu, up);
+        while (todo) {
+          const int leader = __ffs(todo) - 1;
+          const int groot = __shfl_sync(0xffffffffu, root, leader);
+          const unsigned grp = __ballot_sync(0xffffffffu, up && root == groot) & todo;
+          const bool mine = (grp >> lane) & 1u;
+          const Rel rel = make_rel(f, q0.x, q0.y, q0.z, __shfl_sync(0xffffffffu, q0.x, leader),
+                                   __shfl_sync(0xffffffffu, q0.y, leader), __shfl_sync(0xffffffffu, q0.z, leader));
+          float gVV = 0.0f, T = 1.0f;  // T replays the cut-off of the first walk
+          for (int skip = 0;; skip += kBwdList) {
+            HitListVis hv{a.t_min, 1.0f, q0.x, q0.y, q0.z, list, skip, kBwdList, 0};
+            packet_walk(a, f, rel, self, groot, mine, xl, yl, zl, 0.0f, hv, sm, rs, skip ? rs.search_nodes : rs.nodes);
+            if (skip == 0 && mine) {
+              V = hv.T;
+              gVV = gV * V;
+            }
+            __syncwarp();  // lane 0's list
+            const int nl = min(hv.total - skip, kBwdList);
+            for (int g = 0; g < nl; g += 32) {
+              const int pos = g + lane < nl ? list[g + lane] : -1;
+              float et;
+              const Beam all{-FLT_MAX, FLT_MAX, -FLT_MAX, FLT_MAX, -FLT_MAX, FLT_MAX};
+              const int cnt = stage_leaves(a.recs, pos, f, rel, all, 0.0f, 0.0f, sm, et);
+              // the lane's leaf: an orthonormal basis (f1, f2) of the plane across a = A w / |A w|, in the
+              // place of the quick test's terms
+              Frame lf;
+              {
+                const float4* rec = a.recs + 4 * (int64_t)max(pos, 0);
+                const float4 q1 = __ldg(rec + 1), q2 = __ldg(rec + 2), q3 = __ldg(rec + 3);
+                const float adx = fmaf(q1.x, f.wx, fmaf(q1.y, f.wy, q1.z * f.wz));
+                const float ady = fmaf(q1.w, f.wx, fmaf(q2.x, f.wy, q2.y * f.wz));
+                const float adz = fmaf(q2.z, f.wx, fmaf(q2.w, f.wy, q3.x * f.wz));
+                const float id = 1.0f / sqrtf(fmaf(adx, adx, fmaf(ady, ady, adz * adz)));
+                lf = make_frame(adx * id, ady * id, adz * id);
+                if (g + lane < nl) {
+                  sm.quick[0][lane] = make_float4(lf.e1x, lf.e1y, lf.e1z, 0.0f);
+                  sm.quick[1][lane] = make_float4(lf.e2x, lf.e2y, lf.e2z, 0.0f);
+                }
+              }
+              __syncwarp();
+              for (int j0 = 0; j0 < cnt; j0 += kBwdBatch) {
+                const int nb = min(kBwdBatch, cnt - j0);
+                for (int b = 0; b < nb; ++b) {
+                  const int j = j0 + b;
+                  float wx, wy, wz, t;
+                  leaf_offset(rel, sm, j, wx, wy, wz, t);
+                  const float d2 = fmaf(wx, wx, fmaf(wy, wy, wz * wz));
+                  const int lp = __float_as_int(sm.stage[3][j].y);
+                  bool h = mine && lp != self && !(T < a.t_min);
+                  if (h) h = ray_decides(a.recs, f, q0.x, q0.y, q0.z, rel, sm, j, lp, d2, t, d2 <= 9.0f && t > 0.0f);
+                  float ga = 0.0f, g2 = 0.0f, p = 0.0f, q = 0.0f;
+                  if (h) {
+                    const float ex = expf(-0.5f * d2);
+                    const float al = sm.stage[0][j].w * ex;
+                    const float om = 1.0f - al;
+                    T *= om;
+                    const float galpha = -gVV / om;
+                    ga = galpha * ex;
+                    g2 = -0.5f * al * galpha;
+                    const float4 s1 = sm.stage[1][j], s2 = sm.stage[2][j], f1 = sm.quick[0][j], f2 = sm.quick[1][j];
+                    p = fmaf(wx, f1.x, fmaf(wy, f1.y, wz * f1.z));
+                    q = fmaf(wx, f2.x, fmaf(wy, f2.y, wz * f2.z));
+                    go1 = fmaf(2.0f * g2, fmaf(wx, s1.x, fmaf(wy, s1.y, wz * s1.z)), go1);
+                    go2 = fmaf(2.0f * g2, fmaf(wx, s2.x, fmaf(wy, s2.y, wz * s2.z)), go2);
+                  }
+                  const float gp = g2 * p, gq = g2 * q;
+                  float (*row)[kBwdRow] = bs.row + 6 * b;
+                  row[0][lane] = ga;
+                  row[1][lane] = gp;
+                  row[2][lane] = gq;
+                  row[3][lane] = gp * p;
+                  row[4][lane] = gp * q;
+                  row[5][lane] = gq * q;
+                }
+                __syncwarp();
+                if (lane < 6 * nb) {
+                  const float4* r4 = reinterpret_cast<const float4*>(bs.row[lane]);
+                  float4 v = r4[0];
+#pragma unroll
+                  for (int i = 1; i < 8; ++i) {
+                    const float4 u = r4[i];
+                    v.x += u.x;
+                    v.y += u.y;
+                    v.z += u.z;
+                    v.w += u.w;
+                  }
+                  bs.sum[j0 + lane / 6][lane % 6] = (v.x + v.y) + (v.z + v.w);
+                }
+                __syncwarp();
+              }
+              if (lane < cnt) {  // w' = p f1 + q f2, x = a cross w' = p f2 - q f1
+                const float4 m = *reinterpret_cast<const float4*>(bs.sum[lane]);
+                const float mpq = bs.sum[lane][4], mqq = bs.sum[lane][5], mpp = m.w;
+                const float x1 = lf.e1x, y1 = lf.e1y, z1 = lf.e1z, x2 = lf.e2x, y2 = lf.e2y, z2 = lf.e2z;
+                float* out = acc + 12 * (int64_t)pos;
+                red_add4(out, m.x, fmaf(m.y, x2, -m.z * x1), fmaf(m.y, y2, -m.z * y1), fmaf(m.y, z2, -m.z * z1));
+                // sum g x x^T = mpp f2 f2 - mpq (f1 f2 + f2 f1) + mqq f1 f1
+                const float u2x = fmaf(mpp, x2, -mpq * x1), u2y = fmaf(mpp, y2, -mpq * y1), u2z = fmaf(mpp, z2, -mpq * z1);
+                const float u1x = fmaf(mqq, x1, -mpq * x2), u1y = fmaf(mqq, y1, -mpq * y2), u1z = fmaf(mqq, z1, -mpq * z2);
+                red_add4(out + 4, fmaf(u2x, x2, u1x * x1), fmaf(u2x, y2, u1x * y1), fmaf(u2x, z2, u1x * z1),
+                         fmaf(u2y, y2, u1y * y1));
+                red_add4(out + 8, fmaf(u2y, z2, u1y * z1), fmaf(u2z, z2, u1z * z1), 0.0f, 0.0f);
+              }
+              __syncwarp();  // the staged leaves are replaced
+            }
+            if (hv.total <= skip + kBwdList) break;
+          }
+          todo &= ~grp;
+        }
+      }
+      if (up) {
+        const float gn = gc * V;  // dL/dn = g c' V, c = n.w
+        red_add4(rayacc + 8 * (int64_t)self, fmaf(go1, f.e1x, go2 * f.e2x), fmaf(go1, f.e1y, go2 * f.e2y),
+                 fmaf(go1, f.e1z, go2 * f.e2z), 0.0f);
+        red_add4(rayacc + 8 * (int64_t)self + 4, gn * d[0], gn * d[1], gn * d[2], 0.0f);
+      }
+      __syncwarp();
+    }
+    __syncwarp();
+  }
+  if (a.stats) {
+    const unsigned long long c0 = warp_sum_u64(rs.nodes), c1 = warp_sum_u64(rs.search_nodes),
+                             c2 = warp_sum_u64(rs.leaves), c3 = warp_sum_u64(rs.hits);
+    if (lane == 0) {
+      atomicAdd(a.stats + 0, c0);
+      atomicAdd(a.stats + 1, c1);
+      atomicAdd(a.stats + 2, c2);
+      atomicAdd(a.stats + 3, c3);
+    }
+  }
+}
+
+// G[s][i] = w sum_k dP_ik Y_k(w_s) and GV[s][i] = G c + dV_is of the receivers of batch [r0, r1), zero
+// where n.w <= 0; one thread per receiver, w = 4 pi / S.
+__global__ void __launch_bounds__(128) k_ray_grad(TraceArgs a, const float* __restrict__ dP, const float* __restrict__ dV,
+                                                  float* __restrict__ G, float* __restrict__ GV) {
+  const int64_t batch = a.r1 - a.r0;
+  const int64_t li = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (li >= batch) return;
+  const int self = (int)(a.r0 + li);
+  const float4 q3 = __ldg(a.recs + 4 * (int64_t)self + 3);
+  const int64_t gid = a.order[self];
+  const int C = sh_count(a.sh_order);
+  const float wq = 4.0f * kPi / (float)a.S;
+  float p[kMaxC];
+#pragma unroll
+  for (int k = 0; k < kMaxC; ++k) p[k] = dP && C <= kMaxC && k < C ? __ldg(dP + gid * C + k) : 0.0f;
+  for (int s = 0; s < a.S; ++s) {
+    const float d[3] = {__ldg(a.dirs + 3 * s), __ldg(a.dirs + 3 * s + 1), __ldg(a.dirs + 3 * s + 2)};
+    const float c = ray_cos(q3.y, q3.z, q3.w, d);
+    float g = 0.0f, gv = 0.0f;
+    if (c > 0.0f) {
+      if (dP && C <= kMaxC) {
+        float Y[kMaxC];
+        sh_eval_dyn(a.sh_order, d[0], d[1], d[2], Y);
+#pragma unroll
+        for (int k = 0; k < kMaxC; ++k)
+          if (k < C) g = fmaf(p[k], Y[k], g);  // Y holds only the first C values
+      } else if (dP) {  // orders 4-6: the direction set's SH table
+        for (int k = 0; k < C; ++k) g = fmaf(__ldg(dP + gid * C + k), __ldg(a.Ytab + (int64_t)s * C + k), g);
+      }
+      g *= wq;
+      gv = g * c + (dV ? __ldg(dV + gid * a.S + s) : 0.0f);
+    }
+    G[(int64_t)s * batch + li] = g;
+    GV[(int64_t)s * batch + li] = gv;
+  }
+}
+
+// The sums of k_packet_bwd to gradients, one thread per Gaussian (sorted position).
+__global__ void __launch_bounds__(128) k_bwd_finish(int64_t n, const float4* __restrict__ recs, const int32_t* __restrict__ order,
+                                                    const float* __restrict__ quats, const float4* __restrict__ acc,
+                                                    const float4* __restrict__ rayacc, float* __restrict__ d_means,
+                                                    float* __restrict__ d_scales, float* __restrict__ d_quats,
+                                                    float* __restrict__ d_opacity, float* __restrict__ d_normals) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int64_t gid = order[i];
+  const float4 a0 = acc[3 * i], a1 = acc[3 * i + 1], a2 = acc[3 * i + 2], go = rayacc[2 * i], gn = rayacc[2 * i + 1];
+  const float M[3][3] = {{a1.x, a1.y, a1.z}, {a1.y, a1.w, a2.x}, {a1.z, a2.x, a2.y}};
+  float gs[3] = {0.f, 0.f, 0.f}, gm[3] = {0.f, 0.f, 0.f}, gq[4] = {0.f, 0.f, 0.f, 0.f};
+  if (a0.x != 0.f || a0.y != 0.f || a0.z != 0.f || a0.w != 0.f || a1.x != 0.f || a1.w != 0.f || a2.y != 0.f) {
+    const float4 q1 = __ldg(recs + 4 * i + 1), q2 = __ldg(recs + 4 * i + 2), q3 = __ldg(recs + 4 * i + 3);
+    const float A[3][3] = {{q1.x, q1.y, q1.z}, {q1.w, q2.x, q2.y}, {q2.z, q2.w, q3.x}};
+    float gR[3][3], Rs[3][3], inv_s[3];  // Rs[l][j] = R_jl s_l = A_lj s_l^2
+#pragma unroll
+    for (int l = 0; l < 3; ++l) {
+      const float i2 = A[l][0] * A[l][0] + A[l][1] * A[l][1] + A[l][2] * A[l][2];
+      inv_s[l] = sqrtf(i2);
+      const float s2 = 1.0f / i2;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) Rs[l][j] = A[l][j] * s2;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      gs[k] = -2.0f * M[k][k] * inv_s[k];
+      gm[k] = -2.0f * (A[0][k] * a0.y + A[1][k] * a0.z + A[2][k] * a0.w);
+#pragma unroll
+      for (int j = 0; j < 3; ++j) gR[j][k] = 2.0f * inv_s[k] * (Rs[0][j] * M[k][0] + Rs[1][j] * M[k][1] + Rs[2][j] * M[k][2]);
+    }
+    quat_backward(quats[4 * gid], quats[4 * gid + 1], quats[4 * gid + 2], quats[4 * gid + 3], gR, gq);
+  }
+  d_opacity[gid] = a0.x;
+  const float gor[3] = {go.x, go.y, go.z}, gnr[3] = {gn.x, gn.y, gn.z};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    d_means[3 * gid + k] = gm[k] + gor[k];
+    d_scales[3 * gid + k] = gs[k];
+    d_normals[3 * gid + k] = gnr[k];
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) d_quats[4 * gid + k] = gq[k];
+}
+
+// Receivers per launch: G and GV hold S floats each per receiver, at most 2^26.
+static int64_t bwd_batch(int64_t n, int S) {
+  int64_t b = ((int64_t(1) << 26) / (S > 0 ? S : 1)) / 64 * 64;
+  if (b < 64) b = 64;
+  return b < n ? b : n;
+}
+
+size_t packet_bwd_workspace(int64_t n, int S, int sms) {
+  return 2 * align_up(sizeof(float) * (size_t)bwd_batch(n, S) * S) + align_up(sizeof(float) * 20 * (size_t)n) +
+         align_up(sizeof(int) * (size_t)sms * kBwdBlocks * kPacketWarps * kBwdList);
+}
+
+int launch_packet_bwd(TraceArgs a, const float* quats, const float* dP, const float* dV, float* d_means, float* d_scales,
+                      float* d_quats, float* d_opacity, float* d_normals, void* ws, int sms, cudaStream_t stream) {
+  const int64_t b = bwd_batch(a.n, a.S);
+  Carver c(ws);
+  float* G = c.take<float>((size_t)b * a.S);
+  float* GV = c.take<float>((size_t)b * a.S);
+  float* acc = c.take<float>(20 * (size_t)a.n);  // [n][12], then [n][8] of the receivers
+  int* lists = c.take<int>((size_t)sms * kBwdBlocks * kPacketWarps * kBwdList);
+  float* rayacc = acc + 12 * a.n;
+  cudaMemsetAsync(acc, 0, sizeof(float) * 20 * a.n, stream);
+  const size_t smem = (sizeof(PacketSmem) + sizeof(BwdSmem)) * kPacketWarps;
+  cudaFuncSetAttribute(k_packet_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaFuncSetAttribute(k_packet_bwd, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  int per_sm = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_packet_bwd, kPacketThreads, smem);
+  per_sm = per_sm < 1 ? 1 : (per_sm > kBwdBlocks ? kBwdBlocks : per_sm);
+  for (int64_t r0 = 0; r0 < a.n; r0 += b) {
+    a.r0 = r0;
+    a.r1 = r0 + b < a.n ? r0 + b : a.n;
+    cudaMemsetAsync(a.work, 0, sizeof(unsigned int), stream);
+    k_ray_grad<<<(unsigned)((a.r1 - a.r0 + 127) / 128), 128, 0, counted(stream)>>>(a, dP, dV, G, GV);
+    k_packet_bwd<<<sms * per_sm, kPacketThreads, smem, counted(stream)>>>(a, G, GV, acc, rayacc, lists);
+  }
+  k_bwd_finish<<<(unsigned)((a.n + 127) / 128), 128, 0, counted(stream)>>>(
+      a.n, a.recs, a.order, quats, reinterpret_cast<const float4*>(acc), reinterpret_cast<const float4*>(rayacc), d_means,
+      d_scales, d_quats, d_opacity, d_normals);
+  PRTGS_CHECK_LAUNCH();
+  return PRTGS_OK;
 }
 
 // P of the receivers of batch [r0, r1) from V[s][i]: one lane per receiver, a compensated sum

@@ -64,3 +64,50 @@ def test_packet_many_hits_per_ray():
     sc.means *= 0.2
     sc.opacity *= np.float32(0.1)
     _check(sc, np.array([0, sc.n], np.int64), S.direction_set(24, 7), 1, [sc.n])
+
+
+GRADS = ("means", "scales", "quats", "opacity", "normals")
+
+
+def _grads_against_autograd(parts, dirs, order, t_min):
+    """The packet backward of several scenes in one call against FP64 autograd of each scene's
+    brute-force P (tolerance of test_gpu_transfer.py: 2e-3 norm-wise per field)."""
+    from oracle import transfer_torch as TT
+
+    sc, offs = S.concat_scenes(parts)
+    g = api.GaussianTensors.from_scene(sc)
+    st = api.Status()
+    bvh = api.build_bvh(g, torch.from_numpy(offs).cuda(), status=st)
+    w = np.random.default_rng(sc.n).standard_normal((sc.n, (order + 1) ** 2)).astype(np.float32)
+    w[::7] = 0.0  # receivers without a gradient
+    out = api.precompute_transfer_backward(g, bvh, torch.from_numpy(dirs).cuda(), order, torch.from_numpy(w).cuda(),
+                                           t_min=t_min, status=st)
+    torch.cuda.synchronize()
+    assert st.read() == 0
+    for b, p in enumerate(parts):
+        at = slice(int(offs[b]), int(offs[b + 1]))
+        ps = [torch.tensor(np.asarray(getattr(p, f), np.float64), requires_grad=True) for f in GRADS]
+        P = TT.transfer_P(*ps, dirs, oracle.sh(order, dirs))
+        ref = torch.autograd.grad((P * torch.as_tensor(w[at].astype(np.float64))).sum(), ps, allow_unused=True)
+        top = max(float(r.norm()) for r in ref if r is not None)
+        for f, r in zip(GRADS, ref):
+            a = out["d_" + f].cpu().double()[at]
+            r = torch.zeros_like(a) if r is None else r
+            assert float((a - r).norm()) <= 2e-3 * max(float(r.norm()), 1e-3 * top), (b, f)
+
+
+@pytest.mark.parametrize("sizes", [[33], [64, 65], [1, 130, 2, 257]])
+def test_packet_backward_windows(sizes):
+    parts = [S.surface_scene(n, 500 + n) for n in sizes]
+    for p in parts:
+        p.means *= 0.3
+    _grads_against_autograd(parts, S.direction_set(29, 8), 2, 0.0)
+
+
+def test_packet_backward_list_overflow():
+    """More hit leaves per packet than the kernel keeps at a time (2,048): faint splats all over
+    one another, so that the list is continued by further walks."""
+    sc = S.surface_scene(2600, 43)
+    sc.means *= 0.02
+    sc.opacity *= np.float32(0.02)
+    _grads_against_autograd([sc], S.direction_set(5, 9), 1, 0.0)
