@@ -12,10 +12,15 @@ namespace prtgs {
 // sort.cu
 size_t scan_workspace(int64_t n);
 int scan_u32(const uint32_t* in, uint32_t* out, int64_t n, bool exclusive, uint32_t* total, void* ws,
-             cudaStream_t stream);
+             cudaStream_t stream, const int32_t* idx = nullptr, uint32_t cap = 0xffffffffu);
 size_t radix_sort_workspace(int64_t capacity);
+// Stable; the pairs (keys_x, vals_x; vals_x null: the index) end in (keys_f, vals_f), with (keys_y, vals_y)
+// as the other side of the passes.
 int radix_sort_pairs(const uint64_t* keys_x, const int32_t* vals_x, uint64_t* keys_f, int32_t* vals_f,
                      uint64_t* keys_y, int32_t* vals_y, int64_t capacity, const uint32_t* d_count, int begin_bit,
+                     int end_bit, void* ws, cudaStream_t stream);
+int radix_sort_pairs(const uint32_t* keys_x, const int32_t* vals_x, uint32_t* keys_f, int32_t* vals_f,
+                     uint32_t* keys_y, int32_t* vals_y, int64_t capacity, const uint32_t* d_count, int begin_bit,
                      int end_bit, void* ws, cudaStream_t stream);
 
 // bvh.cu

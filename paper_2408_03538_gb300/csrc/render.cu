@@ -2,9 +2,9 @@
 // front-to-back alpha blending) with the 3DGS conventions the paper builds on, and its
 // backward pass.
 //
-// Forward: k_preprocess (one thread per Gaussian) -> inclusive scan of the touched-tile
-// counts -> k_duplicate writes (tile << 32 | depth bits, Gaussian) pairs -> radix sort on
-// the device-side pair count -> k_ranges -> k_composite (one 16x16-pixel tile per block,
+// Forward: k_preprocess (one thread per Gaussian) -> the Gaussians in depth order (radix sort of the depth
+// bits) -> inclusive scan of the touched-tile counts in that order -> k_duplicate writes (tile, Gaussian)
+// pairs -> stable radix sort by tile, on the device-side pair count -> k_ranges -> k_composite (one 16x16-pixel tile per block,
 // Gaussians staged through shared memory in batches of 256, evaluated once for a group of
 // up to 8 light colour sets).
 // Backward: k_composite_bwd walks each pixel's list back to front from its last contributor and sums
@@ -121,8 +121,8 @@ int render_state_layout_batched(void* buffer, int64_t n, int32_t B, int32_t widt
 }
 
 size_t render_workspace(int64_t n, int32_t, int32_t, int64_t max_pairs) {
-  return scan_workspace(n) + 2 * align_up(sizeof(uint64_t) * max_pairs) + 2 * align_up(sizeof(int32_t) * max_pairs) +
-         radix_sort_workspace(max_pairs);
+  return scan_workspace(n) + 6 * align_up(sizeof(uint32_t) * n) + 5 * align_up(sizeof(uint32_t) * max_pairs) +
+         radix_sort_workspace(max_pairs > n ? max_pairs : n);
 }
 
 __device__ __forceinline__ void quat_rot(float qw, float qx, float qy, float qz, float R[3][3]) {
@@ -157,12 +157,14 @@ template <class V>
 __global__ void k_preprocess(int64_t n, const float* __restrict__ means, const float* __restrict__ scales,
                              const float* __restrict__ quats, const float* __restrict__ opacity, V v,
                              float* __restrict__ mean2d, float4* __restrict__ conic_op, float* __restrict__ depth,
-                             int32_t* __restrict__ radius, uint32_t* __restrict__ touched) {
+                             int32_t* __restrict__ radius, uint32_t* __restrict__ touched,
+                             uint32_t* __restrict__ depth_key) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const Cam& c = v.cam(v.scene_of(i));
   radius[i] = 0;
   touched[i] = 0;
+  depth_key[i] = 0xffffffffu;  // behind every visible splat
   const float mx = means[3 * i], my = means[3 * i + 1], mz = means[3 * i + 2];
   const float x = c.r[0] * mx + c.r[1] * my + c.r[2] * mz + c.t[0];
   const float y = c.r[3] * mx + c.r[4] * my + c.r[5] * mz + c.t[1];
@@ -208,47 +210,76 @@ __global__ void k_preprocess(int64_t n, const float* __restrict__ means, const f
   conic_op[i] = make_float4(cc * idet, -b * idet, a * idet, opacity[i]);
   radius[i] = r;
   touched[i] = cnt;
+  depth_key[i] = __float_as_uint(z);  // z > 0: the bits order as the depths
 }
 
+// (tile, Gaussian) pairs in depth order: a warp takes 32 splats of that order and writes their pairs, the
+// lanes on consecutive pairs (each finds its splat in the warp's prefix sums), so that the writes coalesce and a
+// splat of many tiles does not hold the others up. (A thread per splat took 0.54 ms for the 25 M pairs of 300k
+// splats; this takes 0.075.)
 template <class V>
-__global__ void k_duplicate(int64_t n, V v, const float* __restrict__ mean2d, const float* __restrict__ depth,
-                            const int32_t* __restrict__ radius, const uint32_t* __restrict__ incl,
-                            int64_t max_pairs, uint64_t* __restrict__ keys, int32_t* __restrict__ ids,
-                            int32_t* status) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int r = radius[i];
-  if (r <= 0) return;
-  const int b = v.scene_of(i);
-  const Cam& c = v.cam(b);
-  const uint64_t tile0 = (uint64_t)b * (uint64_t)(c.gx * c.gy);  // the scene's first tile
-  int x0, y0, x1, y1;
-  tile_rect(mean2d[2 * i], mean2d[2 * i + 1], r, c, x0, y0, x1, y1);
-  const uint32_t end = incl[i];
-  int64_t p = (int64_t)end - (int64_t)((x1 - x0) * (y1 - y0));
-  if ((int64_t)end > max_pairs) set_status(status, PRTGS_STATUS_CAPACITY);
-  const uint64_t dbits = (uint64_t)__float_as_uint(depth[i]);
-  for (int ty = y0; ty < y1; ++ty)
-    for (int tx = x0; tx < x1; ++tx, ++p) {
-      if (p >= max_pairs) return;
-      keys[p] = ((tile0 + (uint64_t)(ty * c.gx + tx)) << 32) | dbits;
-      ids[p] = (int32_t)i;
+__global__ void __launch_bounds__(256) k_duplicate(int64_t n, V v, const int32_t* __restrict__ by_depth,
+                                                   const float* __restrict__ mean2d, const int32_t* __restrict__ radius,
+                                                   const uint32_t* __restrict__ incl, int64_t max_pairs,
+                                                   uint32_t* __restrict__ tiles, int32_t* __restrict__ ids,
+                                                   int32_t* status) {
+  const int lane = threadIdx.x & 31;
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  int g = 0, x0 = 0, y0 = 0, w = 1, count = 0;
+  uint32_t tile0 = 0;
+  if (i < n) {
+    g = by_depth[i];
+    const int r = radius[g];
+    if (r > 0) {
+      const int b = v.scene_of(g);
+      const Cam& c = v.cam(b);
+      int x1, y1;
+      tile_rect(mean2d[2 * (int64_t)g], mean2d[2 * (int64_t)g + 1], r, c, x0, y0, x1, y1);
+      w = x1 - x0;
+      count = w * (y1 - y0);
+      tile0 = (uint32_t)(b * (c.gx * c.gy) + y0 * c.gx + x0);  // the splat's first tile
+      if ((int64_t)incl[i] > max_pairs) set_status(status, PRTGS_STATUS_CAPACITY);
     }
+  }
+  const int gx = v.cam(0).gx;
+  int end = count;  // inclusive prefix sum over the warp
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, end, off);
+    if (lane >= off) end += y;
+  }
+  const int total = __shfl_sync(0xffffffffu, end, 31);
+  if (total == 0) return;
+  const int64_t first = (int64_t)__shfl_sync(0xffffffffu, i < n ? incl[i] : 0u, 0) - __shfl_sync(0xffffffffu, count, 0);
+  for (int base = 0; base < total; base += 32) {
+    const int p = base + lane;
+    int o = 0;  // the first lane whose prefix sum is above p
+#pragma unroll
+    for (int step = 16; step > 0; step >>= 1)
+      if (__shfl_sync(0xffffffffu, end, o + step - 1) <= p) o += step;
+    o = min(o, 31);
+    const int og = __shfl_sync(0xffffffffu, g, o), ow = __shfl_sync(0xffffffffu, w, o);
+    const uint32_t ot = __shfl_sync(0xffffffffu, tile0, o);
+    const int k = p - __shfl_sync(0xffffffffu, end - count, o);
+    if (p < total && first + p < max_pairs) {
+      tiles[first + p] = ot + (uint32_t)((k / ow) * gx + k % ow);
+      ids[first + p] = og;
+    }
+  }
 }
 
-__global__ void k_clamp_count(uint32_t* count, int64_t max_pairs) {
-  if (*count > (uint64_t)max_pairs) *count = (uint32_t)max_pairs;
-}
-
-__global__ void k_ranges(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ count, int64_t tiles,
-                         uint32_t* __restrict__ ranges) {
-  int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  int64_t n = *count;
+// Tile ranges of the sorted pairs, and the pairs' (tile << 32 | depth bits).
+__global__ void k_ranges(const uint32_t* __restrict__ tile_of, const int32_t* __restrict__ ids,
+                         const float* __restrict__ depth, const uint32_t* __restrict__ count, int64_t tiles,
+                         uint32_t* __restrict__ ranges, uint64_t* __restrict__ keys) {
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t n = *count;
   if (p >= n) return;
-  uint32_t tile = (uint32_t)(keys[p] >> 32);
+  const uint32_t tile = tile_of[p];
+  keys[p] = ((uint64_t)tile << 32) | __float_as_uint(depth[ids[p]]);
   if ((int64_t)tile >= tiles) return;
-  if (p == 0 || (uint32_t)(keys[p - 1] >> 32) != tile) ranges[2 * tile] = (uint32_t)p;
-  if (p == n - 1 || (uint32_t)(keys[p + 1] >> 32) != tile) ranges[2 * tile + 1] = (uint32_t)(p + 1);
+  if (p == 0 || tile_of[p - 1] != tile) ranges[2 * tile] = (uint32_t)p;
+  if (p == n - 1 || tile_of[p + 1] != tile) ranges[2 * tile + 1] = (uint32_t)(p + 1);
 }
 
 // Whether a splat can have alpha >= 1/255 at any pixel centre of [x0, x1] x [y0, y1]: the bounding box of its
@@ -362,32 +393,44 @@ static int render_views(const prtgs_gaussians* g, const float* colors, int32_t k
   const int64_t tiles = (int64_t)c.gx * c.gy * B;
   Carver cv(ws);
   void* scan_ws = cv.take<char>(scan_workspace(n));
-  uint64_t* keys_x = cv.take<uint64_t>(st->max_pairs);
-  uint64_t* keys_y = cv.take<uint64_t>(st->max_pairs);
+  uint32_t* dkey[3];
+  for (auto& p : dkey) p = cv.take<uint32_t>(n);
+  int32_t* by_depth = cv.take<int32_t>(n);
+  int32_t* by_depth_y = cv.take<int32_t>(n);
+  uint32_t* incl = cv.take<uint32_t>(n);
+  uint32_t* tkey[3];
+  for (auto& p : tkey) p = cv.take<uint32_t>(st->max_pairs);
   int32_t* ids_x = cv.take<int32_t>(st->max_pairs);
   int32_t* ids_y = cv.take<int32_t>(st->max_pairs);
-  void* sort_ws = cv.take<char>(radix_sort_workspace(st->max_pairs));
+  void* sort_ws = cv.take<char>(radix_sort_workspace(st->max_pairs > n ? st->max_pairs : n));
   cudaMemsetAsync(st->ranges, 0, sizeof(uint32_t) * 2 * tiles, stream);
-  cudaMemsetAsync(st->n_pairs, 0, sizeof(uint32_t), stream);
+  if (n == 0) cudaMemsetAsync(st->n_pairs, 0, sizeof(uint32_t), stream);
   if (n > 0) {
-    k_preprocess<V><<<(unsigned)((n + 255) / 256), 256, 0, counted(stream)>>>(
+    const unsigned blocks = (unsigned)((n + 255) / 256);
+    k_preprocess<V><<<blocks, 256, 0, counted(stream)>>>(
         n, g->means, g->scales, g->quats, g->opacity, v, st->mean2d, reinterpret_cast<float4*>(st->conic_op),
-        st->depth, st->radius, st->tiles_touched);
+        st->depth, st->radius, st->tiles_touched, dkey[0]);
     PRTGS_CHECK_LAUNCH();
-    int rc = scan_u32(st->tiles_touched, st->tiles_touched, n, false, st->n_pairs, scan_ws, stream);
+    // The (tile, depth) order as the splats' depth order followed by a stable sort of the pairs by tile: the
+    // 32 depth bits are sorted once per splat instead of once per pair (25 M pairs of 300k splats: six
+    // passes over 12-byte pairs, 1.57 ms, became two over 8-byte ones and four short ones, 0.60 ms).
+    int rc = radix_sort_pairs(dkey[0], nullptr, dkey[2], by_depth, dkey[1], by_depth_y, n, nullptr, 0, 32, sort_ws, stream);
     if (rc != PRTGS_OK) return rc;
-    k_duplicate<V><<<(unsigned)((n + 255) / 256), 256, 0, counted(stream)>>>(n, v, st->mean2d, st->depth, st->radius,
-                                                                   st->tiles_touched, st->max_pairs, keys_x, ids_x,
-                                                                   status);
-    k_clamp_count<<<1, 1, 0, counted(stream)>>>(st->n_pairs, st->max_pairs);
+    const uint32_t cap = (uint32_t)(st->max_pairs < 0xffffffffll ? st->max_pairs : 0xffffffffll);
+    rc = scan_u32(st->tiles_touched, incl, n, false, nullptr, scan_ws, stream, by_depth);
+    if (rc != PRTGS_OK) return rc;
+    rc = scan_u32(st->tiles_touched, st->tiles_touched, n, false, st->n_pairs, scan_ws, stream, nullptr, cap);
+    if (rc != PRTGS_OK) return rc;
+    k_duplicate<V><<<blocks, 256, 0, counted(stream)>>>(n, v, by_depth, st->mean2d, st->radius, incl, st->max_pairs, tkey[0],
+                                                        ids_x, status);
     PRTGS_CHECK_LAUNCH();
     int tile_bits = 0;
     while ((int64_t(1) << tile_bits) < tiles) ++tile_bits;
-    rc = radix_sort_pairs(keys_x, ids_x, st->pair_keys, st->pair_ids, keys_y, ids_y, st->max_pairs, st->n_pairs, 0,
-                          32 + tile_bits, sort_ws, stream);
+    rc = radix_sort_pairs(tkey[0], ids_x, tkey[2], st->pair_ids, tkey[1], ids_y, st->max_pairs, st->n_pairs, 0, tile_bits,
+                          sort_ws, stream);
     if (rc != PRTGS_OK) return rc;
-    k_ranges<<<(unsigned)((st->max_pairs + 255) / 256), 256, 0, counted(stream)>>>(st->pair_keys, st->n_pairs, tiles,
-                                                                            st->ranges);
+    k_ranges<<<(unsigned)((st->max_pairs + 255) / 256), 256, 0, counted(stream)>>>(
+        tkey[2], st->pair_ids, st->depth, st->n_pairs, tiles, st->ranges, st->pair_keys);
     PRTGS_CHECK_LAUNCH();
   }
   const int kg = k <= 1 ? 1 : (k <= 4 ? 4 : 8);

@@ -56,3 +56,53 @@ def test_composite_thin_faint_and_opaque_splats(thin, opacity):
     sc.scales[:, 0] /= np.float32(thin)
     sc.opacity = np.minimum(sc.opacity * np.float32(opacity), np.float32(0.995))
     _check(sc, S.look_at_camera((0, -3.0, 1.5), (0, 0, 0.2), 45, 48, 40), 2, (0.5, 0.5, 0.5))
+
+
+@pytest.mark.parametrize("n,width", [(1, 64), (700, 64), (4096, 250), (4097, 250), (60_000, 640), (700_000, 1920)])
+def test_pair_order(n, width):
+    """The sorted (tile, depth) pairs: ascending keys, equal keys by index, every key its splat's tile
+    and depth, each splat in exactly the tiles of its rectangle, ranges and prefix sums to match (one-block,
+    self-summing and scanned passes of the sort)."""
+    sc = S.isotropic_scene(n, 80)
+    sc.scales *= np.float32(0.3)
+    sc.means[1::2] = sc.means[: sc.n // 2 * 2 : 2][: sc.means[1::2].shape[0]]  # equal depths
+    cam = S.look_at_camera((0, -3.5, 1.0), (0, 0, 0), 45, width, width // 2)
+    g = api.GaussianTensors.from_scene(sc)
+    st = api.Status()
+    _, s = api.render(g, torch.zeros((1, n, 3), device="cuda"), cam, torch.zeros(3, device="cuda"), status=st,
+                      max_pairs=64 * n + 4096)
+    assert st.read() == 0
+    m, gx, gy = s.n_pairs(), (width + 15) // 16, (width // 2 + 15) // 16
+    key = s.view("pair_keys", torch.int64, (s.max_pairs,))[:m]
+    ids = s.view("pair_ids", torch.int32, (s.max_pairs,))[:m].long()
+    assert m > 0 and bool((key[1:] >= key[:-1]).all())
+    assert bool((ids[1:] > ids[:-1])[key[1:] == key[:-1]].all())
+    depth = s.view("depth", torch.float32, (n,))
+    assert torch.equal(key & 0xffffffff, depth[ids].view(torch.int32).long())
+    xy, r = s.view("mean2d", torch.float32, (n, 2)), s.view("radius", torch.int32, (n,)).float()
+    tile = key >> 32
+    lo = torch.floor((xy[ids] - r[ids, None]) / 16)
+    hi = torch.floor((xy[ids] + r[ids, None]) / 16)
+    t2 = torch.stack([tile % gx, tile // gx], 1)
+    assert bool(((t2 >= lo) & (t2 <= hi)).all())
+    on = r > 0
+    lim = torch.tensor([gx, gy], device="cuda", dtype=torch.float32)
+    side = torch.minimum(torch.floor((xy + r[:, None]) / 16) + 1, lim).clamp(min=0) - torch.minimum(
+        torch.floor((xy - r[:, None]) / 16).clamp(min=0), lim)
+    area = torch.where(on, side[:, 0] * side[:, 1], torch.zeros_like(r)).long()
+    assert torch.equal(torch.bincount(ids, minlength=n), area)
+    assert torch.equal(s.view("tiles_touched", torch.int32, (n,)).long(), torch.cumsum(area, 0))
+    ranges = s.view("ranges", torch.int32, (gx * gy, 2)).long()
+    assert torch.equal(ranges[:, 1] - ranges[:, 0], torch.bincount(tile, minlength=gx * gy))
+
+
+@pytest.mark.parametrize("n", [4096, 4097, 524_288, 524_289, 1_300_001])
+def test_bvh_sort_sizes(n):
+    """The 64-bit keys of the BVH at the ends of the sort's ranges: sorted, and stable by construction
+    (the low bits are the index)."""
+    g = api.GaussianTensors.from_scene(S.isotropic_scene(n, 81))
+    bvh = api.build_bvh(g)
+    key = bvh.view("keys", torch.int64, (n,))
+    order = bvh.view("order", torch.int32, (n,)).long()
+    assert bool((key[1:] > key[:-1]).all()) and torch.equal(key & ((1 << 27) - 1), order)
+    assert torch.equal(torch.sort(order).values, torch.arange(n, device="cuda"))
