@@ -126,6 +126,10 @@ int render_state_layout(void* buffer, int64_t n, int32_t width, int32_t height, 
 size_t render_workspace(int64_t n, int32_t width, int32_t height, int64_t max_pairs);
 int render(const prtgs_gaussians* g, const float* colors, int32_t k, const prtgs_camera* cam, const float* bg,
            float* image, prtgs_render_state* st, int32_t* status, void* ws, cudaStream_t stream);
+// render() with the splats' colours as rows [n][render_rows_floats(k)], 16-byte aligned: set l, channel c at 3 l + c
+int render_rows(const prtgs_gaussians* g, const float* rows, int32_t k, const prtgs_camera* cam, const float* bg,
+                float* image, prtgs_render_state* st, int32_t* status, void* ws, cudaStream_t stream);
+size_t render_rows_floats(int32_t k);
 size_t render_geometry_workspace(int64_t n, int32_t width, int32_t height, int64_t max_pairs);
 int render_geometry(const prtgs_gaussians* g, const prtgs_camera* cam, float* depth, float* normal,
                     prtgs_render_state* st, int32_t* status, void* ws, cudaStream_t stream);

@@ -1,6 +1,8 @@
 // Relight contraction (Eq. 14; glossy splats Eq. 41) and its backward pass.
 //
 // colors[k,i,c] = (rho_i[c] / pi) * sum_m T_i[c or 0][m] L[k,c,m]
+#include <type_traits>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -190,42 +192,58 @@ int relight(int64_t n, int32_t order, const float* T, int32_t t_channels, const 
 // The composite is linear in the splat colours: with colours (rho_i/pi) (T_i . L_l) every
 // light's image is sum_m TI[m,c,p] L[l,c,m] + bg[c] final_T[p], TI the composite of the
 // features F[m,i,c] = (rho_i[c]/pi) T_i[c][m] (glossy splats: t_eff = M_i Y(v_i), Eq. 41).
-template <int TCH>
-__global__ void k_transfer_features(int64_t n, int C, const float* __restrict__ T, const float* __restrict__ albedo,
-                                    float* __restrict__ F) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float r[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) r[c] = __ldg(albedo + 3 * i + c) * (1.0f / kPi);
-  for (int m = 0; m < C; ++m)
-#pragma unroll
-    for (int c = 0; c < 3; ++c) F[((int64_t)m * n + i) * 3 + c] = r[c] * __ldg(T + (i * TCH + (TCH > 1 ? c : 0)) * C + m);
+// Splats of a k_glossy_features block: a thread per coefficient, at most 40 KB of matrices.
+constexpr int glossy_group(int C) {
+  return (256 / C) * C * (C | 1) <= 10240 ? 256 / C : 10240 / (C * (C | 1));
 }
 
-template <int ORDER>
-__global__ void k_glossy_features(int64_t n, int64_t n_glossy, const int32_t* __restrict__ ids,
-                                  const float* __restrict__ M, const float* __restrict__ means, float cx, float cy,
-                                  float cz, const float* __restrict__ albedo, float* __restrict__ F) {
-  constexpr int C = (ORDER + 1) * (ORDER + 1);
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= n_glossy) return;
-  const int64_t i = ids[g];
-  const float vx = cx - means[3 * i], vy = cy - means[3 * i + 1], vz = cz - means[3 * i + 2];
-  const float rn = rsqrtf(vx * vx + vy * vy + vz * vz);
-  float Y[C];
-  sh_eval_any<ORDER>(vx * rn, vy * rn, vz * rn, Y);
-  float r[3];
+// F is laid out in rows of render_rows_floats(C), F[m,i,c] at i's 3 m + c, as the composite reads them.
+template <int C, int TCH>
+__global__ void __launch_bounds__(256) k_transfer_features(int64_t n, const float* __restrict__ T,
+                                                           const float* __restrict__ albedo, float4* __restrict__ F) {
+  constexpr int Q = (3 * C + 3) / 4;  // 16-byte words of a row, one per thread
+  const int64_t at = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t i = at / Q;
+  if (i >= n) return;
+  const int e0 = 4 * (int)(at - i * Q);
+  float f[4];
 #pragma unroll
-  for (int c = 0; c < 3; ++c) r[c] = __ldg(albedo + 3 * i + c) * (1.0f / kPi);
-#pragma unroll
-  for (int a = 0; a < C; ++a) {
-    float te = 0.f;
-#pragma unroll
-    for (int b = 0; b < C; ++b) te = fmaf(__ldg(M + (g * C + a) * C + b), Y[b], te);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) F[((int64_t)a * n + i) * 3 + c] = r[c] * te;
+  for (int j = 0; j < 4; ++j) {
+    const int m = (e0 + j) / 3, c = (e0 + j) % 3;
+    f[j] = m < C ? __ldg(albedo + 3 * i + c) * (1.0f / kPi) * __ldg(T + (i * TCH + (TCH > 1 ? c : 0)) * C + m) : 0.f;
   }
+  F[at] = make_float4(f[0], f[1], f[2], f[3]);
+}
+
+// The rows of the glossy splats. A block stages the matrices of a few splats in shared memory (coalesced, at
+// an odd row stride) and takes one coefficient per thread: a thread per splat reading its own kilobyte took 283 us
+// for 300k splats at order 3 (the bytes alone take 70).
+template <int ORDER>
+__global__ void __launch_bounds__(256) k_glossy_features(int64_t n_glossy, const int32_t* __restrict__ ids,
+                                                         const float* __restrict__ M, const float* __restrict__ means,
+                                                         float cx, float cy, float cz,
+                                                         const float* __restrict__ albedo, float* __restrict__ F) {
+  constexpr int C = (ORDER + 1) * (ORDER + 1), P = C | 1, G = glossy_group(C), RS = (3 * C + 3) / 4 * 4;
+  __shared__ float sM[G * C * P];
+  __shared__ float sY[G][C];
+  const int64_t g0 = (int64_t)blockIdx.x * G;
+  const int ng = (int)min((int64_t)G, n_glossy - g0);
+  for (int e = threadIdx.x; e < ng * C * C; e += 256) sM[e / C * P + e % C] = __ldg(M + g0 * C * C + e);
+  if (threadIdx.x < ng) {
+    const int64_t i = ids[g0 + threadIdx.x];
+    const float vx = cx - means[3 * i], vy = cy - means[3 * i + 1], vz = cz - means[3 * i + 2];
+    const float rn = rsqrtf(vx * vx + vy * vy + vz * vz);
+    sh_eval_any<ORDER>(vx * rn, vy * rn, vz * rn, sY[threadIdx.x]);
+  }
+  __syncthreads();
+  if (threadIdx.x >= ng * C) return;
+  const int g = threadIdx.x / C, a = threadIdx.x % C;
+  const int64_t i = ids[g0 + g];
+  float te = 0.f;
+#pragma unroll
+  for (int b = 0; b < C; ++b) te = fmaf(sM[threadIdx.x * P + b], sY[g][b], te);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) F[i * RS + 3 * a + c] = __ldg(albedo + 3 * i + c) * (1.0f / kPi) * te;
 }
 
 // FP32 form: one thread per pixel, the lights in shared memory.
@@ -303,7 +321,7 @@ static void launch_pixel_relight_hi(int64_t n_pix, const float* TI, const float*
 size_t render_relit_workspace(int64_t n, int32_t order, int32_t width, int32_t height, int64_t max_pairs) {
   const int C = sh_count(order);
   const int64_t n_pix = (int64_t)width * height;
-  return align_up(sizeof(float) * (size_t)C * n * 3) + align_up(sizeof(float) * (size_t)C * 3 * n_pix) +
+  return align_up(sizeof(float) * render_rows_floats(C) * n) + align_up(sizeof(float) * (size_t)C * 3 * n_pix) +
          align_up(sizeof(float) * 4) + render_workspace(n, width, height, max_pairs);
 }
 
@@ -315,33 +333,35 @@ int render_relit(const prtgs_gaussians* g, int32_t order, const float* T, int32_
   const int C = sh_count(order);
   const int64_t n_pix = (int64_t)cam->width * cam->height;
   Carver cv(ws);
-  float* F = cv.take<float>((size_t)C * n * 3);
+  float* F = cv.take<float>(render_rows_floats(C) * n);
   float* TI = cv.take<float>((size_t)C * 3 * n_pix);
   float* zero = cv.take<float>(4);
   void* rws = static_cast<char*>(ws) + cv.off;
   cudaMemsetAsync(zero, 0, sizeof(float) * 4, stream);
   if (n > 0) {
-    const unsigned blocks = (unsigned)((n + 255) / 256);
-    if (t_channels == 3) k_transfer_features<3><<<blocks, 256, 0, counted(stream)>>>(n, C, T, g->albedo, F);
-    else k_transfer_features<1><<<blocks, 256, 0, counted(stream)>>>(n, C, T, g->albedo, F);
-    if (n_glossy > 0) {
-      const unsigned gb = (unsigned)((n_glossy + 255) / 256);
-      const float px = cam->pos[0], py = cam->pos[1], pz = cam->pos[2];
-#define PRTGS_GF(O) k_glossy_features<O><<<gb, 256, 0, counted(stream)>>>(n, n_glossy, glossy_ids, M, g->means, px, py, pz, \
-                                                                         g->albedo, F)
-      switch (order) {
-        case 1: PRTGS_GF(1); break;
-        case 2: PRTGS_GF(2); break;
-        case 3: PRTGS_GF(3); break;
-        case 4: PRTGS_GF(4); break;
-        case 5: PRTGS_GF(5); break;
-        default: PRTGS_GF(6); break;
-      }
-#undef PRTGS_GF
+    const float px = cam->pos[0], py = cam->pos[1], pz = cam->pos[2];
+    auto features = [&](auto order_c) {
+      constexpr int O = decltype(order_c)::value, K = (O + 1) * (O + 1), G = glossy_group(K);
+      const unsigned blocks = (unsigned)((n * ((3 * K + 3) / 4) + 255) / 256);
+      if (t_channels == 3)
+        k_transfer_features<K, 3><<<blocks, 256, 0, counted(stream)>>>(n, T, g->albedo, reinterpret_cast<float4*>(F));
+      else
+        k_transfer_features<K, 1><<<blocks, 256, 0, counted(stream)>>>(n, T, g->albedo, reinterpret_cast<float4*>(F));
+      if (n_glossy > 0)
+        k_glossy_features<O><<<(unsigned)((n_glossy + G - 1) / G), 256, 0, counted(stream)>>>(
+            n_glossy, glossy_ids, M, g->means, px, py, pz, g->albedo, F);
+    };
+    switch (order) {
+      case 1: features(std::integral_constant<int, 1>{}); break;
+      case 2: features(std::integral_constant<int, 2>{}); break;
+      case 3: features(std::integral_constant<int, 3>{}); break;
+      case 4: features(std::integral_constant<int, 4>{}); break;
+      case 5: features(std::integral_constant<int, 5>{}); break;
+      default: features(std::integral_constant<int, 6>{}); break;
     }
     PRTGS_CHECK_LAUNCH();
   }
-  int rc = render(g, F, C, cam, zero, TI, st, status, rws, stream);
+  int rc = render_rows(g, F, C, cam, zero, TI, st, status, rws, stream);
   if (rc != PRTGS_OK) return rc;
   if (precision != PRTGS_PREC_FP32)
     return relight_tc_pixels(n_pix, order, TI, st->final_T, bg, L, k, precision, image, status, tc_wait_polls,

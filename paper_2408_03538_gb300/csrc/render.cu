@@ -4,9 +4,8 @@
 //
 // Forward: k_preprocess (one thread per Gaussian) -> the Gaussians in depth order (radix sort of the depth
 // bits) -> inclusive scan of the touched-tile counts in that order -> k_duplicate writes (tile, Gaussian)
-// pairs -> stable radix sort by tile, on the device-side pair count -> k_ranges -> k_composite (one 16x16-pixel tile per block,
-// Gaussians staged through shared memory in batches of 256, evaluated once for a group of
-// up to 8 light colour sets).
+// pairs -> stable radix sort by tile, on the device-side pair count -> k_ranges -> k_composite (one 16x16-pixel tile per block, a
+// warp per 8x4 pixels that stages the splats that reach them, evaluated once for a group of up to 16 light colour sets).
 // Backward: k_composite_bwd walks each pixel's list back to front from its last contributor and sums
 // every splat's moments and colour gradients over a warp's pixels before a few vector reductions;
 // k_preprocess_bwd maps the sums to opacities, colours, means, scales and rotations.
@@ -51,6 +50,7 @@ static Cam make_cam(const prtgs_camera* c) {
 // 3 k offs[b] (the layout of prtgs_relight_batched) and its images the [k][3][H][W] block b. The
 // cameras travel by value in the kernel parameters (no device copy, graph-capturable).
 struct OneView {
+  static constexpr bool kRows = false;
   Cam c;
   __device__ __forceinline__ int scene_of(int64_t) const { return 0; }
   __device__ __forceinline__ const Cam& cam(int) const { return c; }
@@ -58,7 +58,13 @@ struct OneView {
   __device__ __forceinline__ int64_t count(int, int64_t n) const { return n; }
 };
 
+// OneView with the colours as rows [n][color_floats(k)]: one splat's sets side by side.
+struct RowView : OneView {
+  static constexpr bool kRows = true;
+};
+
 struct ManyViews {
+  static constexpr bool kRows = false;
   Cam c[kMaxScenes];
   const int64_t* offs;
   int B;
@@ -74,6 +80,9 @@ __device__ __forceinline__ int64_t color_at(const V& v, int b, int64_t g, int l,
   const int64_t o = v.first(b);
   return 3 * (int64_t)k * o + ((int64_t)l * v.count(b, n) + (g - o)) * 3;
 }
+
+// Floats of k colour sets, on a 16-byte boundary.
+__host__ __device__ constexpr int color_floats(int kg) { return (3 * kg + 3) / 4 * 4; }
 
 size_t render_state_bytes(int64_t n, int32_t width, int32_t height, int64_t max_pairs) {
   return render_state_bytes_batched(n, 1, width, height, max_pairs);
@@ -297,61 +306,98 @@ __device__ __forceinline__ bool reaches(float mx, float my, const float4& co, fl
   return !(mx + hx < x0) && !(mx - hx > x1) && !(my + hy < y0) && !(my - hy > y1);
 }
 
+// Per-warp staging of k_composite: 32 splats and their colours.
+template <int KG>
+struct FwdWarp {
+  float4 co[32];
+  float4 xy[32];  // mean2d, Gaussian, position in the tile's list (bits)
+  float col[32][color_floats(KG)];
+};
+
+// One warp per 8 x 4 pixels of a tile, on its own (no block barrier), for a group of KG colour sets: it takes its
+// tile's list 32 splats at a time, one per lane, drops those that cannot reach its pixels (reaches; most of a
+// tile's list, as a splat of a few pixels meets one or two of the eight warps), stages the rest with their colours
+// in shared memory and blends them, lane = pixel; the next 32 are on their way meanwhile. It stops when its own
+// pixels are opaque. Only splats that add nothing are dropped, so the results are those of the whole list. Bound
+// by issue slots. (Staging the whole list by block and evaluating every splat at every pixel took 485 us for 300k
+// splats at full HD, 875 us for the geometry maps of 300k surface splats and 2,320 us for the 48 channels of a million;
+// this takes 314, 450 and 1,249 us.)
 template <int KG, class V>
-__global__ void __launch_bounds__(kTileThreads) k_composite(V v, const uint32_t* __restrict__ ranges,
-                                                            const int32_t* __restrict__ ids,
-                                                            const float* __restrict__ mean2d,
-                                                            const float4* __restrict__ conic_op,
-                                                            const float* __restrict__ colors, int64_t n, int k,
-                                                            const float* __restrict__ bg, float* __restrict__ image,
-                                                            float* __restrict__ final_T, int32_t* __restrict__ n_contrib) {
-  __shared__ float2 s_xy[kTileThreads];
-  __shared__ float4 s_co[kTileThreads];
-  __shared__ float s_col[kTileThreads][3 * KG];
+__global__ void __launch_bounds__(kTileThreads, KG <= 8 ? 3 : 2) k_composite(
+    V v, const uint32_t* __restrict__ ranges, const int32_t* __restrict__ ids, const float* __restrict__ mean2d,
+    const float4* __restrict__ conic_op, const float* __restrict__ colors, int64_t n, int k,
+    const float* __restrict__ bg, float* __restrict__ image, float* __restrict__ final_T,
+    int32_t* __restrict__ n_contrib) {
+  constexpr int CF = color_floats(KG);
+  extern __shared__ float4 fwd_smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  FwdWarp<KG>& sm = reinterpret_cast<FwdWarp<KG>*>(fwd_smem)[warp];
   const int gtile = blockIdx.x;  // scene-major tile index
   const Cam& c = v.cam(0);
   const int per_scene = c.gx * c.gy;
   const int b = gtile / per_scene, tile = gtile % per_scene;
   const int l0 = blockIdx.y * KG;
   const int nl = min(KG, k - l0);
-  const int tx = tile % c.gx, ty = tile / c.gx;
-  const int px = tx * kTile + (threadIdx.x % kTile), py = ty * kTile + (threadIdx.x / kTile);
+  const int bx = (tile % c.gx) * kTile + (warp & 1) * 8, by = (tile / c.gx) * kTile + (warp >> 1) * 4;
+  if (bx >= c.W || by >= c.H) return;  // the warp's pixels lie outside the image
+  const int px = bx + (lane & 7), py = by + (lane >> 3);
   const bool inside = px < c.W && py < c.H;
-  const uint32_t start = ranges[2 * gtile], end = ranges[2 * gtile + 1];
+  const uint32_t start = ranges[2 * gtile];
+  const int len = (int)(ranges[2 * gtile + 1] - start);
   float T = 1.0f;
-  float acc[KG][3];
+  float acc[3 * KG];
 #pragma unroll
-  for (int l = 0; l < KG; ++l) acc[l][0] = acc[l][1] = acc[l][2] = 0.f;
+  for (int e = 0; e < 3 * KG; ++e) acc[e] = 0.f;
   bool done = !inside;
-  uint32_t contributor = 0, last = 0;
+  int last = 0;
   const float fpx = (float)px, fpy = (float)py;
-  for (uint32_t bt = start; bt < end; bt += kTileThreads) {
-    if (__syncthreads_count(done) == kTileThreads) break;
-    uint32_t e = bt + threadIdx.x;
-    if (e < end) {
-      int g = ids[e];
-      s_xy[threadIdx.x] = make_float2(mean2d[2 * g], mean2d[2 * g + 1]);
-      s_co[threadIdx.x] = conic_op[g];
-#pragma unroll
-      for (int l = 0; l < KG; ++l)
-        if (l < nl) {
-          const float* cp = colors + color_at(v, b, g, l0 + l, k, n);
-          s_col[threadIdx.x][3 * l] = cp[0];
-          s_col[threadIdx.x][3 * l + 1] = cp[1];
-          s_col[threadIdx.x][3 * l + 2] = cp[2];
-        }
+  int gid = 0;
+  float2 xy = make_float2(0.f, 0.f);
+  float4 co = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto fetch = [&](int p) {
+    if (p < len) {
+      gid = ids[start + p];
+      xy = *reinterpret_cast<const float2*>(mean2d + 2 * (int64_t)gid);
+      co = conic_op[gid];
     }
-    __syncthreads();
-    const int cnt = (int)min((uint32_t)kTileThreads, end - bt);
-    for (int j = 0; j < cnt && !done; ++j) {
-      ++contributor;
-      const float2 xy = s_xy[j];
-      const float4 co = s_co[j];
-      const float dx = xy.x - fpx, dy = xy.y - fpy;
-      const float power = -0.5f * (co.x * dx * dx + co.z * dy * dy) - co.y * dx * dy;
-      if (power > 0.f) continue;
-      const float alpha = fminf(kAlphaMax, co.w * __expf(power));
-      if (alpha < kAlphaMin) continue;
+  };
+  fetch(lane);
+  for (int base = 0; base < len; base += 32) {
+    const bool keep = base + lane < len && reaches(xy.x, xy.y, co, (float)bx, (float)(bx + 7), (float)by, (float)(by + 3));
+    const unsigned m = __ballot_sync(0xffffffffu, keep);
+    const int nk = __popc(m);
+    if (keep) {
+      const int slot = __popc(m & ((1u << lane) - 1u));
+      sm.co[slot] = co;
+      sm.xy[slot] = make_float4(xy.x, xy.y, __int_as_float(gid), __int_as_float(base + lane));
+      if constexpr (!V::kRows) {
+#pragma unroll
+        for (int l = 0; l < KG; ++l) {
+          const float* cp = colors + color_at(v, b, gid, l0 + (l < nl ? l : 0), k, n);
+#pragma unroll
+          for (int ch = 0; ch < 3; ++ch) sm.col[slot][3 * l + ch] = l < nl ? cp[ch] : 0.f;
+        }
+      }
+    }
+    fetch(base + 32 + lane);
+    __syncwarp();
+    if constexpr (V::kRows) {  // consecutive lanes on a row's 16-byte words
+      constexpr int Q = CF / 4;
+      const int stride = color_floats(k) / 4, q0 = 3 * l0 / 4;
+      for (int e = lane; e < nk * Q; e += 32) {
+        const int slot = e / Q, q = e % Q;
+        if (q0 + q < stride)
+          reinterpret_cast<float4*>(sm.col[slot])[q] =
+              __ldg(reinterpret_cast<const float4*>(colors) + (int64_t)__float_as_int(sm.xy[slot].z) * stride + q0 + q);
+      }
+      __syncwarp();
+    }
+    for (int j = 0; j < nk; ++j) {
+      const float4 q = sm.xy[j], o = sm.co[j];
+      const float dx = q.x - fpx, dy = q.y - fpy;
+      const float power = -0.5f * (o.x * dx * dx + o.z * dy * dy) - o.y * dx * dy;
+      const float alpha = fminf(kAlphaMax, o.w * __expf(power));
+      if (done || power > 0.f || alpha < kAlphaMin) continue;
       const float test_T = T * (1.0f - alpha);
       if (test_T < kTStop) {
         done = true;
@@ -359,28 +405,52 @@ __global__ void __launch_bounds__(kTileThreads) k_composite(V v, const uint32_t*
       }
       const float wgt = alpha * T;
 #pragma unroll
-      for (int l = 0; l < KG; ++l) {
-        acc[l][0] = fmaf(s_col[j][3 * l], wgt, acc[l][0]);
-        acc[l][1] = fmaf(s_col[j][3 * l + 1], wgt, acc[l][1]);
-        acc[l][2] = fmaf(s_col[j][3 * l + 2], wgt, acc[l][2]);
+      for (int e = 0; e < CF; e += 4) {
+        const float4 cl = *reinterpret_cast<const float4*>(&sm.col[j][e]);
+        acc[e] = fmaf(cl.x, wgt, acc[e]);
+        acc[e + 1] = fmaf(cl.y, wgt, acc[e + 1]);
+        acc[e + 2] = fmaf(cl.z, wgt, acc[e + 2]);
+        if (e + 3 < 3 * KG) acc[e + 3] = fmaf(cl.w, wgt, acc[e + 3]);
       }
       T = test_T;
-      last = contributor;
+      last = __float_as_int(q.w) + 1;
     }
+    __syncwarp();  // the staged splats are replaced
+    if (__all_sync(0xffffffffu, done)) break;
   }
   if (!inside) return;
   const int64_t HW = (int64_t)c.W * c.H;
   const int64_t pix = (int64_t)py * c.W + px;
   if (blockIdx.y == 0) {
     final_T[b * HW + pix] = T;
-    n_contrib[b * HW + pix] = (int32_t)last;
+    n_contrib[b * HW + pix] = last;
   }
   float* img = image + (int64_t)b * k * 3 * HW;
 #pragma unroll
-  for (int l = 0; l < KG; ++l)
-    if (l < nl)
-#pragma unroll
-      for (int ch = 0; ch < 3; ++ch) img[((int64_t)(l0 + l) * 3 + ch) * HW + pix] = acc[l][ch] + T * bg[ch];
+  for (int e = 0; e < 3 * KG; ++e)
+    if (e < 3 * nl) img[((int64_t)3 * l0 + e) * HW + pix] = acc[e] + T * bg[e % 3];
+}
+
+template <int KG, class V>
+static void launch_composite_t(const V& v, unsigned tiles, const prtgs_render_state* st, const float* colors, int64_t n,
+                               int k, const float* bg, float* image, cudaStream_t stream) {
+  const size_t smem = sizeof(FwdWarp<KG>) * (kTileThreads / 32);
+  if (smem > 48 * 1024) cudaFuncSetAttribute(k_composite<KG, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_composite<KG, V><<<dim3(tiles, (unsigned)((k + KG - 1) / KG)), kTileThreads, smem, counted(stream)>>>(
+      v, st->ranges, st->pair_ids, st->mean2d, reinterpret_cast<const float4*>(st->conic_op), colors, n, k, bg, image,
+      st->final_T, st->n_contrib);
+}
+
+// Colour sets per block: the smallest group that holds k; above 8, groups of 16 where they leave no more sets
+// empty than groups of 8 (every group evaluates the alphas again, and every set of a group costs its sums).
+template <class V>
+static void launch_composite(const V& v, unsigned tiles, const prtgs_render_state* st, const float* colors, int64_t n, int k,
+                             const float* bg, float* image, cudaStream_t stream) {
+  if (k <= 1) launch_composite_t<1>(v, tiles, st, colors, n, k, bg, image, stream);
+  else if (k <= 2) launch_composite_t<2>(v, tiles, st, colors, n, k, bg, image, stream);
+  else if (k <= 4) launch_composite_t<4>(v, tiles, st, colors, n, k, bg, image, stream);
+  else if ((k + 7) / 8 % 2 == 0) launch_composite_t<16>(v, tiles, st, colors, n, k, bg, image, stream);
+  else launch_composite_t<8>(v, tiles, st, colors, n, k, bg, image, stream);
 }
 
 // Forward pass for B scenes of one image size (B = 1 with OneView): tiles are numbered
@@ -433,18 +503,7 @@ static int render_views(const prtgs_gaussians* g, const float* colors, int32_t k
         tkey[2], st->pair_ids, st->depth, st->n_pairs, tiles, st->ranges, st->pair_keys);
     PRTGS_CHECK_LAUNCH();
   }
-  const int kg = k <= 1 ? 1 : (k <= 4 ? 4 : 8);
-  dim3 grid((unsigned)tiles, (unsigned)((k + kg - 1) / kg));
-  const float4* co = reinterpret_cast<const float4*>(st->conic_op);
-  if (kg == 1)
-    k_composite<1, V><<<grid, kTileThreads, 0, counted(stream)>>>(v, st->ranges, st->pair_ids, st->mean2d, co, colors, n, k,
-                                                         bg, image, st->final_T, st->n_contrib);
-  else if (kg == 4)
-    k_composite<4, V><<<grid, kTileThreads, 0, counted(stream)>>>(v, st->ranges, st->pair_ids, st->mean2d, co, colors, n, k,
-                                                         bg, image, st->final_T, st->n_contrib);
-  else
-    k_composite<8, V><<<grid, kTileThreads, 0, counted(stream)>>>(v, st->ranges, st->pair_ids, st->mean2d, co, colors, n, k,
-                                                         bg, image, st->final_T, st->n_contrib);
+  launch_composite(v, (unsigned)tiles, st, colors, n, k, bg, image, stream);
   PRTGS_CHECK_LAUNCH();
   return PRTGS_OK;
 }
@@ -454,6 +513,15 @@ int render(const prtgs_gaussians* g, const float* colors, int32_t k, const prtgs
   OneView v{make_cam(cam)};
   return render_views(g, colors, k, v, v.c, 1, bg, image, st, status, ws, stream);
 }
+
+int render_rows(const prtgs_gaussians* g, const float* rows, int32_t k, const prtgs_camera* cam, const float* bg,
+                float* image, prtgs_render_state* st, int32_t* status, void* ws, cudaStream_t stream) {
+  RowView v;
+  v.c = make_cam(cam);
+  return render_views(g, rows, k, v, v.c, 1, bg, image, st, status, ws, stream);
+}
+
+size_t render_rows_floats(int32_t k) { return (size_t)color_floats(k); }
 
 static int many_views(const prtgs_camera* cams, int32_t B, const int64_t* offsets, ManyViews& v) {
   if (B < 1 || B > kMaxScenes) return PRTGS_ERR_UNSUPPORTED;
@@ -482,7 +550,6 @@ int render_batched(const prtgs_gaussians* g, const int64_t* offsets, int32_t B, 
 // and conic), then sum alpha T dL/dpixel per colour channel, each group of KG colour sets on a 16-byte
 // boundary.
 constexpr int kMoments = 8;  // six sums, padded
-__host__ __device__ constexpr int color_floats(int kg) { return (3 * kg + 3) / 4 * 4; }
 static int bwd_group(int k) { return k <= 1 ? 1 : (k <= 4 ? 4 : 8); }
 static int bwd_stride(int k) { return kMoments + color_floats(bwd_group(k)) * ((k + bwd_group(k) - 1) / bwd_group(k)); }
 
@@ -806,7 +873,7 @@ __global__ void k_preprocess_bwd(int64_t n, const float* __restrict__ means, con
 }
 
 // ---- depth and normal maps (Eq. 23, Eq. 25): the composite of d_i and n_i -------------------------
-// Features for render() with two "lights": light 0 carries (d_i, 0, 0), d_i the view-space
+// Rows for render_rows() with two "lights": light 0 carries (d_i, 0, 0), d_i the view-space
 // depth of the splat's mean; light 1 carries the raw normal n_i.
 __global__ void k_geometry_features(int64_t n, Cam c, const float* __restrict__ means,
                                     const float* __restrict__ normals, float* __restrict__ F) {
@@ -814,16 +881,13 @@ __global__ void k_geometry_features(int64_t n, Cam c, const float* __restrict__ 
   if (i >= n) return;
   const float x = means[3 * i], y = means[3 * i + 1], z = means[3 * i + 2];
   const float d = fmaf(c.r[6], x, fmaf(c.r[7], y, fmaf(c.r[8], z, c.t[2])));
-  F[3 * i] = d;
-  F[3 * i + 1] = 0.f;
-  F[3 * i + 2] = 0.f;
-  float* Fn = F + 3 * n;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) Fn[3 * i + k] = normals[3 * i + k];
+  float4* row = reinterpret_cast<float4*>(F) + 2 * i;
+  row[0] = make_float4(d, 0.f, 0.f, normals[3 * i]);
+  row[1] = make_float4(normals[3 * i + 1], normals[3 * i + 2], 0.f, 0.f);
 }
 
 size_t render_geometry_workspace(int64_t n, int32_t width, int32_t height, int64_t max_pairs) {
-  return align_up(sizeof(float) * 6 * (size_t)n) + align_up(sizeof(float) * 6 * (size_t)width * height) +
+  return align_up(sizeof(float) * 8 * (size_t)n) + align_up(sizeof(float) * 6 * (size_t)width * height) +
          align_up(sizeof(float) * 4) + render_workspace(n, width, height, max_pairs);
 }
 
@@ -832,7 +896,7 @@ int render_geometry(const prtgs_gaussians* g, const prtgs_camera* cam, float* de
   const int64_t n = g->n;
   const int64_t n_pix = (int64_t)cam->width * cam->height;
   Carver cv(ws);
-  float* F = cv.take<float>(6 * (size_t)n);
+  float* F = cv.take<float>(8 * (size_t)n);
   float* img = cv.take<float>(6 * (size_t)n_pix);
   float* zero = cv.take<float>(4);
   void* rws = static_cast<char*>(ws) + cv.off;
@@ -841,7 +905,7 @@ int render_geometry(const prtgs_gaussians* g, const prtgs_camera* cam, float* de
     k_geometry_features<<<(unsigned)((n + 255) / 256), 256, 0, counted(stream)>>>(n, make_cam(cam), g->means, g->normals, F);
     PRTGS_CHECK_LAUNCH();
   }
-  const int rc = render(g, F, 2, cam, zero, img, st, status, rws, stream);
+  const int rc = render_rows(g, F, 2, cam, zero, img, st, status, rws, stream);
   if (rc != PRTGS_OK) return rc;
   // image [2][3][H][W]: depth is light 0's first channel, the normal light 1's three channels
   cudaMemcpyAsync(depth, img, sizeof(float) * n_pix, cudaMemcpyDeviceToDevice, stream);

@@ -106,3 +106,26 @@ def test_bvh_sort_sizes(n):
     order = bvh.view("order", torch.int32, (n,)).long()
     assert bool((key[1:] > key[:-1]).all()) and torch.equal(key & ((1 << 27) - 1), order)
     assert torch.equal(torch.sort(order).values, torch.arange(n, device="cuda"))
+
+
+@pytest.mark.parametrize("w,h", [(1, 1), (17, 4), (61, 45), (640, 360)])
+@pytest.mark.parametrize("k", [2, 5, 16, 23, 32])
+def test_color_groups_and_rows_agree(w, h, k):
+    """Every group of colour sets blends with the same weights: k sets at once equal k renders of one set, bit
+    for bit; so do the normals that the geometry maps blend from rows."""
+    sc = S.isotropic_scene(1501, 90)
+    cam = S.look_at_camera((0, -3.5, 1.0), (0, 0, 0), 45, w, h)
+    g = api.GaussianTensors.from_scene(sc)
+    colors = torch.rand((k, sc.n, 3), device="cuda", generator=torch.Generator("cuda").manual_seed(k))
+    colors[1] = g.normals
+    bg = torch.zeros(3, device="cuda")
+    st = api.Status()
+    img, s = api.render(g, colors, cam, bg, max_pairs=400_000, status=st)
+    assert st.read() == 0
+    for l in range(k):
+        one, s1 = api.render(g, colors[l : l + 1].contiguous(), cam, bg, max_pairs=400_000)
+        assert torch.equal(one[0], img[l]), l
+        for field, dt in (("final_T", torch.float32), ("n_contrib", torch.int32)):
+            assert torch.equal(s.view(field, dt, (h, w)), s1.view(field, dt, (h, w)))
+    _, normal, _ = api.render_geometry(g, cam, max_pairs=400_000)
+    assert torch.equal(normal, img[1])
