@@ -57,6 +57,10 @@ constexpr int kPHeadroom = 64 + 64 + 4;
 // windows and share the BVH nodes around them in L1/L2 (surface-100k visibility 47 ms against 72
 // at 16 directions; the 1M tiled transfer 1.69 s against 1.97 s)
 constexpr int kPacketDirs = 1;
+// Receivers of a backward window (64 to 256): the wider, the fewer packets are left with a few lanes (isotropic
+// normals: half of a window faces a direction). 100k volume at 128 directions: 83.5 ms at 64, 78.7 at 128, 76.4 at 256.
+// The forward keeps 64: its hit decisions depend on a packet's reference point to the last bit.
+constexpr int kBwdWindow = 256;
 
 struct PacketSmem {
   int stack[kPStack];
@@ -65,7 +69,7 @@ struct PacketSmem {
                            // lanes of a drain read different leaves: 16-byte stride, few bank conflicts)
   float4 quick[2][32];     // ... and the terms of the quick test
   // the window slots of the receivers that face the direction
-  unsigned char rlist[64];
+  unsigned char rlist[kBwdWindow];
 };
 
 // k_search, per warp after the PacketSmem array: the search round's nearest hits of each lane,
@@ -722,10 +726,13 @@ __global__ void __launch_bounds__(kPacketThreads, BOUNCE ? PRTGS_PACKET_BOUNCE_M
     __syncwarp();
     const unsigned item = s_item[warp];
     __syncwarp();
-    if ((int64_t)item >= n_windows * dblocks) break;
-    // a window of 64 receivers adjacent in Morton order; each lane stages two of them
-    const int64_t base = a.r0 + 64 * (item / dblocks);
-    const int s0 = (int)(item % dblocks) * dpi;
+    if ((int64_t)item >= 2 * n_windows * dblocks) break;
+    // a window of 64 receivers adjacent in Morton order, in up to two packets of 32 lanes, an item each (one
+    // after the other in one item, 1,024 splats at 64 directions took 143 us, now 114: few items, long walks);
+    // each lane stages two of them
+    const int pass = (int)(item & 1u);
+    const int64_t base = a.r0 + 64 * ((item >> 1) / dblocks);
+    const int s0 = (int)((item >> 1) % dblocks) * dpi;
     float4 nq[2];  // record row 3 of the lane's two receivers (its .yzw: the normal)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -743,17 +750,17 @@ __global__ void __launch_bounds__(kPacketThreads, BOUNCE ? PRTGS_PACKET_BOUNCE_M
         const int j = lane + 32 * h;
         const bool vj = base + j < a.r1;
         upj[h] = vj && ray_cos(nq[h].y, nq[h].z, nq[h].w, d) > 0.0f;
-        if (vj && !upj[h]) {  // untraced ray: no visibility, no index-matrix entry
+        if (vj && !upj[h] && pass == 0) {  // untraced ray: no visibility, no index-matrix entry
           V[(int64_t)s * batch + (base + j - a.r0)] = 0.0f;
           if (BOUNCE) a.idx[(int64_t)__ldg(a.order + base + j) * a.S + s] = -1;
         }
       }
       const unsigned m0 = __ballot_sync(0xffffffffu, upj[0]), m1 = __ballot_sync(0xffffffffu, upj[1]);
       const int total = __popc(m0) + __popc(m1);
+      if (pass * 32 >= total) continue;
       if (upj[0]) sm.rlist[__popc(m0 & below)] = (unsigned char)lane;
       if (upj[1]) sm.rlist[__popc(m0) + __popc(m1 & below)] = (unsigned char)(lane + 32);
       __syncwarp();
-      for (int pass = 0; pass * 32 < total; ++pass) {
       const bool up = pass * 32 + lane < total;
       const int jw = up ? sm.rlist[pass * 32 + lane] : 0;
       const int self = (int)(base + jw);
@@ -819,8 +826,6 @@ __global__ void __launch_bounds__(kPacketThreads, BOUNCE ? PRTGS_PACKET_BOUNCE_M
         if (lane == 0) a.pending[e] = (uint32_t)s;
         static_cast<SearchRec*>(a.queue)[(int64_t)e * 32 + lane] = rec;
       }
-      __syncwarp();
-      }  // pass
       __syncwarp();  // the compacted list is rewritten for the next direction
     }
     __syncwarp();  // the window is restaged by the next work item
@@ -842,7 +847,7 @@ __global__ void __launch_bounds__(kPacketThreads, BOUNCE ? PRTGS_PACKET_BOUNCE_M
   }
 }
 
-// The index-matrix search of the packets that k_packet<true> left: one warp per item, rounds of 14 hits
+// The index-matrix search of the packets that k_packet<true> left: one warp per item, rounds of kPacketRoundHits hits
 // in key order until every ray's argmax is settled. A kernel of its own: only a third of the packets
 // get here, and beside the visibility walk's code and registers both ran slower.
 #ifndef PRTGS_SEARCH_MIN_BLOCKS
@@ -956,7 +961,7 @@ __global__ void __launch_bounds__(kPacketThreads, PRTGS_SEARCH_MIN_BLOCKS) k_sea
 // shared memory, and one lane per leaf turns them into the ten sums and adds them with three vector
 // reductions. k_bwd_finish forms the gradients, once per Gaussian.
 // Walking each ray alone and twice, with twelve atomics per hit, took 843 ms for a 100k volume at 128
-// directions and 147 ms for 40k surface splats at 256; this takes 80 and 14 ms, bound by issue slots.
+// directions and 147 ms for 40k surface splats at 256; this takes 77 and 14 ms, bound by issue slots.
 // Hits are decided as by the ray's own test (ray_decides, a tenth of that time): on a surface, splats in
 // the receiver's own plane have t* = 0 up to rounding and a large alpha.
 
@@ -1010,31 +1015,32 @@ __global__ void __launch_bounds__(kPacketThreads, kBwdBlocks)
   BwdSmem& bs = reinterpret_cast<BwdSmem*>(wsm + kPacketWarps)[warp];
   int* list = lists + ((int64_t)blockIdx.x * kPacketWarps + warp) * kBwdList;
   const int64_t batch = a.r1 - a.r0;
-  const int64_t n_windows = (batch + 63) / 64;
+  constexpr int kPasses = kBwdWindow / 32;
+  const int64_t n_windows = (batch + kBwdWindow - 1) / kBwdWindow;
   const unsigned below = (1u << lane) - 1u;
   RayStats rs{0u, 0u, 0u, 0u, 0u, 0u};
   for (;;) {
     unsigned item = 0;
     if (lane == 0) item = atomicAdd(a.work, 1u);
     item = __shfl_sync(0xffffffffu, item, 0);
-    if ((int64_t)item >= n_windows * a.S) break;
-    const int64_t base = a.r0 + 64 * (item / a.S);
-    const int s = (int)(item % a.S);
-    const float d[3] = {__ldg(a.dirs + 3 * s), __ldg(a.dirs + 3 * s + 1), __ldg(a.dirs + 3 * s + 2)};
-    const Frame f = make_frame(d[0], d[1], d[2]);
-    bool upj[2];  // k_ray_grad left zeros for the directions below a receiver's horizon
+    if ((int64_t)item >= kPasses * n_windows * a.S) break;
+    const int pass = (int)(item % kPasses);
+    const int64_t base = a.r0 + kBwdWindow * (item / kPasses / a.S);
+    const int s = (int)(item / kPasses % a.S);
+    int total = 0;  // k_ray_grad left zeros for the directions below a receiver's horizon
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < kPasses; ++h) {
       const int64_t j = base + lane + 32 * h;
       const int64_t o = (int64_t)s * batch + (j - a.r0);
-      upj[h] = j < a.r1 && (G[o] != 0.0f || GV[o] != 0.0f);
+      const bool on = j < a.r1 && (G[o] != 0.0f || GV[o] != 0.0f);
+      const unsigned m = __ballot_sync(0xffffffffu, on);
+      if (on) sm.rlist[total + __popc(m & below)] = (unsigned char)(lane + 32 * h);
+      total += __popc(m);
     }
-    const unsigned m0 = __ballot_sync(0xffffffffu, upj[0]), m1 = __ballot_sync(0xffffffffu, upj[1]);
-    const int total = __popc(m0) + __popc(m1);
-    if (upj[0]) sm.rlist[__popc(m0 & below)] = (unsigned char)lane;
-    if (upj[1]) sm.rlist[__popc(m0) + __popc(m1 & below)] = (unsigned char)(lane + 32);
     __syncwarp();
-    for (int pass = 0; pass * 32 < total; ++pass) {
+    if (pass * 32 < total) {
+      const float d[3] = {__ldg(a.dirs + 3 * s), __ldg(a.dirs + 3 * s + 1), __ldg(a.dirs + 3 * s + 2)};
+      const Frame f = make_frame(d[0], d[1], d[2]);
       const bool up = pass * 32 + lane < total;
       const int self = (int)(base + (up ? sm.rlist[pass * 32 + lane] : 0));
       const float4 q0 = __ldg(a.recs + 4 * (int64_t)self);

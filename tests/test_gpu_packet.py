@@ -111,3 +111,15 @@ def test_packet_backward_list_overflow():
     sc.means *= 0.02
     sc.opacity *= np.float32(0.02)
     _grads_against_autograd([sc], S.direction_set(5, 9), 1, 0.0)
+
+
+@pytest.mark.parametrize("sizes", [[255], [256], [600], [200, 100, 213]])
+def test_packet_backward_wide_windows(sizes):
+    """Backward windows that are full, one short and in part; normals at random, so that a packet's rays come from
+    all over its window."""
+    parts = [S.isotropic_scene(n, 700 + n) for n in sizes]
+    for p in parts:
+        p.scales *= np.float32(1.5)
+        p.scales[:, 0] *= np.float32(0.7)
+        p.scales[:, 1] *= np.float32(1.2)
+    _grads_against_autograd(parts, S.direction_set(31, 10), 2, 0.0)
