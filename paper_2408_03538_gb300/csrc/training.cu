@@ -77,19 +77,25 @@ __device__ __forceinline__ float reduce_scatter(float* v, int lane, int& k) {
   return x;
 }
 
+// Row of the SH table in shared memory: whole 16-byte words, an odd number of them, so that lanes on
+// neighbouring directions read them without bank conflicts.
+constexpr int tt_row(int C) { return ((C + 3) / 4 | 1) * 4; }
+
+// Bound by issue slots (the BRDF) and the latency of V: a row's chunks are loaded four ahead, and a term reads its
+// SH row in 16-byte words. 300k receivers, order 3, 256 directions: 380 us a chunk at a time and a word per
+// coefficient, 363 us like this; the backward 397 and 371 us.
 template <int ORDER, bool BACKWARD>
 __global__ void __launch_bounds__(kTTThreads, ORDER <= 3 ? 4 : 2) k_training_transfer(TTArgs a) {
-  constexpr int C = (ORDER + 1) * (ORDER + 1);
-  extern __shared__ float sm[];
+  constexpr int C = (ORDER + 1) * (ORDER + 1), R = tt_row(C);
+  extern __shared__ float4 tt_smem[];
   const int S = a.S;
-  float* sdir = sm;              // [3S]
-  float* sY = sdir + 3 * S;      // [C][S]: coefficient-major, so that the lanes (consecutive
-                                 // directions) read consecutive words, free of bank conflicts
-  float* sdt = sY + S * C;       // [warps][C] (backward)
+  float* sY = reinterpret_cast<float*>(tt_smem);  // [S][R]
+  float* sdt = sY + S * R;                        // [warps][R] (backward)
+  float* sdir = sdt + (BACKWARD ? kTTWarps * R : 0);  // [3S]
   __shared__ int qs_all[kTTWarps][kTTQueue];    // queued direction
   __shared__ float qw_all[kTTWarps][kTTQueue];  // its (n.w_s) V_s
   for (int i = threadIdx.x; i < 3 * S; i += blockDim.x) sdir[i] = a.dirs[i];
-  for (int i = threadIdx.x; i < S * C; i += blockDim.x) sY[i] = a.Ytab[(i % S) * C + i / S];
+  for (int i = threadIdx.x; i < S * C; i += blockDim.x) sY[i / C * R + i % C] = a.Ytab[i];
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned lt_mask = (1u << lane) - 1u;
@@ -113,7 +119,7 @@ __global__ void __launch_bounds__(kTTThreads, ORDER <= 3 ? 4 : 2) k_training_tra
 #pragma unroll
     for (int k = 0; k < (BACKWARD ? 1 : C); ++k) acc[k] = 0.0f;
     float gr = 0.0f, gm = 0.0f;
-    float* dts = sdt + warp * C;
+    float* dts = sdt + warp * R;
     if (BACKWARD) {
       for (int k = lane; k < C; k += 32) dts[k] = __ldg(a.dt + i * C + k);
       __syncwarp();
@@ -121,15 +127,27 @@ __global__ void __launch_bounds__(kTTThreads, ORDER <= 3 ? 4 : 2) k_training_tra
     // one live term (direction s, cv = (n.w_s) V_s) on this lane
     auto term = [&](int s, float cv) {
       const float* d = sdir + 3 * s;
-      if (!BACKWARD) {
+      if constexpr (!BACKWARD) {
         const float c = fmaf(nx, d[0], fmaf(ny, d[1], nz * d[2]));  // > 0 for a queued term
         const float f = wq * brdf_kernel(nx, ny, nz, d, v, c, no, alpha, m) * cv;
 #pragma unroll
-        for (int k = 0; k < (BACKWARD ? 1 : C); ++k) acc[k] = fmaf(f, sY[k * S + s], acc[k]);
+        for (int k = 0; k < (BACKWARD ? 1 : C); k += 4) {
+          const float4 y = *reinterpret_cast<const float4*>(sY + s * R + k);
+          acc[k] = fmaf(f, y.x, acc[k]);
+          if (k + 1 < C) acc[k + 1] = fmaf(f, y.y, acc[k + 1]);
+          if (k + 2 < C) acc[k + 2] = fmaf(f, y.z, acc[k + 2]);
+          if (k + 3 < C) acc[k + 3] = fmaf(f, y.w, acc[k + 3]);
+        }
       } else {
         float q = 0.0f;
 #pragma unroll
-        for (int k = 0; k < C; ++k) q = fmaf(dts[k], sY[k * S + s], q);
+        for (int k = 0; k < C; k += 4) {
+          const float4 y = *reinterpret_cast<const float4*>(sY + s * R + k), t = *reinterpret_cast<const float4*>(dts + k);
+          q = fmaf(t.x, y.x, q);
+          if (k + 1 < C) q = fmaf(t.y, y.y, q);
+          if (k + 2 < C) q = fmaf(t.z, y.z, q);
+          if (k + 3 < C) q = fmaf(t.w, y.w, q);
+        }
         float kv;
         const float dk = brdf_kernel_dr(nx, ny, nz, d, v, fmaf(nx, d[0], fmaf(ny, d[1], nz * d[2])), no, r, m, kv);
         const float f = wq * cv * q;
@@ -139,13 +157,21 @@ __global__ void __launch_bounds__(kTTThreads, ORDER <= 3 ? 4 : 2) k_training_tra
     };
     if (front) {
       int qn = 0;  // warp-uniform queue length, < 32 between chunks
+      float ahead[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) ahead[j] = lane + 32 * j < S ? __ldg(Vi + lane + 32 * j) : 0.0f;
       for (int base = 0; base < S; base += 32) {
         const int s = base + lane;
+        const float vs = ahead[0];
+        ahead[0] = ahead[1];
+        ahead[1] = ahead[2];
+        ahead[2] = ahead[3];
+        ahead[3] = s + 128 < S ? __ldg(Vi + s + 128) : 0.0f;
         float cv = 0.0f;
         if (s < S) {
           const float* d = sdir + 3 * s;
           const float c = fmaf(nx, d[0], fmaf(ny, d[1], nz * d[2]));
-          if (c > 0.0f) cv = c * __ldg(Vi + s);
+          if (c > 0.0f) cv = c * vs;
         }
         const bool live = cv != 0.0f;  // a NaN visibility stays live and reaches the output
         const unsigned mask = __ballot_sync(0xffffffffu, live);
@@ -210,8 +236,8 @@ __global__ void __launch_bounds__(kTTThreads, ORDER <= 3 ? 4 : 2) k_training_tra
 
 template <int ORDER, bool BACKWARD>
 static int launch_tt(const TTArgs& a, cudaStream_t stream) {
-  constexpr int C = (ORDER + 1) * (ORDER + 1);
-  const size_t smem = sizeof(float) * (3 * (size_t)a.S + (size_t)a.S * C + (BACKWARD ? kTTWarps * C : 0));
+  constexpr int R = tt_row((ORDER + 1) * (ORDER + 1));
+  const size_t smem = sizeof(float) * (3 * (size_t)a.S + (size_t)a.S * R + (BACKWARD ? kTTWarps * R : 0));
   cudaFuncSetAttribute(k_training_transfer<ORDER, BACKWARD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int per_sm = 0, dev = 0, sms = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_training_transfer<ORDER, BACKWARD>, kTTThreads, smem);
@@ -360,10 +386,19 @@ __global__ void __launch_bounds__(kNLThreads) k_nl_partial(int64_t hw, const flo
   }
 }
 
-__global__ void k_nl_finish(int nb, const double* __restrict__ part, float* __restrict__ loss) {
+// The block sums by one block, in a fixed order (a single thread's chain of up to 1,024 loads took 51 us).
+__global__ void __launch_bounds__(kNLThreads) k_nl_finish(int nb, const double* __restrict__ part, float* __restrict__ loss) {
+  __shared__ double sw[kNLThreads / 32];
+  double v = 0.0;
+#pragma unroll 4
+  for (int b = threadIdx.x; b < nb; b += kNLThreads) v += part[b];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = v;
+  __syncthreads();
   if (threadIdx.x != 0) return;
   double s = 0.0;
-  for (int b = 0; b < nb; ++b) s += part[b];
+  for (int w = 0; w < kNLThreads / 32; ++w) s += sw[w];
   loss[0] = (float)sqrt(s);
 }
 
@@ -388,7 +423,7 @@ int normal_loss(int32_t width, int32_t height, const float* normal, const float*
   const int nb = nl_blocks(hw);
   double* part = static_cast<double*>(ws);
   k_nl_partial<<<nb, kNLThreads, 0, counted(stream)>>>(hw, normal, pseudo, part);
-  k_nl_finish<<<1, 32, 0, counted(stream)>>>(nb, part, loss);
+  k_nl_finish<<<1, kNLThreads, 0, counted(stream)>>>(nb, part, loss);
   if (d_normal && hw > 0)
     k_nl_grad<<<(unsigned)((hw + 255) / 256), 256, 0, counted(stream)>>>(hw, normal, pseudo, loss, d_normal);
   PRTGS_CHECK_LAUNCH();

@@ -24,39 +24,40 @@ namespace prtgs {
 // Q_l^m = P_l^m / sin^m (Condon-Shortley phase) from Q_m^m = (-1)^m (2m-1)!!,
 // Q_{m+1}^m = (2m+1) z Q_m^m, (l-m) Q_l^m = (2l-1) z Q_{l-1}^m - (l+m-1) Q_{l-2}^m, and
 // K_lm = sqrt((2l+1)/(4 pi) (l-m)!/(l+m)!), index l*l+l+m as for orders <= 3.
+// One thread per (direction, m): the FP64 divisions and square roots are chains of their own (a thread per direction
+// took 20 us at 256 directions and order 3).
 __global__ void k_sh_table(int S, int order, const float* __restrict__ dirs, float* __restrict__ Y) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
+  const int s = blockIdx.x * blockDim.x + threadIdx.x, m = blockIdx.y;
   if (s >= S) return;
   const double x = dirs[3 * s], y = dirs[3 * s + 1], z = dirs[3 * s + 2];
   const int C = (order + 1) * (order + 1);
   double re = 1.0, im = 0.0;  // (x + i y)^m
   double qmm = 1.0;           // Q_m^m
-  for (int m = 0; m <= order; ++m) {
-    if (m > 0) {
-      const double r2 = re * x - im * y, i2 = re * y + im * x;
-      re = r2;
-      im = i2;
-      qmm *= -(2.0 * m - 1.0);
+  double fall = 1.0;          // (l + m)! / (l - m)!
+  for (int j = 1; j <= m; ++j) {
+    const double r2 = re * x - im * y, i2 = re * y + im * x;
+    re = r2;
+    im = i2;
+    qmm *= -(2.0 * j - 1.0);
+    fall *= (double)((2 * j - 1) * (2 * j));
+  }
+  double q2 = 0.0, q1 = qmm;  // Q_{l-2}^m, Q_{l-1}^m walking up in l
+  for (int l = m; l <= order; ++l) {
+    double q;
+    if (l == m) q = qmm;
+    else if (l == m + 1) q = (2.0 * m + 1.0) * z * qmm;
+    else q = ((2.0 * l - 1.0) * z * q1 - (double)(l + m - 1) * q2) / (double)(l - m);
+    if (l > m) {
+      q2 = q1;
+      q1 = q;
+      fall = fall * (double)(l + m) / (double)(l - m);  // whole numbers: exact
     }
-    double q2 = 0.0, q1 = qmm;  // Q_{l-2}^m, Q_{l-1}^m walking up in l
-    for (int l = m; l <= order; ++l) {
-      double q;
-      if (l == m) q = qmm;
-      else if (l == m + 1) q = (2.0 * m + 1.0) * z * qmm;
-      else q = ((2.0 * l - 1.0) * z * q1 - (double)(l + m - 1) * q2) / (double)(l - m);
-      if (l > m) {
-        q2 = q1;
-        q1 = q;
-      }
-      double ratio = 1.0;  // (l-m)! / (l+m)!
-      for (int j = l - m + 1; j <= l + m; ++j) ratio /= (double)j;
-      const double K = sqrt((2.0 * l + 1.0) / (4.0 * 3.14159265358979323846) * ratio);
-      if (m == 0) {
-        Y[(int64_t)s * C + l * l + l] = (float)(K * q);
-      } else {
-        Y[(int64_t)s * C + l * l + l + m] = (float)(1.4142135623730951 * K * q * re);
-        Y[(int64_t)s * C + l * l + l - m] = (float)(1.4142135623730951 * K * q * im);
-      }
+    const double K = sqrt((2.0 * l + 1.0) / (4.0 * 3.14159265358979323846 * fall));
+    if (m == 0) {
+      Y[(int64_t)s * C + l * l + l] = (float)(K * q);
+    } else {
+      Y[(int64_t)s * C + l * l + l + m] = (float)(1.4142135623730951 * K * q * re);
+      Y[(int64_t)s * C + l * l + l - m] = (float)(1.4142135623730951 * K * q * im);
     }
   }
 }
@@ -937,7 +938,7 @@ int precompute_transfer(const prtgs_gaussians* g, const prtgs_bvh* bvh, const pr
   a.sh_order = p->sh_order;
   a.Ytab = ytab;
   if (ytab) {
-    k_sh_table<<<(unsigned)((S + 127) / 128), 128, 0, counted(stream)>>>(S, p->sh_order, p->dirs, ytab);
+    k_sh_table<<<dim3((unsigned)((S + 63) / 64), (unsigned)p->sh_order + 1), 64, 0, counted(stream)>>>(S, p->sh_order, p->dirs, ytab);
     PRTGS_CHECK_LAUNCH();
   }
   a.t_min = p->t_min;
@@ -1101,7 +1102,7 @@ int glossy_backward(const prtgs_gaussians* g, const prtgs_transfer_params* p, co
 
 int sh_table(int S, int order, const float* dirs, float* Y, cudaStream_t stream) {
   if (S <= 0) return PRTGS_OK;
-  k_sh_table<<<(unsigned)((S + 127) / 128), 128, 0, counted(stream)>>>(S, order, dirs, Y);
+  k_sh_table<<<dim3((unsigned)((S + 63) / 64), (unsigned)order + 1), 64, 0, counted(stream)>>>(S, order, dirs, Y);
   PRTGS_CHECK_LAUNCH();
   return PRTGS_OK;
 }
