@@ -15,13 +15,14 @@ int scan_u32(const uint32_t* in, uint32_t* out, int64_t n, bool exclusive, uint3
              cudaStream_t stream, const int32_t* idx = nullptr, uint32_t cap = 0xffffffffu);
 size_t radix_sort_workspace(int64_t capacity);
 // Stable; the pairs (keys_x, vals_x; vals_x null: the index) end in (keys_f, vals_f), with (keys_y, vals_y)
-// as the other side of the passes.
+// as the other side of the passes. With wide the sorted keys end there instead of in keys_f, as
+// key << 32 | the bits of low[value].
 int radix_sort_pairs(const uint64_t* keys_x, const int32_t* vals_x, uint64_t* keys_f, int32_t* vals_f,
                      uint64_t* keys_y, int32_t* vals_y, int64_t capacity, const uint32_t* d_count, int begin_bit,
                      int end_bit, void* ws, cudaStream_t stream);
 int radix_sort_pairs(const uint32_t* keys_x, const int32_t* vals_x, uint32_t* keys_f, int32_t* vals_f,
                      uint32_t* keys_y, int32_t* vals_y, int64_t capacity, const uint32_t* d_count, int begin_bit,
-                     int end_bit, void* ws, cudaStream_t stream);
+                     int end_bit, void* ws, cudaStream_t stream, const float* low = nullptr, uint64_t* wide = nullptr);
 
 // bvh.cu
 size_t bvh_bytes(int64_t n, int32_t n_scenes);

@@ -277,18 +277,32 @@ __global__ void __launch_bounds__(256) k_duplicate(int64_t n, V v, const int32_t
   }
 }
 
-// Tile ranges of the sorted pairs, and the pairs' (tile << 32 | depth bits).
-__global__ void k_ranges(const uint32_t* __restrict__ tile_of, const int32_t* __restrict__ ids,
-                         const float* __restrict__ depth, const uint32_t* __restrict__ count, int64_t tiles,
-                         uint32_t* __restrict__ ranges, uint64_t* __restrict__ keys) {
-  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// First of the n sorted pairs whose tile is at least `tile`, by a warp: each round cuts the range into 32.
+__device__ __forceinline__ int64_t first_pair(const uint64_t* __restrict__ keys, int64_t n, uint64_t tile) {
+  const int lane = threadIdx.x & 31;
+  int64_t lo = 0, hi = n;
+  while (lo < hi) {
+    const int64_t step = (hi - lo + 31) / 32, at = lo + lane * step;
+    const bool below = at < hi && (__ldg(keys + min(at + step, hi) - 1) >> 32) < tile;  // the whole part lies in front
+    lo = min(hi, lo + __popc(__ballot_sync(0xffffffffu, below)) * step);
+    hi = min(hi, lo + step - 1);
+  }
+  return lo;
+}
+
+// Tile ranges of the sorted pairs, a warp per tile (empty tiles: 0, 0). A pass over all pairs that compared
+// neighbours and wrote their 64-bit keys took 165 us for 25 M pairs; the sort's last pass writes those now.
+__global__ void __launch_bounds__(256) k_ranges(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ count,
+                                                int64_t tiles, uint32_t* __restrict__ ranges) {
+  const int64_t tile = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (tile >= tiles) return;
   const int64_t n = *count;
-  if (p >= n) return;
-  const uint32_t tile = tile_of[p];
-  keys[p] = ((uint64_t)tile << 32) | __float_as_uint(depth[ids[p]]);
-  if ((int64_t)tile >= tiles) return;
-  if (p == 0 || tile_of[p - 1] != tile) ranges[2 * tile] = (uint32_t)p;
-  if (p == n - 1 || tile_of[p + 1] != tile) ranges[2 * tile + 1] = (uint32_t)(p + 1);
+  const int64_t lo = first_pair(keys, n, (uint64_t)tile);
+  const int64_t hi = first_pair(keys, n, (uint64_t)tile + 1);
+  if ((threadIdx.x & 31) == 0) {
+    ranges[2 * tile] = lo < hi ? (uint32_t)lo : 0u;
+    ranges[2 * tile + 1] = lo < hi ? (uint32_t)hi : 0u;
+  }
 }
 
 // Whether a splat can have alpha >= 1/255 at any pixel centre of [x0, x1] x [y0, y1]: the smallest value of its
@@ -480,9 +494,11 @@ static int render_views(const prtgs_gaussians* g, const float* colors, int32_t k
   int32_t* ids_x = cv.take<int32_t>(st->max_pairs);
   int32_t* ids_y = cv.take<int32_t>(st->max_pairs);
   void* sort_ws = cv.take<char>(radix_sort_workspace(st->max_pairs > n ? st->max_pairs : n));
-  cudaMemsetAsync(st->ranges, 0, sizeof(uint32_t) * 2 * tiles, stream);
-  if (n == 0) cudaMemsetAsync(st->n_pairs, 0, sizeof(uint32_t), stream);
-  if (n > 0) {
+  if (n == 0) {
+    cudaMemsetAsync(st->ranges, 0, sizeof(uint32_t) * 2 * tiles, stream);
+    cudaMemsetAsync(st->n_pairs, 0, sizeof(uint32_t), stream);
+  } else {
+    if (st->max_pairs <= 0) return PRTGS_ERR_CUDA;  // no room for any pair: nothing to launch the sort on
     const unsigned blocks = (unsigned)((n + 255) / 256);
     k_preprocess<V><<<blocks, 256, 0, counted(stream)>>>(
         n, g->means, g->scales, g->quats, g->opacity, v, st->mean2d, reinterpret_cast<float4*>(st->conic_op),
@@ -504,10 +520,9 @@ static int render_views(const prtgs_gaussians* g, const float* colors, int32_t k
     int tile_bits = 0;
     while ((int64_t(1) << tile_bits) < tiles) ++tile_bits;
     rc = radix_sort_pairs(tkey[0], ids_x, tkey[2], st->pair_ids, tkey[1], ids_y, st->max_pairs, st->n_pairs, 0, tile_bits,
-                          sort_ws, stream);
+                          sort_ws, stream, st->depth, st->pair_keys);
     if (rc != PRTGS_OK) return rc;
-    k_ranges<<<(unsigned)((st->max_pairs + 255) / 256), 256, 0, counted(stream)>>>(
-        tkey[2], st->pair_ids, st->depth, st->n_pairs, tiles, st->ranges, st->pair_keys);
+    k_ranges<<<(unsigned)((tiles + 7) / 8), 256, 0, counted(stream)>>>(st->pair_keys, st->n_pairs, tiles, st->ranges);
     PRTGS_CHECK_LAUNCH();
   }
   launch_composite(v, (unsigned)tiles, st, colors, n, k, bg, image, stream);

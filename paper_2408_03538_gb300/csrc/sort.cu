@@ -173,6 +173,12 @@ __device__ __forceinline__ int64_t sort_count(const uint32_t* d_count, int64_t c
   return c < capacity ? c : capacity;
 }
 
+// A sorted key with its value's 32 low bits behind it.
+template <class K>
+__device__ __forceinline__ uint64_t wide_key(K k, float low) {
+  return ((uint64_t)k << 32) | __float_as_uint(low);
+}
+
 // hist: [tile][256] when self (the scatter blocks sum it), else [256][tile] for one exclusive scan.
 template <class K>
 __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const K* __restrict__ keys, int64_t capacity,
@@ -222,7 +228,9 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const K* __restr
                                                                 K* __restrict__ keys_out, int32_t* __restrict__ vals_out,
                                                                 int64_t capacity, const uint32_t* d_count, int shift,
                                                                 unsigned mask, int n_tiles, int self,
-                                                                const uint32_t* __restrict__ hist) {
+                                                                const uint32_t* __restrict__ hist,
+                                                                const float* __restrict__ low,
+                                                                uint64_t* __restrict__ wide_out) {
   constexpr int ITEMS = SortShape<K>::kItems, TILE = SortShape<K>::kTile;
   __shared__ K skey[TILE];
   __shared__ int32_t sval[TILE];
@@ -289,8 +297,10 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const K* __restr
     const K k = skey[i];
     const int64_t dst = gofs[(unsigned)(k >> shift) & mask] + i;
     if (dst < n) {  // always true when the histograms are consistent
-      keys_out[dst] = k;
-      vals_out[dst] = sval[i];
+      const int32_t v = sval[i];
+      if (wide_out) wide_out[dst] = wide_key(k, low[v]);
+      else keys_out[dst] = k;
+      vals_out[dst] = v;
     }
   }
 }
@@ -301,7 +311,8 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_small(const K* __restric
                                                               const int32_t* __restrict__ vals_in,
                                                               K* __restrict__ keys_out, int32_t* __restrict__ vals_out,
                                                               int64_t capacity, const uint32_t* d_count, int begin_bit,
-                                                              int end_bit, int width) {
+                                                              int end_bit, int width, const float* __restrict__ low,
+                                                              uint64_t* __restrict__ wide_out) {
   constexpr int ITEMS = kSmallSort / kSortThreads;
   extern __shared__ unsigned char sort_smem[];
   K* skey = reinterpret_cast<K*>(sort_smem);
@@ -363,7 +374,8 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_small(const K* __restric
   for (int r = 0; r < ITEMS; ++r) {
     const int i = first + r * 32 + lane;
     if (r < rounds && i < n) {
-      keys_out[i] = key[r];
+      if (wide_out) wide_out[i] = wide_key(key[r], low[val[r]]);
+      else keys_out[i] = key[r];
       vals_out[i] = val[r];
     }
   }
@@ -383,7 +395,7 @@ size_t radix_sort_workspace(int64_t capacity) {
 template <class K>
 static int radix_sort_t(const K* keys_x, const int32_t* vals_x, K* keys_f, int32_t* vals_f, K* keys_y, int32_t* vals_y,
                         int64_t capacity, const uint32_t* d_count, int begin_bit, int end_bit, void* ws,
-                        cudaStream_t stream) {
+                        cudaStream_t stream, const float* low = nullptr, uint64_t* wide = nullptr) {
   if (capacity <= 0) return PRTGS_OK;
   const int bits = end_bit > begin_bit ? end_bit - begin_bit : 1;
   const int passes = (bits + 7) / 8;
@@ -392,7 +404,7 @@ static int radix_sort_t(const K* keys_x, const int32_t* vals_x, K* keys_f, int32
     const int smem = kSmallSort * (int)(sizeof(K) + sizeof(int32_t));
     cudaFuncSetAttribute(k_radix_small<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     k_radix_small<K><<<1, kSortThreads, smem, counted(stream)>>>(keys_x, vals_x, keys_f, vals_f, capacity, d_count,
-                                                                 begin_bit, begin_bit + bits, width);
+                                                                 begin_bit, begin_bit + bits, width, low, wide);
     PRTGS_CHECK_LAUNCH();
     return PRTGS_OK;
   }
@@ -413,11 +425,11 @@ static int radix_sort_t(const K* keys_x, const int32_t* vals_x, K* keys_f, int32
     const unsigned mask = (1u << w) - 1u;
     k_radix_hist<K><<<tiles, kSortThreads, 0, counted(stream)>>>(ksrc, capacity, d_count, shift, mask, tiles, self, hist);
     if (!self) {
-      const int rc = scan_u32(hist, hist, 256 * (int64_t)tiles, true, nullptr, scan_ws, stream);
+      const int rc = scan_u32(hist, hist, ((int64_t)mask + 1) * tiles, true, nullptr, scan_ws, stream);
       if (rc != PRTGS_OK) return rc;
     }
     k_radix_scatter<K><<<tiles, kSortThreads, 0, counted(stream)>>>(ksrc, vsrc, kdst, vdst, capacity, d_count, shift, mask,
-                                                                    tiles, self, hist);
+                                                                    tiles, self, hist, low, p == passes - 1 ? wide : nullptr);
     PRTGS_CHECK_LAUNCH();
     ksrc = kdst;
     vsrc = vdst;
@@ -434,9 +446,9 @@ int radix_sort_pairs(const uint64_t* keys_x, const int32_t* vals_x, uint64_t* ke
 
 int radix_sort_pairs(const uint32_t* keys_x, const int32_t* vals_x, uint32_t* keys_f, int32_t* vals_f,
                      uint32_t* keys_y, int32_t* vals_y, int64_t capacity, const uint32_t* d_count, int begin_bit,
-                     int end_bit, void* ws, cudaStream_t stream) {
+                     int end_bit, void* ws, cudaStream_t stream, const float* low, uint64_t* wide) {
   return radix_sort_t<uint32_t>(keys_x, vals_x, keys_f, vals_f, keys_y, vals_y, capacity, d_count, begin_bit, end_bit, ws,
-                                stream);
+                                stream, low, wide);
 }
 
 }  // namespace prtgs
