@@ -594,54 +594,81 @@ __global__ void __launch_bounds__(kRelightThreads) k_relight_bwd_local(int64_t n
 // dL[k,c,m] = sum_i dc[k,i,c] (rho_i[c]/pi) T_i[c][m]: per-chunk partial sums (each block walks
 // its chunk of Gaussians in order), then a fixed-order sum of the partials: deterministic.
 constexpr int kDLChunk = 2048;
-constexpr int kDLBatch = 32;
+
+// The sums of Gaussians i0 .. i1 to out [k][3][C]; light l, Gaussian i of dc: dc[(l n + i - first) 3 + c]. The
+// Gaussians are staged a batch at a time; where a pass has fewer outputs than threads, groups of threads take every
+// G-th Gaussian and their sums are added at the end. Bound by the latency of a batch (load, barrier, sum): 300k
+// Gaussians, order 3, one light, 81 us with 32 a batch and 48 of 256 threads at work, 33 us like this.
+template <int C, int TCH>
+__device__ __forceinline__ void dL_chunk(int64_t i0, int64_t i1, const float* __restrict__ T,
+                                         const float* __restrict__ albedo, int k, const float* __restrict__ dc, int64_t n,
+                                         int64_t first, float* __restrict__ out) {
+  constexpr int kBatch = TCH * C <= 48 ? 128 : 32;
+  constexpr int kOuts = 3 * C;                           // per light
+  constexpr int LPP = 512 / kOuts < 8 ? 512 / kOuts : 8;  // lights per pass: <= 512 outputs
+  constexpr int TC = TCH * C;
+  __shared__ float sT[kBatch * TC > kRelightThreads ? kBatch * TC : kRelightThreads];
+  __shared__ float sW[kBatch][3 * 8];  // dc * rho / pi for up to 8 lights per pass
+  const int tid = threadIdx.x;
+  for (int l0 = 0; l0 < k; l0 += LPP) {
+    const int nl = min(LPP, k - l0);
+    const int nout = nl * kOuts;
+    const int G = nout <= kRelightThreads ? kRelightThreads / nout : 1;
+    const int grp = G > 1 ? tid / nout : 0;
+    const int o0 = G > 1 ? tid % nout : tid;
+    float acc[2] = {0.f, 0.f};  // outputs o0 and, with one group, tid + 256 (nout <= 512)
+    for (int64_t b = i0; b < i1; b += kBatch) {
+      const int nb = (int)min((int64_t)kBatch, i1 - b);
+      __syncthreads();
+#pragma unroll 8
+      for (int e = tid; e < nb * TC; e += kRelightThreads) sT[e] = T[b * TC + e];
+      for (int e = tid; e < nb * 3 * nl; e += kRelightThreads) {
+        const int l = e / (3 * nb), r = e - l * 3 * nb;  // r = 3 j + c: a light's colours are contiguous
+        const int j = r / 3, c = r - 3 * j;
+        sW[j][3 * l + c] = dc[((int64_t)(l0 + l) * n + (b - first)) * 3 + r] * albedo[3 * b + r] * (1.0f / kPi);
+      }
+      __syncthreads();
+      if (grp < G) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int o = o0 + q * kRelightThreads;
+          if (o < nout) {
+            const int l = o / kOuts, r = o % kOuts;
+            const int c = r / C, m = r % C;
+            const float* w = &sW[0][3 * l + c];
+            const float* t = sT + (TCH > 1 ? c : 0) * C + m;
+            float a = acc[q];
+#pragma unroll 4
+            for (int j = grp; j < nb; j += G) a = fmaf(w[24 * j], t[TC * j], a);
+            acc[q] = a;
+          }
+        }
+      }
+    }
+    if (G > 1) {
+      __syncthreads();
+      sT[tid] = acc[0];
+      __syncthreads();
+      if (grp == 0)
+        for (int g = 1; g < G; ++g) acc[0] += sT[g * nout + tid];
+    }
+    if (grp == 0) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int o = o0 + q * kRelightThreads;
+        if (o < nout) out[l0 * kOuts + o] = acc[q];
+      }
+    }
+  }
+}
 
 template <int C, int TCH>
 __global__ void __launch_bounds__(kRelightThreads) k_relight_dL_partial(int64_t n, const float* __restrict__ T,
                                                                         const float* __restrict__ albedo, int k,
                                                                         const float* __restrict__ dcol,
                                                                         float* __restrict__ partial) {
-  __shared__ float sT[kDLBatch][TCH * C];
-  __shared__ float sW[kDLBatch][3 * 8];  // dc * rho / pi for up to 8 lights per pass
-  const int outs_per_light = 3 * C;
   const int64_t i0 = (int64_t)blockIdx.x * kDLChunk;
-  constexpr int LPP = 512 / (3 * C) < 8 ? 512 / (3 * C) : 8;  // lights per pass: <= 512 outputs
-  for (int l0 = 0; l0 < k; l0 += LPP) {
-    const int nl = min(LPP, k - l0);
-    const int nout = nl * outs_per_light;
-    float acc[2] = {0.f, 0.f};  // outputs tid and tid + 256 (nout <= 512)
-    for (int64_t b = i0; b < i0 + kDLChunk && b < n; b += kDLBatch) {
-      __syncthreads();
-      for (int e = threadIdx.x; e < kDLBatch * TCH * C; e += blockDim.x) {
-        int j = e / (TCH * C), r = e % (TCH * C);
-        int64_t i = b + j;
-        sT[j][r] = i < n ? T[i * TCH * C + r] : 0.f;
-      }
-      for (int e = threadIdx.x; e < kDLBatch * 3 * nl; e += blockDim.x) {
-        int j = e / (3 * nl), r = e % (3 * nl);
-        int l = r / 3, c = r % 3;
-        int64_t i = b + j;
-        sW[j][r] = i < n ? dcol[((int64_t)(l0 + l) * n + i) * 3 + c] * albedo[3 * i + c] * (1.0f / kPi) : 0.f;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        int o = threadIdx.x + q * kRelightThreads;
-        if (o < nout) {
-          int l = o / outs_per_light, r = o % outs_per_light;
-          int c = r / C, m = r % C;
-          float a = acc[q];
-          for (int j = 0; j < kDLBatch; ++j) a = fmaf(sW[j][3 * l + c], sT[j][(TCH > 1 ? c : 0) * C + m], a);
-          acc[q] = a;
-        }
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      int o = threadIdx.x + q * kRelightThreads;
-      if (o < nout) partial[(int64_t)blockIdx.x * k * outs_per_light + (int64_t)l0 * outs_per_light + o] = acc[q];
-    }
-  }
+  dL_chunk<C, TCH>(i0, min(n, i0 + kDLChunk), T, albedo, k, dcol, n, 0, partial + (int64_t)blockIdx.x * k * 3 * C);
 }
 
 __global__ void k_sum_partials(const float* __restrict__ partial, int64_t nblocks, int nout, float* __restrict__ out) {
@@ -743,53 +770,13 @@ template <int C, int TCH>
 __global__ void __launch_bounds__(kRelightThreads) k_relight_dL_partial_batched(
     const int64_t* __restrict__ offs, const float* __restrict__ T, const float* __restrict__ albedo, int k,
     const float* __restrict__ dcol, float* __restrict__ partial) {
-  __shared__ float sT[kDLBatch][TCH * C];
-  __shared__ float sW[kDLBatch][3 * 8];
   const int b = blockIdx.y;
   const int64_t o = offs[b], nb = offs[b + 1] - o;
   const int64_t i0 = o + (int64_t)blockIdx.x * kDLChunk;
   if ((int64_t)blockIdx.x * kDLChunk >= nb) return;  // uniform: past the scene's chunks
-  const int64_t i1 = min(o + nb, i0 + kDLChunk);
-  const float* dc = dcol + 3 * (int64_t)k * o;
-  const int outs_per_light = 3 * C;
   const int64_t slot = o / kDLChunk + b + blockIdx.x;
-  constexpr int LPP = 512 / (3 * C) < 8 ? 512 / (3 * C) : 8;  // lights per pass: <= 512 outputs
-  for (int l0 = 0; l0 < k; l0 += LPP) {
-    const int nl = min(LPP, k - l0);
-    const int nout = nl * outs_per_light;
-    float acc[2] = {0.f, 0.f};
-    for (int64_t bb = i0; bb < i1; bb += kDLBatch) {
-      __syncthreads();
-      for (int e = threadIdx.x; e < kDLBatch * TCH * C; e += blockDim.x) {
-        const int j = e / (TCH * C), r = e % (TCH * C);
-        const int64_t i = bb + j;
-        sT[j][r] = i < i1 ? T[i * TCH * C + r] : 0.f;
-      }
-      for (int e = threadIdx.x; e < kDLBatch * 3 * nl; e += blockDim.x) {
-        const int j = e / (3 * nl), r = e % (3 * nl);
-        const int l = r / 3, c = r % 3;
-        const int64_t i = bb + j;
-        sW[j][r] = i < i1 ? dc[((int64_t)(l0 + l) * nb + (i - o)) * 3 + c] * albedo[3 * i + c] * (1.0f / kPi) : 0.f;
-      }
-      __syncthreads();
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int ot = threadIdx.x + q * kRelightThreads;
-        if (ot < nout) {
-          const int l = ot / outs_per_light, r = ot % outs_per_light;
-          const int c = r / C, m = r % C;
-          float a = acc[q];
-          for (int j = 0; j < kDLBatch; ++j) a = fmaf(sW[j][3 * l + c], sT[j][(TCH > 1 ? c : 0) * C + m], a);
-          acc[q] = a;
-        }
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int ot = threadIdx.x + q * kRelightThreads;
-      if (ot < nout) partial[slot * k * outs_per_light + (int64_t)l0 * outs_per_light + ot] = acc[q];
-    }
-  }
+  dL_chunk<C, TCH>(i0, min(o + nb, i0 + kDLChunk), T, albedo, k, dcol + 3 * (int64_t)k * o, nb, o,
+                   partial + slot * k * 3 * C);
 }
 
 // dL[b] = the scene's partial sums in chunk order (compensated): deterministic.
