@@ -117,7 +117,9 @@ class Bvh:
 def build_bvh(g: GaussianTensors, scene_offsets: torch.Tensor | None = None, status: Status | None = None) -> Bvh:
     lib = L.load()
     if scene_offsets is None:
-        scene_offsets = torch.tensor([0, g.n], dtype=torch.int64, device=g.means.device)
+        # [0, n] made on the device: a copy from the host would wait for all the work queued before
+        scene_offsets = torch.arange(0, g.n + 1, g.n, dtype=torch.int64, device=g.means.device) if g.n else \
+            torch.zeros(2, dtype=torch.int64, device=g.means.device)
     bvh = Bvh(g.n, scene_offsets)
     ws, nb = _ws(lib.prtgs_build_bvh_workspace_size(g.n, bvh.n_scenes), g.means.device)
     gs = g.struct()
