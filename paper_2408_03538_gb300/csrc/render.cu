@@ -58,11 +58,6 @@ struct OneView {
   __device__ __forceinline__ int64_t count(int, int64_t n) const { return n; }
 };
 
-// OneView with the colours as rows [n][color_floats(k)]: one splat's sets side by side.
-struct RowView : OneView {
-  static constexpr bool kRows = true;
-};
-
 struct ManyViews {
   static constexpr bool kRows = false;
   Cam c[kMaxScenes];
@@ -72,6 +67,12 @@ struct ManyViews {
   __device__ __forceinline__ const Cam& cam(int b) const { return c[b]; }
   __device__ __forceinline__ int64_t first(int b) const { return offs[b]; }
   __device__ __forceinline__ int64_t count(int b, int64_t) const { return offs[b + 1] - offs[b]; }
+};
+
+// A view with the colours as rows [n][color_floats(k)]: one splat's sets side by side.
+template <class V>
+struct Rows : V {
+  static constexpr bool kRows = true;
 };
 
 // Colour of light l, channel ch of Gaussian g (in scene b).
@@ -327,6 +328,35 @@ __device__ __forceinline__ bool reaches(float mx, float my, const float4& co, fl
   return !(fx > K) || !(fy > K);
 }
 
+// The colours of k >= 2 sets as rows. A warp's 32 splats lie anywhere, so from [k][n][3] each of their sets is a
+// sector of its own, read a word at a time; from rows it is 16-byte words of a few lines. 8 lights of 100k splats:
+// composite 423 us from [k][n][3], 370 from rows, which take 7 to write; the backward of 8 scenes x 4 lights 1,644
+// and 1,394 us.
+template <class V>
+__global__ void __launch_bounds__(256) k_color_rows(int64_t n, V v, const float* __restrict__ colors, int k,
+                                                    float4* __restrict__ rows) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int b = v.scene_of(i);
+  const int q = color_floats(k) / 4;
+  for (int j = 0; j < q; ++j) {
+    float f[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int l = (4 * j + e) / 3, ch = (4 * j + e) % 3;
+      f[e] = l < k ? __ldg(colors + color_at(v, b, i, l, k, n) + ch) : 0.f;
+    }
+    rows[i * q + j] = make_float4(f[0], f[1], f[2], f[3]);
+  }
+}
+
+template <class V>
+static Rows<V> rows_of(const V& v) {
+  Rows<V> r;
+  static_cast<V&>(r) = v;
+  return r;
+}
+
 // Per-warp staging of k_composite: 32 splats and their colours.
 template <int KG>
 struct FwdWarp {
@@ -334,6 +364,21 @@ struct FwdWarp {
   float4 xy[32];  // mean2d, Gaussian, position in the tile's list (bits)
   float col[32][color_floats(KG)];
 };
+
+// The colour sets l0 .. l0 + KG of nk staged splats (xy.z: the Gaussian) from rows: consecutive lanes on a row's
+// 16-byte words; past the row's end, zeros.
+template <int KG>
+__device__ __forceinline__ void stage_rows(float (*col)[color_floats(KG)], const float4* xy, int nk,
+                                           const float* __restrict__ rows, int l0, int k) {
+  constexpr int Q = color_floats(KG) / 4;
+  const int stride = color_floats(k) / 4, q0 = 3 * l0 / 4;
+  for (int e = threadIdx.x & 31; e < nk * Q; e += 32) {
+    const int slot = e / Q, q = e % Q;
+    reinterpret_cast<float4*>(col[slot])[q] =
+        q0 + q < stride ? __ldg(reinterpret_cast<const float4*>(rows) + (int64_t)__float_as_int(xy[slot].z) * stride + q0 + q)
+                        : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+}
 
 // One warp per 8 x 4 pixels of a tile, on its own (no block barrier), for a group of KG colour sets: it takes its
 // tile's list 32 splats at a time, one per lane, drops those that cannot reach its pixels (reaches; most of a
@@ -402,15 +447,8 @@ __global__ void __launch_bounds__(kTileThreads, KG <= 8 ? 3 : 2) k_composite(
     }
     fetch(base + 32 + lane);
     __syncwarp();
-    if constexpr (V::kRows) {  // consecutive lanes on a row's 16-byte words
-      constexpr int Q = CF / 4;
-      const int stride = color_floats(k) / 4, q0 = 3 * l0 / 4;
-      for (int e = lane; e < nk * Q; e += 32) {
-        const int slot = e / Q, q = e % Q;
-        if (q0 + q < stride)
-          reinterpret_cast<float4*>(sm.col[slot])[q] =
-              __ldg(reinterpret_cast<const float4*>(colors) + (int64_t)__float_as_int(sm.xy[slot].z) * stride + q0 + q);
-      }
+    if constexpr (V::kRows) {
+      stage_rows<KG>(sm.col, sm.xy, nk, colors, l0, k);
       __syncwarp();
     }
     for (int j = 0; j < nk; ++j) {
@@ -525,6 +563,17 @@ static int render_views(const prtgs_gaussians* g, const float* colors, int32_t k
     k_ranges<<<(unsigned)((tiles + 7) / 8), 256, 0, counted(stream)>>>(st->pair_keys, st->n_pairs, tiles, st->ranges);
     PRTGS_CHECK_LAUNCH();
   }
+  if constexpr (!V::kRows) {
+    // rows for the colours, where the sort's buffers, which are free again, have the room
+    const size_t room = reinterpret_cast<char*>(sort_ws) - reinterpret_cast<char*>(tkey[0]);
+    if (k >= 2 && n > 0 && sizeof(float) * color_floats(k) * (size_t)n <= room) {
+      k_color_rows<V><<<(unsigned)((n + 255) / 256), 256, 0, counted(stream)>>>(n, v, colors, k,
+                                                                                reinterpret_cast<float4*>(tkey[0]));
+      launch_composite(rows_of(v), (unsigned)tiles, st, reinterpret_cast<const float*>(tkey[0]), n, k, bg, image, stream);
+      PRTGS_CHECK_LAUNCH();
+      return PRTGS_OK;
+    }
+  }
   launch_composite(v, (unsigned)tiles, st, colors, n, k, bg, image, stream);
   PRTGS_CHECK_LAUNCH();
   return PRTGS_OK;
@@ -538,7 +587,7 @@ int render(const prtgs_gaussians* g, const float* colors, int32_t k, const prtgs
 
 int render_rows(const prtgs_gaussians* g, const float* rows, int32_t k, const prtgs_camera* cam, const float* bg,
                 float* image, prtgs_render_state* st, int32_t* status, void* ws, cudaStream_t stream) {
-  RowView v;
+  Rows<OneView> v;
   v.c = make_cam(cam);
   return render_views(g, rows, k, v, v.c, 1, bg, image, st, status, ws, stream);
 }
@@ -659,14 +708,20 @@ __global__ void __launch_bounds__(kTileThreads) k_composite_bwd(
       const int slot = __popc(m & ((1u << lane) - 1u));
       sm.co[slot] = co;
       sm.xy[slot] = make_float4(xy.x, xy.y, __int_as_float(gid), __int_as_float(p));
+      if constexpr (!V::kRows) {
 #pragma unroll
-      for (int l = 0; l < KG; ++l) {
-        const float* cp = colors + color_at(v, b, gid, l0 + (l < nl ? l : 0), k, n);
+        for (int l = 0; l < KG; ++l) {
+          const float* cp = colors + color_at(v, b, gid, l0 + (l < nl ? l : 0), k, n);
 #pragma unroll
-        for (int ch = 0; ch < 3; ++ch) sm.col[slot][3 * l + ch] = l < nl ? cp[ch] : 0.f;
+          for (int ch = 0; ch < 3; ++ch) sm.col[slot][3 * l + ch] = l < nl ? cp[ch] : 0.f;
+        }
       }
     }
     __syncwarp();
+    if constexpr (V::kRows) {
+      stage_rows<KG>(sm.col, sm.xy, nk, colors, l0, k);
+      __syncwarp();
+    }
     for (int c0 = 0; c0 < nk; c0 += kBwdChunk) {
       const int cnt = min(kBwdChunk, nk - c0);
       for (int i = 0; i < cnt; ++i) {
@@ -937,7 +992,7 @@ int render_geometry(const prtgs_gaussians* g, const prtgs_camera* cam, float* de
 }
 
 size_t render_backward_workspace(int64_t n, int32_t k) {
-  return align_up(sizeof(float) * (size_t)bwd_stride(k) * n);
+  return align_up(sizeof(float) * (size_t)bwd_stride(k) * n) + (k >= 2 ? align_up(sizeof(float) * color_floats(k) * (size_t)n) : 0);
 }
 
 template <int KG, class V>
@@ -958,14 +1013,21 @@ static int render_backward_views(const prtgs_gaussians* g, const float* colors, 
   const int64_t n = g->n;
   if (n == 0) return PRTGS_OK;
   const int64_t tiles = (int64_t)c.gx * c.gy * B;
-  float* acc = static_cast<float*>(ws);
   const int kg = bwd_group(k), stride = bwd_stride(k);
+  Carver cv(ws);
+  float* acc = cv.take<float>((size_t)stride * n);
   cudaMemsetAsync(acc, 0, sizeof(float) * stride * n, stream);
   // every light's colour sets in groups of up to 8 (shared memory bound)
   dim3 grid((unsigned)tiles, (unsigned)((k + kg - 1) / kg));
-  if (kg == 1) launch_composite_bwd<1>(grid, v, st, colors, n, k, bg, dimage, acc, stride, stream);
-  else if (kg == 4) launch_composite_bwd<4>(grid, v, st, colors, n, k, bg, dimage, acc, stride, stream);
-  else launch_composite_bwd<8>(grid, v, st, colors, n, k, bg, dimage, acc, stride, stream);
+  if (kg == 1) {
+    launch_composite_bwd<1>(grid, v, st, colors, n, k, bg, dimage, acc, stride, stream);
+  } else {
+    float* rows = cv.take<float>((size_t)color_floats(k) * n);
+    k_color_rows<V><<<(unsigned)((n + 255) / 256), 256, 0, counted(stream)>>>(n, v, colors, k,
+                                                                              reinterpret_cast<float4*>(rows));
+    if (kg == 4) launch_composite_bwd<4>(grid, rows_of(v), st, rows, n, k, bg, dimage, acc, stride, stream);
+    else launch_composite_bwd<8>(grid, rows_of(v), st, rows, n, k, bg, dimage, acc, stride, stream);
+  }
   PRTGS_CHECK_LAUNCH();
   k_preprocess_bwd<V><<<(unsigned)((n + 255) / 256), 256, 0, counted(stream)>>>(
       n, g->means, g->scales, g->quats, v, st->radius, reinterpret_cast<const float4*>(st->conic_op), acc, stride, k, kg,

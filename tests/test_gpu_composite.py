@@ -127,5 +127,7 @@ def test_color_groups_and_rows_agree(w, h, k):
         assert torch.equal(one[0], img[l]), l
         for field, dt in (("final_T", torch.float32), ("n_contrib", torch.int32)):
             assert torch.equal(s.view(field, dt, (h, w)), s1.view(field, dt, (h, w)))
+    tight, _ = api.render(g, colors, cam, bg, max_pairs=s.n_pairs(), status=st)  # the colours read in place
+    assert st.read() == 0 and torch.equal(tight, img)
     _, normal, _ = api.render_geometry(g, cam, max_pairs=400_000)
     assert torch.equal(normal, img[1])
