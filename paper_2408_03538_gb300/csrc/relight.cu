@@ -596,79 +596,84 @@ __global__ void __launch_bounds__(kRelightThreads) k_relight_bwd_local(int64_t n
 constexpr int kDLChunk = 2048;
 
 // The sums of Gaussians i0 .. i1 to out [k][3][C]; light l, Gaussian i of dc: dc[(l n + i - first) 3 + c]. The
-// Gaussians are staged a batch at a time; where a pass has fewer outputs than threads, groups of threads take every
-// G-th Gaussian and their sums are added at the end. Bound by the latency of a batch (load, barrier, sum): 300k
-// Gaussians, order 3, one light, 81 us with 32 a batch and 48 of 256 threads at work, 33 us like this.
-template <int C, int TCH>
+// Gaussians are staged a batch at a time; a thread holds one (c, m) of LQ lights, groups of threads take every G-th
+// Gaussian and their sums are added at the end. Bound by the latency of a batch (load, barrier, sum): 300k
+// Gaussians, order 3, one light, 81 us with 32 a batch and 48 of 256 threads at work, 33 us like this; 8 scenes of
+// 400k in all and 4 lights 122 us with a thread per output, 68 us like this.
+template <int C, int TCH, int LQ>
 __device__ __forceinline__ void dL_chunk(int64_t i0, int64_t i1, const float* __restrict__ T,
                                          const float* __restrict__ albedo, int k, const float* __restrict__ dc, int64_t n,
                                          int64_t first, float* __restrict__ out) {
   constexpr int kBatch = TCH * C <= 48 ? 128 : 32;
-  constexpr int kOuts = 3 * C;                           // per light
-  constexpr int LPP = 512 / kOuts < 8 ? 512 / kOuts : 8;  // lights per pass: <= 512 outputs
+  constexpr int kOuts = 3 * C;  // per light
+  constexpr int kQuads = kRelightThreads / kOuts;  // thread groups' worth of (c, m)
+  constexpr int LPP = kQuads * LQ < 8 ? kQuads * LQ : (8 / LQ) * LQ;  // lights per pass
   constexpr int TC = TCH * C;
-  __shared__ float sT[kBatch * TC > kRelightThreads ? kBatch * TC : kRelightThreads];
-  __shared__ float sW[kBatch][3 * 8];  // dc * rho / pi for up to 8 lights per pass
+  __shared__ float sT[kBatch * TC > LQ * kRelightThreads ? kBatch * TC : LQ * kRelightThreads];
+  __shared__ __align__(16) float sW[kBatch][3][8];  // dc * rho / pi
   const int tid = threadIdx.x;
   for (int l0 = 0; l0 < k; l0 += LPP) {
     const int nl = min(LPP, k - l0);
-    const int nout = nl * kOuts;
-    const int G = nout <= kRelightThreads ? kRelightThreads / nout : 1;
-    const int grp = G > 1 ? tid / nout : 0;
-    const int o0 = G > 1 ? tid % nout : tid;
-    float acc[2] = {0.f, 0.f};  // outputs o0 and, with one group, tid + 256 (nout <= 512)
+    const int nthr = (nl + LQ - 1) / LQ * kOuts;  // <= 256
+    const int G = kRelightThreads / nthr;
+    const int grp = tid / nthr, o = tid % nthr;
+    const int lq = o / kOuts * LQ, c = o % kOuts / C, m = o % C;
+    float acc[LQ];
+#pragma unroll
+    for (int q = 0; q < LQ; ++q) acc[q] = 0.f;
     for (int64_t b = i0; b < i1; b += kBatch) {
       const int nb = (int)min((int64_t)kBatch, i1 - b);
       __syncthreads();
 #pragma unroll 8
       for (int e = tid; e < nb * TC; e += kRelightThreads) sT[e] = T[b * TC + e];
       for (int e = tid; e < nb * 3 * nl; e += kRelightThreads) {
-        const int l = e / (3 * nb), r = e - l * 3 * nb;  // r = 3 j + c: a light's colours are contiguous
-        const int j = r / 3, c = r - 3 * j;
-        sW[j][3 * l + c] = dc[((int64_t)(l0 + l) * n + (b - first)) * 3 + r] * albedo[3 * b + r] * (1.0f / kPi);
+        const int l = e / (3 * nb), r = e - l * 3 * nb;  // r = 3 j + channel: a light's colours are contiguous
+        sW[r / 3][r % 3][l] = dc[((int64_t)(l0 + l) * n + (b - first)) * 3 + r] * albedo[3 * b + r] * (1.0f / kPi);
       }
       __syncthreads();
       if (grp < G) {
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int o = o0 + q * kRelightThreads;
-          if (o < nout) {
-            const int l = o / kOuts, r = o % kOuts;
-            const int c = r / C, m = r % C;
-            const float* w = &sW[0][3 * l + c];
-            const float* t = sT + (TCH > 1 ? c : 0) * C + m;
-            float a = acc[q];
+        const float* t = sT + (TCH > 1 ? c : 0) * C + m;
 #pragma unroll 4
-            for (int j = grp; j < nb; j += G) a = fmaf(w[24 * j], t[TC * j], a);
-            acc[q] = a;
+        for (int j = grp; j < nb; j += G) {
+          const float v = t[TC * j];
+          if constexpr (LQ == 4) {
+            const float4 w = *reinterpret_cast<const float4*>(&sW[j][c][lq]);
+            acc[0] = fmaf(w.x, v, acc[0]);
+            acc[1] = fmaf(w.y, v, acc[1]);
+            acc[2] = fmaf(w.z, v, acc[2]);
+            acc[3] = fmaf(w.w, v, acc[3]);
+          } else {
+            acc[0] = fmaf(sW[j][c][lq], v, acc[0]);
           }
         }
       }
     }
     if (G > 1) {
       __syncthreads();
-      sT[tid] = acc[0];
+#pragma unroll
+      for (int q = 0; q < LQ; ++q) sT[q * kRelightThreads + tid] = acc[q];
       __syncthreads();
       if (grp == 0)
-        for (int g = 1; g < G; ++g) acc[0] += sT[g * nout + tid];
+        for (int g = 1; g < G; ++g)
+#pragma unroll
+          for (int q = 0; q < LQ; ++q) acc[q] += sT[q * kRelightThreads + g * nthr + tid];
     }
     if (grp == 0) {
 #pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int o = o0 + q * kRelightThreads;
-        if (o < nout) out[l0 * kOuts + o] = acc[q];
-      }
+      for (int q = 0; q < LQ; ++q)
+        if (lq + q < nl) out[(l0 + lq + q) * kOuts + c * C + m] = acc[q];
     }
   }
 }
 
-template <int C, int TCH>
+template <int C, int TCH, int LQ>
 __global__ void __launch_bounds__(kRelightThreads) k_relight_dL_partial(int64_t n, const float* __restrict__ T,
                                                                         const float* __restrict__ albedo, int k,
                                                                         const float* __restrict__ dcol,
                                                                         float* __restrict__ partial) {
   const int64_t i0 = (int64_t)blockIdx.x * kDLChunk;
-  dL_chunk<C, TCH>(i0, min(n, i0 + kDLChunk), T, albedo, k, dcol, n, 0, partial + (int64_t)blockIdx.x * k * 3 * C);
+  float* out = partial + (int64_t)blockIdx.x * k * 3 * C;
+  dL_chunk<C, TCH, LQ>(i0, min(n, i0 + kDLChunk), T, albedo, k, dcol, n, 0, out);
 }
 
 __global__ void k_sum_partials(const float* __restrict__ partial, int64_t nblocks, int nout, float* __restrict__ out) {
@@ -703,10 +708,9 @@ static void launch_relight_bwd(int64_t n, const float* T, int tch, const float* 
     k_relight_bwd_local<C, 3><<<grid, kRelightThreads, smem, counted(stream)>>>(n, T, albedo, L, k, dcol, d_albedo, dT);
   else
     k_relight_bwd_local<C, 1><<<grid, kRelightThreads, smem, counted(stream)>>>(n, T, albedo, L, k, dcol, d_albedo, dT);
-  if (tch == 3)
-    k_relight_dL_partial<C, 3><<<(unsigned)nb, kRelightThreads, 0, counted(stream)>>>(n, T, albedo, k, dcol, partial);
-  else
-    k_relight_dL_partial<C, 1><<<(unsigned)nb, kRelightThreads, 0, counted(stream)>>>(n, T, albedo, k, dcol, partial);
+  const auto dl = k <= 2 ? (tch == 3 ? k_relight_dL_partial<C, 3, 1> : k_relight_dL_partial<C, 1, 1>)
+                         : (tch == 3 ? k_relight_dL_partial<C, 3, 4> : k_relight_dL_partial<C, 1, 4>);
+  dl<<<(unsigned)nb, kRelightThreads, 0, counted(stream)>>>(n, T, albedo, k, dcol, partial);
   int nout = k * 3 * C;
   k_sum_partials<<<(nout + 255) / 256, 256, 0, counted(stream)>>>(partial, nb, nout, dL);
 }
@@ -766,7 +770,7 @@ __global__ void __launch_bounds__(kRelightThreads) k_relight_bwd_local_batched(
 
 // Partial sums of dL over chunk x of scene y (blockIdx), written to slot offs[y] / kDLChunk + y + x
 // (the slots of a scene are consecutive and disjoint from the other scenes').
-template <int C, int TCH>
+template <int C, int TCH, int LQ>
 __global__ void __launch_bounds__(kRelightThreads) k_relight_dL_partial_batched(
     const int64_t* __restrict__ offs, const float* __restrict__ T, const float* __restrict__ albedo, int k,
     const float* __restrict__ dcol, float* __restrict__ partial) {
@@ -775,8 +779,8 @@ __global__ void __launch_bounds__(kRelightThreads) k_relight_dL_partial_batched(
   const int64_t i0 = o + (int64_t)blockIdx.x * kDLChunk;
   if ((int64_t)blockIdx.x * kDLChunk >= nb) return;  // uniform: past the scene's chunks
   const int64_t slot = o / kDLChunk + b + blockIdx.x;
-  dL_chunk<C, TCH>(i0, min(o + nb, i0 + kDLChunk), T, albedo, k, dcol + 3 * (int64_t)k * o, nb, o,
-                   partial + slot * k * 3 * C);
+  dL_chunk<C, TCH, LQ>(i0, min(o + nb, i0 + kDLChunk), T, albedo, k, dcol + 3 * (int64_t)k * o, nb, o,
+                       partial + slot * k * 3 * C);
 }
 
 // dL[b] = the scene's partial sums in chunk order (compensated): deterministic.
@@ -818,10 +822,9 @@ static void launch_relight_bwd_batched(int64_t n, const float* T, int tch, const
   else
     k_relight_bwd_local_batched<C, 1><<<grid, kRelightThreads, 0, counted(stream)>>>(n, T, albedo, offs, B, L, k, dcol,
                                                                                     d_albedo, dT);
-  if (tch == 3)
-    k_relight_dL_partial_batched<C, 3><<<pgrid, kRelightThreads, 0, counted(stream)>>>(offs, T, albedo, k, dcol, partial);
-  else
-    k_relight_dL_partial_batched<C, 1><<<pgrid, kRelightThreads, 0, counted(stream)>>>(offs, T, albedo, k, dcol, partial);
+  const auto dl = k <= 2 ? (tch == 3 ? k_relight_dL_partial_batched<C, 3, 1> : k_relight_dL_partial_batched<C, 1, 1>)
+                         : (tch == 3 ? k_relight_dL_partial_batched<C, 3, 4> : k_relight_dL_partial_batched<C, 1, 4>);
+  dl<<<pgrid, kRelightThreads, 0, counted(stream)>>>(offs, T, albedo, k, dcol, partial);
   const int nout = k * 3 * C;
   k_sum_partials_batched<<<dim3((unsigned)((nout + 255) / 256), (unsigned)B), 256, 0, counted(stream)>>>(partial, offs, nout,
                                                                                                  dL);
