@@ -148,10 +148,10 @@ int scan_u32(const uint32_t* in, uint32_t* out, int64_t n, bool exclusive, uint3
 // ------------------------------------------------------------------------------------------
 // Stable LSD radix sort, digits of at most 8 bits. One pass = digit histograms per tile of 4,096 (or
 // 2,048 64-bit) keys, their prefix sums, and a stable scatter: a warp ranks its own contiguous part of the tile
-// (__match_any_sync, counters in shared memory, no block barrier), the tile is put in digit order in
-// shared memory, and runs of one digit leave it as coalesced writes. (Ranking round by round with five
-// block barriers each and writing from the ranks took 200 us a pass for 25 M pairs of 12 bytes; this takes the same for
-// 8-byte ones, at two blocks an SM, and 16 us where three launches more and 45 us went at 1 M.)
+// (eight ballots, one per bit, counters in shared memory, no block barrier), the tile is put in digit order in
+// shared memory, and runs of one digit leave it as coalesced writes. 25 M pairs in two passes, the second writing
+// 12 bytes a pair: 383 us at three blocks an SM; 515 with __match_any_sync, whose time grows with the distinct
+// digits of a round; 483 with the values loaded after the ranks; 659 at two blocks, 447 at four (which spill).
 // Up to 256 tiles a scatter block sums the histograms itself, which saves three launches a pass; one
 // tile alone is sorted over all digits in one launch.
 // The element count may live on the device (d_count), so the whole sort can be enqueued
@@ -195,7 +195,8 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const K* __restrict
     if (i < n) atomicAdd(&h[(unsigned)(keys[i] >> shift) & mask], 1u);
   }
   __syncthreads();
-  hist[self ? (int64_t)blockIdx.x * 256 + threadIdx.x : (int64_t)threadIdx.x * n_tiles + blockIdx.x] = h[threadIdx.x];
+  if (self) hist[(int64_t)blockIdx.x * 256 + threadIdx.x] = h[threadIdx.x];
+  else if (threadIdx.x <= mask) hist[(int64_t)threadIdx.x * n_tiles + blockIdx.x] = h[threadIdx.x];
 }
 
 // Ranks of a warp's keys (round by round, in order) among the warp's keys of the same digit; cnt: the warp's
@@ -209,21 +210,26 @@ __device__ __forceinline__ void warp_ranks(const K (&key)[ITEMS], int rounds, in
   for (int r = 0; r < ITEMS; ++r) {
     if (r >= rounds) break;  // uniform
     const bool valid = first + r * 32 + lane < n;
-    const unsigned digit = valid ? (unsigned)(key[r] >> shift) & mask : 256u;
-    const unsigned peers = __match_any_sync(0xffffffffu, digit);
-    const int leader = __ffs(peers) - 1;
+    const unsigned digit = (unsigned)(key[r] >> shift) & mask;
+    unsigned peers = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+    for (int bit = 0; bit < 8; ++bit) {
+      const unsigned ones = __ballot_sync(0xffffffffu, (digit >> bit) & 1u);
+      peers &= (digit >> bit) & 1u ? ones : ~ones;
+    }
+    const int leader = __ffs(peers) - 1;  // (an invalid lane's peers are the valid lanes of its digit, or none)
     unsigned old = 0;
     if (valid && lane == leader) {
       old = cnt[digit];
       cnt[digit] = old + __popc(peers);
     }
-    rank[r] = __shfl_sync(0xffffffffu, old, leader) + __popc(peers & lt_mask);
+    rank[r] = __shfl_sync(0xffffffffu, old, leader & 31) + __popc(peers & lt_mask);
     __syncwarp();
   }
 }
 
 template <class K>
-__global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const K* __restrict__ keys_in,
+__global__ void __launch_bounds__(kSortThreads, 3) k_radix_scatter(const K* __restrict__ keys_in,
                                                                 const int32_t* __restrict__ vals_in,
                                                                 K* __restrict__ keys_out, int32_t* __restrict__ vals_out,
                                                                 int64_t capacity, const uint32_t* d_count, int shift,
@@ -246,12 +252,16 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const K* __restr
   for (int w = 0; w < kSortWarps; ++w) cnt[w][tid] = 0;
   const int64_t first = base + warp * 32 * ITEMS;
   K key[ITEMS];
-  int32_t val[ITEMS];
   unsigned rank[ITEMS];
 #pragma unroll
   for (int r = 0; r < ITEMS; ++r) {
     const int64_t i = first + r * 32 + lane;
     key[r] = i < n ? keys_in[i] : (K)0;
+  }
+  int32_t val[ITEMS];
+#pragma unroll
+  for (int r = 0; r < ITEMS; ++r) {
+    const int64_t i = first + r * 32 + lane;
     val[r] = i < n ? (vals_in ? vals_in[i] : (int32_t)i) : 0;
   }
   __syncthreads();
@@ -277,7 +287,7 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_scatter(const K* __restr
     }
     gbase = (int64_t)block_exclusive_scan(total, sw, all) + before;
   } else {
-    gbase = hist[(int64_t)tid * n_tiles + blockIdx.x];
+    gbase = tid <= mask ? hist[(int64_t)tid * n_tiles + blockIdx.x] : 0;
   }
   dstart[tid] = ds;
   gofs[tid] = gbase - ds;
