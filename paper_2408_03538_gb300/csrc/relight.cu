@@ -48,7 +48,38 @@ __global__ void __launch_bounds__(kRelightThreads) k_relight(int64_t n, const fl
   }
 }
 
-// Glossy splats: t_eff[a] = sum_b M[a,b] Y_b(v), v = normalize(cam - mu) (Eq. 41).
+// Splats of a block of glossy matrices: a thread per coefficient, at most 40 KB of matrices.
+constexpr int glossy_group(int C) {
+  return (256 / C) * C * (C | 1) <= 10240 ? 256 / C : 10240 / (C * (C | 1));
+}
+
+// t_eff[a] = sum_b M[a,b] Y_b(v), v = normalize(cam - mu) (Eq. 41) of ng glossy splats from g0 on: thread g C + a
+// returns its coefficient (0 past ng C). The matrices are staged in shared memory (coalesced, at an odd row
+// stride): a thread per splat that reads its own kilobyte took 283 us for the features of 300k splats at order 3, 80
+// like this (the bytes alone 70), and 39 us for the colours of 30k, 16 like this.
+template <int ORDER>
+__device__ __forceinline__ float glossy_teff(int64_t g0, int ng, const int32_t* __restrict__ ids, const float* __restrict__ M,
+                                             const float* __restrict__ means, float cx, float cy, float cz) {
+  constexpr int C = (ORDER + 1) * (ORDER + 1), P = C | 1, G = glossy_group(C);
+  __shared__ float sM[G * C * P];
+  __shared__ float sY[G][C];
+  for (int e = threadIdx.x; e < ng * C * C; e += 256) sM[e / C * P + e % C] = __ldg(M + g0 * C * C + e);
+  if (threadIdx.x < ng) {
+    const int64_t i = ids[g0 + threadIdx.x];
+    const float vx = cx - means[3 * i], vy = cy - means[3 * i + 1], vz = cz - means[3 * i + 2];
+    const float rn = rsqrtf(vx * vx + vy * vy + vz * vz);
+    sh_eval_any<ORDER>(vx * rn, vy * rn, vz * rn, sY[threadIdx.x]);
+  }
+  __syncthreads();
+  float te = 0.f;
+  if (threadIdx.x < ng * C) {
+#pragma unroll
+    for (int b = 0; b < C; ++b) te = fmaf(sM[threadIdx.x * P + b], sY[threadIdx.x / C][b], te);
+  }
+  return te;
+}
+
+// Colours of the glossy splats, a few threads per splat.
 template <int ORDER>
 __global__ void __launch_bounds__(kRelightThreads) k_relight_glossy(int64_t n, int64_t n_glossy,
                                                                     const int32_t* __restrict__ ids,
@@ -58,40 +89,27 @@ __global__ void __launch_bounds__(kRelightThreads) k_relight_glossy(int64_t n, i
                                                                     const float* __restrict__ albedo,
                                                                     const float* __restrict__ L, int k,
                                                                     float* __restrict__ colors) {
-  constexpr int C = (ORDER + 1) * (ORDER + 1);
-  extern __shared__ float sL[];
-  for (int e = threadIdx.x; e < k * 3 * C; e += blockDim.x) sL[e] = L[e];
+  constexpr int C = (ORDER + 1) * (ORDER + 1), P = C | 1, G = glossy_group(C), kPer = kRelightThreads / G;
+  extern __shared__ float sL[];  // [k][3][P]
+  __shared__ float sT[G][C];
+  const int64_t g0 = (int64_t)blockIdx.x * G;
+  const int ng = (int)min((int64_t)G, n_glossy - g0);
+  for (int e = threadIdx.x; e < k * 3 * C; e += kRelightThreads) sL[e / C * P + e % C] = L[e];
+  const float t = glossy_teff<ORDER>(g0, ng, ids, M, means, cam[0], cam[1], cam[2]);
+  if (threadIdx.x < ng * C) sT[threadIdx.x / C][threadIdx.x % C] = t;
   __syncthreads();
-  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (g >= n_glossy) return;
-  const int64_t i = ids[g];
-  float vx = cam[0] - means[3 * i], vy = cam[1] - means[3 * i + 1], vz = cam[2] - means[3 * i + 2];
-  float rn = rsqrtf(vx * vx + vy * vy + vz * vz);
-  float Y[C];
-  sh_eval_any<ORDER>(vx * rn, vy * rn, vz * rn, Y);
+  const int g = threadIdx.x / kPer;
+  if (g >= ng) return;
+  const int64_t i = ids[g0 + g];
   float te[C];
 #pragma unroll
-  for (int a = 0; a < C; ++a) {
-    float acc = 0.f;
+  for (int m = 0; m < C; ++m) te[m] = sT[g][m];
+  for (int e = threadIdx.x % kPer; e < 3 * k; e += kPer) {
+    const int l = e / 3, c = e % 3;
+    float d = 0.f;
 #pragma unroll
-    for (int b = 0; b < C; ++b) acc = fmaf(__ldg(M + (g * C + a) * C + b), Y[b], acc);
-    te[a] = acc;
-  }
-  const float r0 = albedo[3 * i] * (1.0f / kPi), r1 = albedo[3 * i + 1] * (1.0f / kPi),
-              r2 = albedo[3 * i + 2] * (1.0f / kPi);
-  for (int l = 0; l < k; ++l) {
-    const float* Ll = sL + l * 3 * C;
-    float d0 = 0.f, d1 = 0.f, d2 = 0.f;
-#pragma unroll
-    for (int m = 0; m < C; ++m) {
-      d0 = fmaf(te[m], Ll[m], d0);
-      d1 = fmaf(te[m], Ll[C + m], d1);
-      d2 = fmaf(te[m], Ll[2 * C + m], d2);
-    }
-    float* out = colors + ((int64_t)l * n + i) * 3;
-    out[0] = r0 * d0;
-    out[1] = r1 * d1;
-    out[2] = r2 * d2;
+    for (int m = 0; m < C; ++m) d = fmaf(te[m], sL[e * P + m], d);
+    colors[((int64_t)l * n + i) * 3 + c] = albedo[3 * i + c] * (1.0f / kPi) * d;
   }
 }
 
@@ -126,9 +144,9 @@ static void launch_relight_glossy(int64_t n, int64_t n_glossy, const int32_t* id
                                   const float* cam, const float* albedo, const float* L, int k, float* colors,
                                   cudaStream_t stream) {
   constexpr int C = (ORDER + 1) * (ORDER + 1);
-  const size_t smem = sizeof(float) * k * 3 * C;
-  cudaFuncSetAttribute(k_relight_glossy<ORDER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  const unsigned grid = (unsigned)((n_glossy + kRelightThreads - 1) / kRelightThreads);
+  const size_t smem = sizeof(float) * k * 3 * (C | 1);
+  if (smem > 4096) cudaFuncSetAttribute(k_relight_glossy<ORDER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const unsigned grid = (unsigned)((n_glossy + glossy_group(C) - 1) / glossy_group(C));
   k_relight_glossy<ORDER><<<grid, kRelightThreads, smem, counted(stream)>>>(n, n_glossy, ids, M, means, cam, albedo, L, k,
                                                                             colors);
 }
@@ -192,11 +210,6 @@ int relight(int64_t n, int32_t order, const float* T, int32_t t_channels, const 
 // The composite is linear in the splat colours: with colours (rho_i/pi) (T_i . L_l) every
 // light's image is sum_m TI[m,c,p] L[l,c,m] + bg[c] final_T[p], TI the composite of the
 // features F[m,i,c] = (rho_i[c]/pi) T_i[c][m] (glossy splats: t_eff = M_i Y(v_i), Eq. 41).
-// Splats of a k_glossy_features block: a thread per coefficient, at most 40 KB of matrices.
-constexpr int glossy_group(int C) {
-  return (256 / C) * C * (C | 1) <= 10240 ? 256 / C : 10240 / (C * (C | 1));
-}
-
 // F is laid out in rows of render_rows_floats(C), F[m,i,c] at i's 3 m + c, as the composite reads them.
 template <int C, int TCH>
 __global__ void __launch_bounds__(256) k_transfer_features(int64_t n, const float* __restrict__ T,
@@ -215,35 +228,20 @@ __global__ void __launch_bounds__(256) k_transfer_features(int64_t n, const floa
   F[at] = make_float4(f[0], f[1], f[2], f[3]);
 }
 
-// The rows of the glossy splats. A block stages the matrices of a few splats in shared memory (coalesced, at
-// an odd row stride) and takes one coefficient per thread: a thread per splat reading its own kilobyte took 283 us
-// for 300k splats at order 3 (the bytes alone take 70).
+// The rows of the glossy splats.
 template <int ORDER>
 __global__ void __launch_bounds__(256) k_glossy_features(int64_t n_glossy, const int32_t* __restrict__ ids,
                                                          const float* __restrict__ M, const float* __restrict__ means,
                                                          float cx, float cy, float cz,
                                                          const float* __restrict__ albedo, float* __restrict__ F) {
-  constexpr int C = (ORDER + 1) * (ORDER + 1), P = C | 1, G = glossy_group(C), RS = (3 * C + 3) / 4 * 4;
-  __shared__ float sM[G * C * P];
-  __shared__ float sY[G][C];
+  constexpr int C = (ORDER + 1) * (ORDER + 1), G = glossy_group(C), RS = (3 * C + 3) / 4 * 4;
   const int64_t g0 = (int64_t)blockIdx.x * G;
   const int ng = (int)min((int64_t)G, n_glossy - g0);
-  for (int e = threadIdx.x; e < ng * C * C; e += 256) sM[e / C * P + e % C] = __ldg(M + g0 * C * C + e);
-  if (threadIdx.x < ng) {
-    const int64_t i = ids[g0 + threadIdx.x];
-    const float vx = cx - means[3 * i], vy = cy - means[3 * i + 1], vz = cz - means[3 * i + 2];
-    const float rn = rsqrtf(vx * vx + vy * vy + vz * vz);
-    sh_eval_any<ORDER>(vx * rn, vy * rn, vz * rn, sY[threadIdx.x]);
-  }
-  __syncthreads();
+  const float te = glossy_teff<ORDER>(g0, ng, ids, M, means, cx, cy, cz);
   if (threadIdx.x >= ng * C) return;
-  const int g = threadIdx.x / C, a = threadIdx.x % C;
-  const int64_t i = ids[g0 + g];
-  float te = 0.f;
+  const int64_t i = ids[g0 + threadIdx.x / C];
 #pragma unroll
-  for (int b = 0; b < C; ++b) te = fmaf(sM[threadIdx.x * P + b], sY[g][b], te);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) F[i * RS + 3 * a + c] = __ldg(albedo + 3 * i + c) * (1.0f / kPi) * te;
+  for (int c = 0; c < 3; ++c) F[i * RS + 3 * (threadIdx.x % C) + c] = __ldg(albedo + 3 * i + c) * (1.0f / kPi) * te;
 }
 
 // FP32 form: one thread per pixel, the lights in shared memory.
