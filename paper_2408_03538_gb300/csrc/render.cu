@@ -16,6 +16,11 @@ namespace prtgs {
 
 constexpr int kTile = 16;
 constexpr int kTileThreads = kTile * kTile;
+// Blocks of a tile's eight warps: its warps end at different times, and a block keeps its place until the last
+// has. Composite of 300k splats at 1080p, forward and backward, at 1, 2, 4 and 8: 261, 235, 236, 242 and 470, 459, 469,
+// 474 us; of 8 scenes x 4 lights 658, 589, 598, 607 and 1,394, 1,325, 1,273, 1,509.
+constexpr int kSplit = 2;
+constexpr int kCompThreads = kTileThreads / kSplit;
 constexpr float kNear = 0.2f;
 constexpr float kDilation = 0.3f;
 constexpr float kAlphaMax = 0.99f;
@@ -387,18 +392,18 @@ __device__ __forceinline__ void stage_rows(float (*col)[color_floats(KG)], const
 // pixels are opaque. Only splats that add nothing are dropped, so the results are those of the whole list. Bound
 // by issue slots. (Staging the whole list by block and evaluating every splat at every pixel took 485 us for 300k
 // splats at full HD, 875 us for the geometry maps of 300k surface splats and 2,320 us for the 48 channels of a million;
-// this takes 300, 392 and 1,168 us.)
+// this takes 221, 391 and 1,130 us.) The blocks per SM are what the registers of a group allow (a spill of 12 bytes in two forms).
 template <int KG, class V>
-__global__ void __launch_bounds__(kTileThreads, KG <= 8 ? 3 : 2) k_composite(
+__global__ void __launch_bounds__(kCompThreads, (KG <= 2 ? 5 : KG <= 4 ? 4 : KG <= 8 ? 3 : 2) * kSplit) k_composite(
     V v, const uint32_t* __restrict__ ranges, const int32_t* __restrict__ ids, const float* __restrict__ mean2d,
     const float4* __restrict__ conic_op, const float* __restrict__ colors, int64_t n, int k,
     const float* __restrict__ bg, float* __restrict__ image, float* __restrict__ final_T,
     int32_t* __restrict__ n_contrib) {
   constexpr int CF = color_floats(KG);
   extern __shared__ float4 fwd_smem[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  FwdWarp<KG>& sm = reinterpret_cast<FwdWarp<KG>*>(fwd_smem)[warp];
-  const int gtile = blockIdx.x;  // scene-major tile index
+  const int lane = threadIdx.x & 31, warp = (blockIdx.x % kSplit) * (8 / kSplit) + (threadIdx.x >> 5);
+  FwdWarp<KG>& sm = reinterpret_cast<FwdWarp<KG>*>(fwd_smem)[threadIdx.x >> 5];
+  const int gtile = blockIdx.x / kSplit;  // scene-major tile index
   const Cam& c = v.cam(0);
   const int per_scene = c.gx * c.gy;
   const int b = gtile / per_scene, tile = gtile % per_scene;
@@ -493,9 +498,9 @@ __global__ void __launch_bounds__(kTileThreads, KG <= 8 ? 3 : 2) k_composite(
 template <int KG, class V>
 static void launch_composite_t(const V& v, unsigned tiles, const prtgs_render_state* st, const float* colors, int64_t n,
                                int k, const float* bg, float* image, cudaStream_t stream) {
-  const size_t smem = sizeof(FwdWarp<KG>) * (kTileThreads / 32);
+  const size_t smem = sizeof(FwdWarp<KG>) * (kCompThreads / 32);
   if (smem > 48 * 1024) cudaFuncSetAttribute(k_composite<KG, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_composite<KG, V><<<dim3(tiles, (unsigned)((k + KG - 1) / KG)), kTileThreads, smem, counted(stream)>>>(
+  k_composite<KG, V><<<dim3(tiles * kSplit, (unsigned)((k + KG - 1) / KG)), kCompThreads, smem, counted(stream)>>>(
       v, st->ranges, st->pair_ids, st->mean2d, reinterpret_cast<const float4*>(st->conic_op), colors, n, k, bg, image,
       st->final_T, st->n_contrib);
 }
@@ -544,7 +549,7 @@ static int render_views(const prtgs_gaussians* g, const float* colors, int32_t k
     PRTGS_CHECK_LAUNCH();
     // The (tile, depth) order as the splats' depth order followed by a stable sort of the pairs by tile: the
     // 32 depth bits are sorted once per splat instead of once per pair (25 M pairs of 300k splats: six
-    // passes over 12-byte pairs, 1.57 ms, became two over 8-byte ones and four short ones, 0.60 ms).
+    // passes over 12-byte pairs, 1.57 ms, became two over 8-byte ones and four short ones, 0.52 ms).
     int rc = radix_sort_pairs(dkey[0], nullptr, dkey[2], by_depth, dkey[1], by_depth_y, n, nullptr, 0, 32, sort_ws, stream);
     if (rc != PRTGS_OK) return rc;
     const uint32_t cap = (uint32_t)(st->max_pairs < 0xffffffffll ? st->max_pairs : 0xffffffffll);
@@ -647,20 +652,20 @@ __device__ __forceinline__ void red_add4(float* p, float a, float b, float c, fl
 // (splat, half of the pixels): the moments of g and the colour sums of w are plain sums in registers, and a
 // splat's sums leave the warp as a few vector reductions. (Reducing every value of every splat over the warp
 // by shuffles and adding it to shared memory by one lane was 5.47 ms of the 8.4 ms of a 300k-splat full-HD
-// frame; this takes 0.56 ms. 8 scenes x 4 lights at 720p: 14.8 -> 1.64 ms.) Bound by issue slots.
+// frame; this takes 0.46 ms. 8 scenes x 4 lights at 720p: 14.8 -> 1.33 ms.) Bound by issue slots.
 // The colours enter dL/dalpha through the scalar c . dL/dpixel only, whose blended remainder follows the same
 // recursion as the colours'.
 template <int KG, class V>
-__global__ void __launch_bounds__(kTileThreads) k_composite_bwd(
+__global__ void __launch_bounds__(kCompThreads) k_composite_bwd(
     V v, const uint32_t* __restrict__ ranges, const int32_t* __restrict__ ids, const float* __restrict__ mean2d,
     const float4* __restrict__ conic_op, const float* __restrict__ colors, int64_t n, int k,
     const float* __restrict__ bg, const float* __restrict__ final_T, const int32_t* __restrict__ n_contrib,
     const float* __restrict__ dimage, float* __restrict__ acc, int stride) {
   constexpr int CF = color_floats(KG);
   extern __shared__ float4 bwd_smem[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  BwdWarp<KG>& sm = reinterpret_cast<BwdWarp<KG>*>(bwd_smem)[warp];
-  const int gtile = blockIdx.x;  // scene-major tile index
+  const int lane = threadIdx.x & 31, warp = (blockIdx.x % kSplit) * (8 / kSplit) + (threadIdx.x >> 5);
+  BwdWarp<KG>& sm = reinterpret_cast<BwdWarp<KG>*>(bwd_smem)[threadIdx.x >> 5];
+  const int gtile = blockIdx.x / kSplit;  // scene-major tile index
   const Cam& c = v.cam(0);
   const int per_scene = c.gx * c.gy;
   const int b = gtile / per_scene, tile = gtile % per_scene;
@@ -998,9 +1003,9 @@ size_t render_backward_workspace(int64_t n, int32_t k) {
 template <int KG, class V>
 static void launch_composite_bwd(dim3 grid, const V& v, const prtgs_render_state* st, const float* colors, int64_t n, int k,
                                  const float* bg, const float* dimage, float* acc, int stride, cudaStream_t stream) {
-  const size_t smem = sizeof(BwdWarp<KG>) * (kTileThreads / 32);
+  const size_t smem = sizeof(BwdWarp<KG>) * (kCompThreads / 32);
   cudaFuncSetAttribute(k_composite_bwd<KG, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_composite_bwd<KG, V><<<grid, kTileThreads, smem, counted(stream)>>>(
+  k_composite_bwd<KG, V><<<grid, kCompThreads, smem, counted(stream)>>>(
       v, st->ranges, st->pair_ids, st->mean2d, reinterpret_cast<const float4*>(st->conic_op), colors, n, k, bg,
       st->final_T, st->n_contrib, dimage, acc, stride);
 }
@@ -1018,7 +1023,7 @@ static int render_backward_views(const prtgs_gaussians* g, const float* colors, 
   float* acc = cv.take<float>((size_t)stride * n);
   cudaMemsetAsync(acc, 0, sizeof(float) * stride * n, stream);
   // every light's colour sets in groups of up to 8 (shared memory bound)
-  dim3 grid((unsigned)tiles, (unsigned)((k + kg - 1) / kg));
+  dim3 grid((unsigned)tiles * kSplit, (unsigned)((k + kg - 1) / kg));
   if (kg == 1) {
     launch_composite_bwd<1>(grid, v, st, colors, n, k, bg, dimage, acc, stride, stream);
   } else {
