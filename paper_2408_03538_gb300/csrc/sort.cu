@@ -179,6 +179,8 @@ __device__ __forceinline__ uint64_t wide_key(K k, float low) {
   return ((uint64_t)k << 32) | __float_as_uint(low);
 }
 
+// Digit counts of a tile. Its keys are all loaded before the first count: loads between the shared-memory atomics wait
+// for them (25 M keys in two passes 140 us, 61 like this; four private histograms per block change nothing).
 // hist: [tile][256] when self (the scatter blocks sum it), else [256][tile] for one exclusive scan.
 template <class K>
 __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const K* __restrict__ keys, int64_t capacity,
@@ -189,11 +191,15 @@ __global__ void __launch_bounds__(kSortThreads) k_radix_hist(const K* __restrict
   __syncthreads();
   const int64_t n = sort_count(d_count, capacity);
   const int64_t base = (int64_t)blockIdx.x * SortShape<K>::kTile;
+  K key[SortShape<K>::kItems];
 #pragma unroll
   for (int r = 0; r < SortShape<K>::kItems; ++r) {
     const int64_t i = base + r * kSortThreads + threadIdx.x;
-    if (i < n) atomicAdd(&h[(unsigned)(keys[i] >> shift) & mask], 1u);
+    key[r] = i < n ? keys[i] : (K)0;
   }
+#pragma unroll
+  for (int r = 0; r < SortShape<K>::kItems; ++r)
+    if (base + r * kSortThreads + threadIdx.x < n) atomicAdd(&h[(unsigned)(key[r] >> shift) & mask], 1u);
   __syncthreads();
   if (self) hist[(int64_t)blockIdx.x * 256 + threadIdx.x] = h[threadIdx.x];
   else if (threadIdx.x <= mask) hist[(int64_t)threadIdx.x * n_tiles + blockIdx.x] = h[threadIdx.x];
