@@ -9,6 +9,7 @@
 // Backward: k_composite_bwd walks each pixel's list back to front from its last contributor and sums
 // every splat's moments and colour gradients over a warp's pixels before a few vector reductions;
 // k_preprocess_bwd maps the sums to opacities, colours, means, scales and rotations.
+#include "blend.cuh"
 #include "common.cuh"
 #include "internal.h"
 
@@ -86,9 +87,6 @@ __device__ __forceinline__ int64_t color_at(const V& v, int b, int64_t g, int l,
   const int64_t o = v.first(b);
   return 3 * (int64_t)k * o + ((int64_t)l * v.count(b, n) + (g - o)) * 3;
 }
-
-// Floats of k colour sets, on a 16-byte boundary.
-__host__ __device__ constexpr int color_floats(int kg) { return (3 * kg + 3) / 4 * 4; }
 
 size_t render_state_bytes(int64_t n, int32_t width, int32_t height, int64_t max_pairs) {
   return render_state_bytes_batched(n, 1, width, height, max_pairs);
@@ -399,7 +397,6 @@ __global__ void __launch_bounds__(kCompThreads, (KG <= 2 ? 5 : KG <= 4 ? 4 : KG 
     const float4* __restrict__ conic_op, const float* __restrict__ colors, int64_t n, int k,
     const float* __restrict__ bg, float* __restrict__ image, float* __restrict__ final_T,
     int32_t* __restrict__ n_contrib) {
-  constexpr int CF = color_floats(KG);
   extern __shared__ float4 fwd_smem[];
   const int lane = threadIdx.x & 31, warp = (blockIdx.x % kSplit) * (8 / kSplit) + (threadIdx.x >> 5);
   FwdWarp<KG>& sm = reinterpret_cast<FwdWarp<KG>*>(fwd_smem)[threadIdx.x >> 5];
@@ -468,14 +465,7 @@ __global__ void __launch_bounds__(kCompThreads, (KG <= 2 ? 5 : KG <= 4 ? 4 : KG 
         continue;
       }
       const float wgt = alpha * T;
-#pragma unroll
-      for (int e = 0; e < CF; e += 4) {
-        const float4 cl = *reinterpret_cast<const float4*>(&sm.col[j][e]);
-        acc[e] = fmaf(cl.x, wgt, acc[e]);
-        acc[e + 1] = fmaf(cl.y, wgt, acc[e + 1]);
-        acc[e + 2] = fmaf(cl.z, wgt, acc[e + 2]);
-        if (e + 3 < 3 * KG) acc[e + 3] = fmaf(cl.w, wgt, acc[e + 3]);
-      }
+      blend_row<KG>(acc, sm.col[j], wgt);
       T = test_T;
       last = __float_as_int(q.w) + 1;
     }
