@@ -785,10 +785,9 @@ __global__ void __launch_bounds__(kCompThreads) k_composite_bwd(
       if (i < cnt) {
         float* out = acc + (int64_t)__float_as_int(sm.xy[c0 + i].z) * stride;
         if (half == 0) {
-          if (m0 != 0.f || mx != 0.f || my != 0.f) {
-            red_add4(out, m0, mx, my, mxx);
-            red_add4(out + 4, mxy, myy, 0.f, 0.f);
-          }
+          // g has both signs: the second moments can be all that is left
+          if (m0 != 0.f || mx != 0.f || my != 0.f || mxx != 0.f) red_add4(out, m0, mx, my, mxx);
+          if (mxy != 0.f || myy != 0.f) red_add4(out + 4, mxy, myy, 0.f, 0.f);
         } else {
           out += kMoments + CF * (int)blockIdx.y;
 #pragma unroll
