@@ -1237,7 +1237,9 @@ __global__ void __launch_bounds__(128) k_bwd_finish(int64_t n, const float4* __r
   const float4 a0 = acc[3 * i], a1 = acc[3 * i + 1], a2 = acc[3 * i + 2], go = rayacc[2 * i], gn = rayacc[2 * i + 1];
   const float M[3][3] = {{a1.x, a1.y, a1.z}, {a1.y, a1.w, a2.x}, {a1.z, a2.x, a2.y}};
   float gs[3] = {0.f, 0.f, 0.f}, gm[3] = {0.f, 0.f, 0.f}, gq[4] = {0.f, 0.f, 0.f, 0.f};
-  if (a0.x != 0.f || a0.y != 0.f || a0.z != 0.f || a0.w != 0.f || a1.x != 0.f || a1.w != 0.f || a2.y != 0.f) {
+  // (the sums have both signs: the mixed second moments can be all that is left)
+  if (a0.x != 0.f || a0.y != 0.f || a0.z != 0.f || a0.w != 0.f || a1.x != 0.f || a1.y != 0.f || a1.z != 0.f ||
+      a1.w != 0.f || a2.x != 0.f || a2.y != 0.f) {
     const float4 q1 = __ldg(recs + 4 * i + 1), q2 = __ldg(recs + 4 * i + 2), q3 = __ldg(recs + 4 * i + 3);
     const float A[3][3] = {{q1.x, q1.y, q1.z}, {q1.w, q2.x, q2.y}, {q2.z, q2.w, q3.x}};
     float gR[3][3], Rs[3][3], inv_s[3];  // Rs[l][j] = R_jl s_l = A_lj s_l^2

@@ -1,5 +1,6 @@
 """Gradients whose lower moments cancel exactly, so that only the second moments are left: a splat seen by four
-pixels at its corners whose image gradients alternate in sign turns, and neither moves nor grows.
+pixels at its corners whose image gradients alternate in sign turns, and neither moves nor grows; so does an
+occluder met by four parallel rays whose gradients alternate.
 
 Against FP64 autograd of the oracle, 2e-3 norm-wise (the bar of test_gpu_render.py).
 """
@@ -7,7 +8,8 @@ import numpy as np
 import pytest
 import torch
 
-from oracle import render as OR
+import oracle
+from oracle import render as OR, transfer_torch as TT
 from paper_2408_03538_gb300 import api, scenes as S
 
 pytestmark = pytest.mark.gpu
@@ -41,3 +43,33 @@ def test_render_backward_keeps_second_moments(k):
                               ps[2])[0]
     assert float(ref.norm()) > 0.1 * k
     assert float((dq - ref).norm()) <= 2e-3 * float(ref.norm())
+
+
+def quadrupole_rays():
+    """An occluder, wider than deep, and four receivers below its corners that look up along z: the gradients of their
+    first coefficients alternate in sign."""
+    sc = S.isotropic_scene(5, 4)
+    sc.means[0] = 0.0
+    sc.means[1:] = [(x, y, -2.0) for x in (-0.25, 0.25) for y in (-0.125, 0.125)]
+    sc.scales[0] = (0.5, 0.25, 0.5)
+    sc.scales[1:] = 0.03125
+    sc.quats[:] = (1.0, 0.0, 0.0, 0.0)
+    sc.opacity[:] = (0.5, 0.25, 0.25, 0.25, 0.25)
+    sc.normals[0] = (0.0, 0.0, -1.0)
+    sc.normals[1:] = (0.0, 0.0, 1.0)
+    dP = np.zeros((5, 4), np.float32)
+    dP[1:, 0] = (1.0, -1.0, -1.0, 1.0)
+    return sc, np.array([[0.0, 0.0, 1.0]], np.float32), dP
+
+
+def test_transfer_backward_keeps_second_moments():
+    sc, dirs, dP = quadrupole_rays()
+    g = api.GaussianTensors.from_scene(sc)
+    out = api.precompute_transfer_backward(g, api.build_bvh(g), torch.from_numpy(dirs).cuda(), 1,
+                                           torch.from_numpy(dP).cuda(), t_min=0.0)
+    ps = [torch.tensor(np.asarray(getattr(sc, f), np.float64), requires_grad=True)
+          for f in ("means", "scales", "quats", "opacity", "normals")]
+    P = TT.transfer_P(*ps, dirs, oracle.sh(1, dirs))
+    ref = torch.autograd.grad((P * torch.as_tensor(dP.astype(np.float64))).sum(), ps)[2]
+    assert float(ref.norm()) > 0.1
+    assert float((out["d_quats"].cpu().double() - ref).norm()) <= 2e-3 * float(ref.norm())
