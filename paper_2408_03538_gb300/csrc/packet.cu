@@ -989,6 +989,7 @@ struct HitListVis {
 };
 
 constexpr int kBwdBlocks = 4;      // per SM
+constexpr int kBwdMaxBlocks = 152 * kBwdBlocks;  // of a launch: the workspace depends on the arguments, not on a device
 constexpr int kBwdList = 2048;     // hit leaves of a packet kept at a time
 constexpr int kBwdBatch = 5;       // leaves whose six moments are summed together (30 lanes, one sum each)
 constexpr int kBwdRow = 36;        // 32 lanes' values and padding: 16-byte reads of 30 rows without conflicts
@@ -1279,9 +1280,16 @@ static int64_t bwd_batch(int64_t n, int S) {
   return b < n ? b : n;
 }
 
-size_t packet_bwd_workspace(int64_t n, int S, int sms) {
+// Blocks of a launch at most, each with its warps' lists: a warp per packet is enough.
+static int64_t bwd_blocks(int64_t n, int S) {
+  const int64_t items = kBwdWindow / 32 * ((bwd_batch(n, S) + kBwdWindow - 1) / kBwdWindow) * S;
+  const int64_t b = (items + kPacketWarps - 1) / kPacketWarps;
+  return b < 1 ? 1 : (b < kBwdMaxBlocks ? b : kBwdMaxBlocks);
+}
+
+size_t packet_bwd_workspace(int64_t n, int S) {
   return 2 * align_up(sizeof(float) * (size_t)bwd_batch(n, S) * S) + align_up(sizeof(float) * 20 * (size_t)n) +
-         align_up(sizeof(int) * (size_t)sms * kBwdBlocks * kPacketWarps * kBwdList);
+         align_up(sizeof(int) * (size_t)bwd_blocks(n, S) * kPacketWarps * kBwdList);
 }
 
 int launch_packet_bwd(TraceArgs a, const float* quats, const float* dP, const float* dV, float* d_means, float* d_scales,
@@ -1291,7 +1299,7 @@ int launch_packet_bwd(TraceArgs a, const float* quats, const float* dP, const fl
   float* G = c.take<float>((size_t)b * a.S);
   float* GV = c.take<float>((size_t)b * a.S);
   float* acc = c.take<float>(20 * (size_t)a.n);  // [n][12], then [n][8] of the receivers
-  int* lists = c.take<int>((size_t)sms * kBwdBlocks * kPacketWarps * kBwdList);
+  int* lists = c.take<int>((size_t)bwd_blocks(a.n, a.S) * kPacketWarps * kBwdList);
   float* rayacc = acc + 12 * a.n;
   cudaMemsetAsync(acc, 0, sizeof(float) * 20 * a.n, stream);
   const size_t smem = (sizeof(PacketSmem) + sizeof(BwdSmem)) * kPacketWarps;
@@ -1299,13 +1307,14 @@ int launch_packet_bwd(TraceArgs a, const float* quats, const float* dP, const fl
   cudaFuncSetAttribute(k_packet_bwd, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_packet_bwd, kPacketThreads, smem);
-  per_sm = per_sm < 1 ? 1 : (per_sm > kBwdBlocks ? kBwdBlocks : per_sm);
+  const int64_t most = bwd_blocks(a.n, a.S), resident = (int64_t)sms * (per_sm < 1 ? 1 : per_sm);
+  const unsigned blocks = (unsigned)(resident < most ? resident : most);
   for (int64_t r0 = 0; r0 < a.n; r0 += b) {
     a.r0 = r0;
     a.r1 = r0 + b < a.n ? r0 + b : a.n;
     cudaMemsetAsync(a.work, 0, sizeof(unsigned int), stream);
     k_ray_grad<<<(unsigned)((a.r1 - a.r0 + 127) / 128), 128, 0, counted(stream)>>>(a, dP, dV, G, GV);
-    k_packet_bwd<<<sms * per_sm, kPacketThreads, smem, counted(stream)>>>(a, G, GV, acc, rayacc, lists);
+    k_packet_bwd<<<blocks, kPacketThreads, smem, counted(stream)>>>(a, G, GV, acc, rayacc, lists);
   }
   k_bwd_finish<<<(unsigned)((a.n + 127) / 128), 128, 0, counted(stream)>>>(
       a.n, a.recs, a.order, quats, reinterpret_cast<const float4*>(acc), reinterpret_cast<const float4*>(rayacc), d_means,

@@ -414,7 +414,7 @@ int precompute_transfer_backward(const prtgs_gaussians* gs, const prtgs_bvh* bvh
 size_t transfer_backward_workspace(int64_t n, const prtgs_transfer_params* p) {
   const int C = sh_count(p->sh_order);
   return align_up(sizeof(unsigned int)) + (C > kMaxC ? align_up(sizeof(float) * (size_t)p->n_dirs * C) : 0) +
-         packet_bwd_workspace(n, p->n_dirs, device_sms());
+         packet_bwd_workspace(n, p->n_dirs);
 }
 
 // ---- self-transfer bounces (Eq. 33; n bounces Eq. 34-35) ----------------------------------------
