@@ -664,6 +664,10 @@ __device__ __forceinline__ void dL_chunk(int64_t i0, int64_t i1, const float* __
   }
 }
 
+// One light per thread (LQ = 1) for one or two lights that take one pass together, else four: at order 6 the threads
+// hold one light's outputs, so that two lights would be two passes (100k Gaussians 270 us a call; four a thread 172).
+static bool dL_single(int C, int k) { return k <= 2 && 3 * C * k <= kRelightThreads; }
+
 template <int C, int TCH, int LQ>
 __global__ void __launch_bounds__(kRelightThreads) k_relight_dL_partial(int64_t n, const float* __restrict__ T,
                                                                         const float* __restrict__ albedo, int k,
@@ -706,7 +710,7 @@ static void launch_relight_bwd(int64_t n, const float* T, int tch, const float* 
     k_relight_bwd_local<C, 3><<<grid, kRelightThreads, smem, counted(stream)>>>(n, T, albedo, L, k, dcol, d_albedo, dT);
   else
     k_relight_bwd_local<C, 1><<<grid, kRelightThreads, smem, counted(stream)>>>(n, T, albedo, L, k, dcol, d_albedo, dT);
-  const auto dl = k <= 2 ? (tch == 3 ? k_relight_dL_partial<C, 3, 1> : k_relight_dL_partial<C, 1, 1>)
+  const auto dl = dL_single(C, k) ? (tch == 3 ? k_relight_dL_partial<C, 3, 1> : k_relight_dL_partial<C, 1, 1>)
                          : (tch == 3 ? k_relight_dL_partial<C, 3, 4> : k_relight_dL_partial<C, 1, 4>);
   dl<<<(unsigned)nb, kRelightThreads, 0, counted(stream)>>>(n, T, albedo, k, dcol, partial);
   int nout = k * 3 * C;
@@ -820,7 +824,7 @@ static void launch_relight_bwd_batched(int64_t n, const float* T, int tch, const
   else
     k_relight_bwd_local_batched<C, 1><<<grid, kRelightThreads, 0, counted(stream)>>>(n, T, albedo, offs, B, L, k, dcol,
                                                                                     d_albedo, dT);
-  const auto dl = k <= 2 ? (tch == 3 ? k_relight_dL_partial_batched<C, 3, 1> : k_relight_dL_partial_batched<C, 1, 1>)
+  const auto dl = dL_single(C, k) ? (tch == 3 ? k_relight_dL_partial_batched<C, 3, 1> : k_relight_dL_partial_batched<C, 1, 1>)
                          : (tch == 3 ? k_relight_dL_partial_batched<C, 3, 4> : k_relight_dL_partial_batched<C, 1, 4>);
   dl<<<pgrid, kRelightThreads, 0, counted(stream)>>>(offs, T, albedo, k, dcol, partial);
   const int nout = k * 3 * C;
