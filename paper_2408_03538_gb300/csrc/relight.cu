@@ -113,6 +113,64 @@ __global__ void __launch_bounds__(kRelightThreads) k_relight_glossy(int64_t n, i
   }
 }
 
+// The same with a thread per splat, which reads its own matrix and goes through the lights with the block's copy.
+template <int ORDER>
+__global__ void __launch_bounds__(kRelightThreads) k_relight_glossy_each(int64_t n, int64_t n_glossy,
+                                                                         const int32_t* __restrict__ ids,
+                                                                         const float* __restrict__ M,
+                                                                         const float* __restrict__ means,
+                                                                         const float* __restrict__ cam,
+                                                                         const float* __restrict__ albedo,
+                                                                         const float* __restrict__ L, int k,
+                                                                         float* __restrict__ colors) {
+  constexpr int C = (ORDER + 1) * (ORDER + 1);
+  extern __shared__ float sL[];
+  for (int e = threadIdx.x; e < k * 3 * C; e += blockDim.x) sL[e] = L[e];
+  __syncthreads();
+  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= n_glossy) return;
+  const int64_t i = ids[g];
+  float vx = cam[0] - means[3 * i], vy = cam[1] - means[3 * i + 1], vz = cam[2] - means[3 * i + 2];
+  float rn = rsqrtf(vx * vx + vy * vy + vz * vz);
+  float Y[C];
+  sh_eval_any<ORDER>(vx * rn, vy * rn, vz * rn, Y);
+  float te[C];
+#pragma unroll
+  for (int a = 0; a < C; ++a) {
+    float acc = 0.f;
+#pragma unroll
+    for (int b = 0; b < C; ++b) acc = fmaf(__ldg(M + (g * C + a) * C + b), Y[b], acc);
+    te[a] = acc;
+  }
+  const float r0 = albedo[3 * i] * (1.0f / kPi), r1 = albedo[3 * i + 1] * (1.0f / kPi),
+              r2 = albedo[3 * i + 2] * (1.0f / kPi);
+  for (int l = 0; l < k; ++l) {
+    const float* Ll = sL + l * 3 * C;
+    float d0 = 0.f, d1 = 0.f, d2 = 0.f;
+#pragma unroll
+    for (int m = 0; m < C; ++m) {
+      d0 = fmaf(te[m], Ll[m], d0);
+      d1 = fmaf(te[m], Ll[C + m], d1);
+      d2 = fmaf(te[m], Ll[2 * C + m], d2);
+    }
+    float* out = colors + ((int64_t)l * n + i) * 3;
+    out[0] = r0 * d0;
+    out[1] = r1 * d1;
+    out[2] = r2 * d2;
+  }
+}
+
+// Whether a thread per splat is the better form for the colours: where there are splats enough for it to fill the
+// GPU and a block of k_relight_glossy pays most for its few splats, each of whose blocks stages all the lights. Glossy
+// part of the call, a block per few splats and a thread per splat: order 6, 10k splats 47 and 137 us (8 lights 51 and
+// 145), 33k 156 and 142 (64 lights 304 and 248), 100k 456 and 418; 256 lights 313 and 465, 1,006 and 469, 3,074 and
+// 1,418. Order 3, 33k splats, 128 lights 78 and 94, 256 lights 163 and 155; 100k 244 and 231, 506 and 404. The other orders
+// keep the block form at every size measured (1k to 300k splats, 1 to 256 lights).
+static bool glossy_each(int order, int64_t n_glossy, int k) {
+  if (order == 6) return n_glossy >= (k > 128 ? 15000 : 30000);
+  return order == 3 && k >= 128 && n_glossy * k >= 8000000;
+}
+
 // Orders 4-6 (25-49 coefficients): one thread per Gaussian, the transfer row and the lights read
 // through the cache instead of held in registers.
 __global__ void __launch_bounds__(kRelightThreads) k_relight_any(int64_t n, int C, int tch, const float* __restrict__ T,
@@ -144,6 +202,15 @@ static void launch_relight_glossy(int64_t n, int64_t n_glossy, const int32_t* id
                                   const float* cam, const float* albedo, const float* L, int k, float* colors,
                                   cudaStream_t stream) {
   constexpr int C = (ORDER + 1) * (ORDER + 1);
+  if constexpr (ORDER == 3 || ORDER == 6) {
+    if (glossy_each(ORDER, n_glossy, k)) {
+      const size_t smem = sizeof(float) * k * 3 * C;
+      cudaFuncSetAttribute(k_relight_glossy_each<ORDER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      k_relight_glossy_each<ORDER><<<(unsigned)((n_glossy + kRelightThreads - 1) / kRelightThreads), kRelightThreads, smem,
+                                     counted(stream)>>>(n, n_glossy, ids, M, means, cam, albedo, L, k, colors);
+      return;
+    }
+  }
   const size_t smem = sizeof(float) * k * 3 * (C | 1);
   if (smem > 4096) cudaFuncSetAttribute(k_relight_glossy<ORDER>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const unsigned grid = (unsigned)((n_glossy + glossy_group(C) - 1) / glossy_group(C));
