@@ -83,10 +83,13 @@ constexpr int tt_row(int C) { return ((C + 3) / 4 | 1) * 4; }
 
 // Bound by issue slots (the BRDF) and the latency of V: a row's chunks are loaded four ahead, and a term reads its
 // SH row in 16-byte words. 300k receivers, order 3, 256 directions: 380 us a chunk at a time and a word per
-// coefficient, 363 us like this; the backward 397 and 371 us.
+// coefficient, 363 us like this; the backward 397 and 371 us. At order 1, whose terms are short and whose blocks fill
+// the SM, V is read where the direction is above the horizon instead: 100k receivers 108 us and, read ahead, 117 (the
+// backward 116 and 124); at order 2 reading ahead is the faster form from about a thousand directions (466 and 502).
 template <int ORDER, bool BACKWARD>
 __global__ void __launch_bounds__(kTTThreads, ORDER <= 3 ? 4 : 2) k_training_transfer(TTArgs a) {
   constexpr int C = (ORDER + 1) * (ORDER + 1), R = tt_row(C);
+  constexpr bool AHEAD = ORDER >= 2;
   extern __shared__ float4 tt_smem[];
   const int S = a.S;
   float* sY = reinterpret_cast<float*>(tt_smem);  // [S][R]
@@ -159,19 +162,19 @@ __global__ void __launch_bounds__(kTTThreads, ORDER <= 3 ? 4 : 2) k_training_tra
       int qn = 0;  // warp-uniform queue length, < 32 between chunks
       float ahead[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) ahead[j] = lane + 32 * j < S ? __ldg(Vi + lane + 32 * j) : 0.0f;
+      for (int j = 0; j < 4; ++j) ahead[j] = AHEAD && lane + 32 * j < S ? __ldg(Vi + lane + 32 * j) : 0.0f;
       for (int base = 0; base < S; base += 32) {
         const int s = base + lane;
         const float vs = ahead[0];
         ahead[0] = ahead[1];
         ahead[1] = ahead[2];
         ahead[2] = ahead[3];
-        ahead[3] = s + 128 < S ? __ldg(Vi + s + 128) : 0.0f;
+        ahead[3] = AHEAD && s + 128 < S ? __ldg(Vi + s + 128) : 0.0f;
         float cv = 0.0f;
         if (s < S) {
           const float* d = sdir + 3 * s;
           const float c = fmaf(nx, d[0], fmaf(ny, d[1], nz * d[2]));
-          if (c > 0.0f) cv = c * vs;
+          if (c > 0.0f) cv = c * (AHEAD ? vs : __ldg(Vi + s));
         }
         const bool live = cv != 0.0f;  // a NaN visibility stays live and reaches the output
         const unsigned mask = __ballot_sync(0xffffffffu, live);
