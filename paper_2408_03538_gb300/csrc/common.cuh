@@ -143,6 +143,12 @@ __device__ __forceinline__ void sh_eval_any(float x, float y, float z, float* Y)
   else sh_eval_rec<ORDER>(x, y, z, Y);
 }
 
+// p[0..3] += (a, b, c, d) in one reduction (p on a 16-byte boundary).
+__device__ __forceinline__ void red_add4(float* p, float a, float b, float c, float d) {
+  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d)
+               : "memory");
+}
+
 // ---- error-free transformations (Knuth TwoSum) for compensated sums
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = __fadd_rn(a, b);

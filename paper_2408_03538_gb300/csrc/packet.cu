@@ -999,11 +999,6 @@ struct BwdSmem {
   float sum[32][8];
 };
 
-__device__ __forceinline__ void red_add4(float* p, float a, float b, float c, float d) {
-  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d)
-               : "memory");
-}
-
 // G, GV: [S][batch] gradients of each ray's c V (for the normal) and of its V; acc: [n][12] sums per
 // Gaussian, ray: [n][8] (d o, d n) per receiver, both in sorted order; lists: kBwdList ints per warp.
 __global__ void __launch_bounds__(kPacketThreads, kBwdBlocks)

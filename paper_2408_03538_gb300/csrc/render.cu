@@ -500,8 +500,10 @@ static void launch_composite_t(const V& v, unsigned tiles, const prtgs_render_st
 template <class V>
 static void launch_composite(const V& v, unsigned tiles, const prtgs_render_state* st, const float* colors, int64_t n, int k,
                              const float* bg, float* image, cudaStream_t stream) {
-  if (k <= 1) launch_composite_t<1>(v, tiles, st, colors, n, k, bg, image, stream);
-  else if (k <= 2) launch_composite_t<2>(v, tiles, st, colors, n, k, bg, image, stream);
+  if constexpr (!V::kRows) {  // rows hold two sets or more
+    if (k <= 1) return launch_composite_t<1>(v, tiles, st, colors, n, k, bg, image, stream);
+  }
+  if (k <= 2) launch_composite_t<2>(v, tiles, st, colors, n, k, bg, image, stream);
   else if (k <= 4) launch_composite_t<4>(v, tiles, st, colors, n, k, bg, image, stream);
   else if ((k + 7) / 8 % 2 == 0) launch_composite_t<16>(v, tiles, st, colors, n, k, bg, image, stream);
   else launch_composite_t<8>(v, tiles, st, colors, n, k, bg, image, stream);
@@ -629,11 +631,6 @@ struct BwdWarp {
   float dpix[32][color_floats(KG)];    // dL/dimage of the warp's pixels
   float g[kBwdChunk][33], w[kBwdChunk][33];
 };
-
-__device__ __forceinline__ void red_add4(float* p, float a, float b, float c, float d) {
-  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d)
-               : "memory");
-}
 
 // One warp per 8 x 4 pixels of a tile, on its own (no block barrier): it takes its tile's list from the
 // last contributor of its pixels backwards, 32 splats at a time, drops those that cannot reach its pixels
