@@ -162,11 +162,11 @@ int prtgs_build_bvh(const prtgs_gaussians* g, prtgs_bvh* bvh, int32_t* status, v
  *   walk            tuning: 0 = warp packets (default: the rays that 32 receivers adjacent in
  *                   Morton order cast along one direction walk the BVH together), 1 = one ray
  *                   per lane (the plain per-ray walk); both give the same results
- *   packet_dirs     tuning: directions per work item of the packet walk (a work item is a
- *                   window of 64 receivers adjacent in Morton order x packet_dirs directions;
- *                   for each direction the window's receivers that face it are compacted into
- *                   packets of 32 lanes), 1..64; 0 = the default (1, see prtgs_autotune); the
- *                   results do not depend on it
+ *   packet_dirs     tuning: directions per work item of the packet walk (for each direction the
+ *                   receivers of a window of 64 adjacent in Morton order that face it are
+ *                   compacted into two packets of 32 lanes at most; a work item is one of the
+ *                   two x packet_dirs directions), 1..64; 0 = the default (1, see
+ *                   prtgs_autotune); the results do not depend on it
  *   stats           optional device uint64[10] that the call ADDS its work counters to:
  *                   BVH node visits of the visibility walks, node visits of the index-matrix
  *                   search, leaf tests, ray-Gaussian hits, search rounds, traced rays, rays
@@ -188,6 +188,11 @@ typedef struct prtgs_transfer_params {
   int32_t packet_dirs;
 } prtgs_transfer_params;
 
+/*
+ * Bytes of workspace: 4 a ray for at most 2^26 rays at a time; with PRTGS_BOUNCE instead 36 a ray for at
+ * most 2^25 (1.2 GB from 131,072 Gaussians at 256 directions: the search records of every packet), with
+ * PRTGS_GLOSSY also 4 S a glossy Gaussian; plus the buffers of further bounces (n_bounces above).
+ */
 size_t prtgs_transfer_workspace_size(int64_t n, int64_t n_glossy, const prtgs_transfer_params* p);
 
 /*
@@ -220,9 +225,12 @@ int prtgs_precompute_transfer(const prtgs_gaussians* g, const prtgs_bvh* bvh, co
 /*
  * Transfer backward: gradients of a loss through P (the shadowed diffuse transfer of Eq. 29
  * projected by Eq. 9) to the Gaussians, for optimising geometry against relit images
- * (Sec. 4.4). Each traced ray is walked again for V_is, as part of its packet, and pushes
- * dL/dalpha_j = -g V_is / (1 - alpha_j) to every occluder up to the same early exit; a packet's
- * hit leaves are listed while it is in flight, no per-ray hit list is stored. The hit set (t* > 0, D^2 <= 9) and the
+ * (Sec. 4.4). Each traced ray is walked again for V_is, as part of a packet, and pushes
+ * dL/dalpha_j = -g V_is / (1 - alpha_j) to its occluders up to its early exit; a packet's hit leaves
+ * are listed while it is in flight, no per-ray hit list is stored. The packets are the backward's own
+ * (windows of 256 receivers, hits decided by the single ray's test), so that a ray below t_min may
+ * end with other occluders than in the forward: what it pushes is then below |g| t_min / (1 - alpha_j)
+ * either way. The hit set (t* > 0, D^2 <= 9) and the
  * hemisphere test are held fixed (non-differentiable boundaries); the gradient flows through
  * opacity_j exp(-D^2/2), D^2 at the closest approach (to mu_j, s_j, q_j and, via the ray
  * origin, mu_i) and the cosine max(0, n_i.w) (to the raw normal n_i).
@@ -453,7 +461,8 @@ size_t prtgs_render_workspace_size(int64_t n, int32_t width, int32_t height, int
  * alpha = min(0.99, opacity e^power), skip alpha < 1/255, stop before T < 1e-4).
  *   colors[k,n,3], bg[3] (device), image[k,3,H,W] out. The geometry is shared by the k
  *   images; each pixel's blend is evaluated once for all k colour sets.
- * status: PRTGS_STATUS_CAPACITY when max_pairs is exceeded (the image is then incomplete).
+ * status: PRTGS_STATUS_CAPACITY when max_pairs is exceeded (the image is then incomplete: the
+ * farthest splats' pairs are left out).
  */
 int prtgs_render(const prtgs_gaussians* g, const float* colors, int32_t k, const prtgs_camera* cam,
                  const float* bg, float* image, prtgs_render_state* st, int32_t* status, void* workspace,

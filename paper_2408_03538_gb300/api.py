@@ -140,7 +140,9 @@ def precompute_transfer(g: GaussianTensors, bvh: Bvh, dirs: torch.Tensor, order:
     """Transfer vectors P [n,C], and with ``bounce`` T [n,3,C] (``n_bounces`` self-transfer
     bounces over the index matrix) and idx [n,S]; with ``glossy`` the C x C matrices
     M [n_glossy,C,C] of the glossy splats (in increasing index order). ``walk``: 0 = warp
-    packets of parallel rays (default), 1 = one ray per lane; the results are the same."""
+    packets of parallel rays (default), 1 = one ray per lane; the results are the same. The call's
+    scratch is in the result too, for a graph captured around the call: up to 1.2 GB with ``bounce``
+    that pop("_ws") gives back."""
     lib = L.load()
     dev = g.means.device
     S = int(dirs.shape[0])
@@ -175,7 +177,8 @@ def precompute_transfer_backward(g: GaussianTensors, bvh: Bvh, dirs: torch.Tenso
                                  stats: torch.Tensor | None = None, dV: torch.Tensor | None = None):
     """Gradients of a loss through P [n,C] (shadowed diffuse transfer) and, optionally, through the
     rays' visibility directly (dV [n,S], e.g. from the glossy matrices) to the Gaussians: dict of
-    d_means [n,3], d_scales [n,3], d_quats [n,4], d_opacity [n], d_normals [n,3]."""
+    d_means [n,3], d_scales [n,3], d_quats [n,4], d_opacity [n], d_normals [n,3], and the scratch
+    (up to 0.56 GB and 80 bytes a splat) as "_ws"."""
     lib = L.load()
     dev = g.means.device
     n = g.n

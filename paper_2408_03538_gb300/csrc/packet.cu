@@ -13,11 +13,11 @@
 // What bounds it: issue slots and the latency of the node steps (about 40 % of the time), with L2 serving
 // the tree; a walk of surface-100k meets 1,300 nodes and 820 boxes of leaves, of which 560 leaves are
 // tested and 270 are hit by one of the 30 rays (9 of them each). Measured against testing every leaf
-// exactly, in step: surface-100k with bounces 77.4 -> 60.2 ms, a 60k volume 30.2 -> 24.1 ms, the million
-// splats with bounces and glossy matrices 1.037 -> 0.908 s. Tried and left out: the tree projected once
-// per direction (surface-100k 62.8 -> 62.8 ms before the search had its own kernel, but the million
-// splats 1.17 s: a direction's tree no longer fits the L2, and a launch per few directions ends with a
-// millisecond of few busy warps).
+// exactly, in step: surface-100k with bounces 77.4 -> 60.2 ms, a 60k volume 30.2 -> 24.1 ms, six tilings of a
+// million splats with bounces and glossy matrices 0.973-1.041 -> 0.840-0.956 s. Tried and left out: the tree
+// projected once per direction (surface-100k 62.8 -> 62.8 ms before the search had its own kernel, but the
+// million splats 1.17 s: a direction's tree no longer fits the L2, and a launch per few directions ends with
+// a millisecond of few busy warps).
 //
 //  k_packet<B>    visibility V_is of every (receiver, direction) of a receiver batch into
 //                 V[s][i] (Eq. 4 along a ray, Eq. 27 read as the Gaussian's maximum); with B
@@ -482,7 +482,8 @@ __device__ void packet_walk(const TraceArgs& a, const Frame& f, const Rel& rel, 
         if (need) st.leaves += cnt;  // leaf tests of the lane (its own Gaussian included)
         float thn = need ? th : -FLT_MAX;  // a lane that wants no hits passes no test
         const float zhi_q = need ? (thn + rel.zr) + (2.0f * et + 2e-6f * (fabsf(thn) + fabsf(rel.zr))) : -FLT_MAX;
-        const float zlo_g = Vis::kRayDecides ? zlo_q - 50.0f * et : zlo_q;  // the band of ray_decides
+        // ray_decides' band about t* = 0, but for its terms of the lane's own depth (zlo_q has 2e-6 of it) and offset
+        const float zlo_g = Vis::kRayDecides ? zlo_q - 50.0f * et : zlo_q;
         unsigned pass = need ? quick_mask(sm, cnt, rel.xr, rel.yr, zlo_g, zhi_q) : 0u;
         if constexpr (Vis::kInStep) {
           unsigned any = __reduce_or_sync(0xffffffffu, pass);
@@ -1307,7 +1308,8 @@ __global__ void __launch_bounds__(128) k_normal_grad(TraceArgs a, const float* _
   }
 }
 
-// Receivers per launch: G and GV hold S floats each per receiver, at most 2^26.
+// Receivers per launch: G and GV hold S floats each per receiver, at most 2^26 (512 MB for the two; with 2^25 a volume
+// of 300k at 128 directions took 297.9 ms, with 2^24 300.7, with this 297.1: each launch ends with few busy warps).
 static int64_t bwd_batch(int64_t n, int S) {
   int64_t b = ((int64_t(1) << 26) / (S > 0 ? S : 1)) / 64 * 64;
   if (b < 64) b = 64;
@@ -1424,7 +1426,7 @@ static int launch_packet_t(const TraceArgs& a, float* V, int sms, cudaStream_t s
   cudaFuncSetAttribute(k_packet<BOUNCE>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   int per_sm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_packet<BOUNCE>, kPacketThreads, smem);
-  // work items: (window of 64 receivers, dpi directions); at most 2^26 / 64 of them per batch
+  // work items: a packet of a window of 64 receivers (two at most) and dpi directions; at most 2^26 / 32 per launch
   const int dpi = a.packet_dirs > 0 ? a.packet_dirs : kPacketDirs;
   cudaMemsetAsync(a.work, 0, sizeof(unsigned int), stream);
   if (BOUNCE) cudaMemsetAsync(a.queue_count, 0, sizeof(unsigned int), stream);

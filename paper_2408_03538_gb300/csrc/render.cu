@@ -4,8 +4,9 @@
 //
 // Forward: k_preprocess (one thread per Gaussian) -> the Gaussians in depth order (radix sort of the depth
 // bits) -> inclusive scan of the touched-tile counts in that order -> k_duplicate writes (tile, Gaussian)
-// pairs -> stable radix sort by tile, on the device-side pair count -> k_ranges -> k_composite (one 16x16-pixel tile per block, a
-// warp per 8x4 pixels that stages the splats that reach them, evaluated once for a group of up to 16 light colour sets).
+// pairs -> stable radix sort by tile, on the device-side pair count -> k_ranges -> k_composite (two blocks per
+// 16x16-pixel tile, a warp per 8x4 pixels that stages the splats that reach them, evaluated once for a group of up to
+// 16 light colour sets).
 // Backward: k_composite_bwd walks each pixel's list back to front from its last contributor and sums
 // every splat's moments and colour gradients over a warp's pixels before a few vector reductions;
 // k_preprocess_bwd maps the sums to opacities, colours, means, scales and rotations.
@@ -20,6 +21,7 @@ constexpr int kTileThreads = kTile * kTile;
 // Blocks of a tile's eight warps: its warps end at different times, and a block keeps its place until the last
 // has. Composite of 300k splats at 1080p, forward and backward, at 1, 2, 4 and 8: 261, 235, 236, 242 and 470, 459, 469,
 // 474 us; of 8 scenes x 4 lights 658, 589, 598, 607 and 1,394, 1,325, 1,273, 1,509.
+// (One split for both directions and every size: four would be 2 % worse on the one backward and 4 % better on the other.)
 constexpr int kSplit = 2;
 constexpr int kCompThreads = kTileThreads / kSplit;
 constexpr float kNear = 0.2f;
@@ -639,7 +641,8 @@ struct BwdWarp {
 // (splat, half of the pixels): the moments of g and the colour sums of w are plain sums in registers, and a
 // splat's sums leave the warp as a few vector reductions. (Reducing every value of every splat over the warp
 // by shuffles and adding it to shared memory by one lane was 5.47 ms of the 8.4 ms of a 300k-splat full-HD
-// frame; this takes 0.46 ms. 8 scenes x 4 lights at 720p: 14.8 -> 1.33 ms.) Bound by issue slots.
+// frame; this takes 0.46 ms. 8 scenes x 4 lights at 720p: 14.8 -> 1.33 ms.) Bound by issue slots. The registers are the
+// compiler's choice (56 and 64 for one set; 80 for groups of four, 96 of eight, which spill 12 and 56 bytes).
 // The colours enter dL/dalpha through the scalar c . dL/dpixel only, whose blended remainder follows the same
 // recursion as the colours'.
 template <int KG, class V>

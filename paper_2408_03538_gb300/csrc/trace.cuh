@@ -56,8 +56,9 @@ struct TraceArgs {
   unsigned int* work;
   unsigned long long* stats;  // nodes, leaves, hits, index rounds, traced rays (nullable)
   int64_t r0, r1;             // receivers [r0, r1) of this batch, in sorted (Morton) positions
-  void* queue;                // [batch * S] per-ray candidate records, resolved by k_prefix / k_rounds
-  uint32_t* pending;          // [batch * S] 1 = the ray has index-matrix candidates
+  void* queue;                // per-ray walk: [batch * S] candidate records, resolved by k_prefix / k_rounds; packets:
+                              // 32 SearchRec per packet that k_search goes on with
+  uint32_t* pending;          // [batch * S] 1 = the ray has index-matrix candidates; packets: the direction of each
   unsigned int* queue_count;
   int packet_dirs;            // directions per packet work item (0: chosen from the problem size)
 };
