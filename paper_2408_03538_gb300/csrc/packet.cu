@@ -1132,7 +1132,7 @@ __global__ void __launch_bounds__(kPacketThreads, kBwdBlocks)
                 if (lane < 6 * nb) {
                   const float4* r4 = reinterpret_cast<const float4*>(bs.row[lane]);
                   float4 v = r4[0];
-  #pragma unroll
+#pragma unroll
                   for (int i = 1; i < 8; ++i) {
                     const float4 u = r4[i];
                     v.x += u.x;
