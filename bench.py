@@ -405,6 +405,8 @@ def transfer_traffic_bytes(workload, traced_rays):
     """DRAM bytes per launch of the dominant transfer kernel, from the committed ncu summary of
     the current kernel sources: the per-traced-ray figure of the capture times the traced rays of
     one launch here. None when the summary is absent or was measured on other sources."""
+    if workload != WORKLOAD:  # the capture's; a smaller tree lies in the L2
+        return None
     p = os.path.join(ROOT, "profiles", "dram_transfer_packet.md")
     vals = {}
     try:
@@ -510,9 +512,9 @@ def run_kernels_small():
 
 def run_transfer_traffic(args):
     """The transfer of the bench workload (shadow + bounce, no glossy matrices) called twice, for
-    a one-pass ncu capture of the DRAM bytes of the second call's k_packet launches. Prints the
-    traced rays and the receiver batches (k_packet launches) of a call and the kernel sources'
-    hash, which the committed summary records."""
+    a one-pass ncu capture of the DRAM bytes of the second call's k_packet and k_search launches.
+    Prints the traced rays and the parts (launches of either kernel) of a call and the kernel
+    sources' hash, which the committed summary records."""
     import torch
 
     from paper_2408_03538_gb300 import api, scenes as S
@@ -525,9 +527,11 @@ def run_transfer_traffic(args):
         api.precompute_transfer(g, bvh, dirs, w["order"], bounce=True)
     torch.cuda.synchronize()
     traced = int((sc.normals.astype(np.float64) @ dirs_np.astype(np.float64).T > 0).sum())
-    batch = max(32, ((1 << 26) // dirs_np.shape[0]) // 32 * 32)
+    part = lambda rays: max(64, rays // dirs_np.shape[0] // 64 * 64)  # receivers of a batch, and of a part of it
+    whole = [min(part(1 << 26), sc.n - b) for b in range(0, sc.n, part(1 << 26))]
     print(json.dumps({"case": "transfer-traffic", "workload": sc.n, "traced_rays_per_call": traced,
-                      "k_packet_launches_per_call": math.ceil(sc.n / batch), "source_sha16": source_sha16()}))
+                      "k_packet_launches_per_call": sum(math.ceil(b / part(1 << 25)) for b in whole),
+                      "source_sha16": source_sha16()}))
 
 
 # Flops of one BRDF kernel evaluation in the training transfer (brdf.cuh: three TwoSums, three
