@@ -615,10 +615,14 @@ int render_batched(const prtgs_gaussians* g, const int64_t* offsets, int32_t B, 
 }
 
 // ---- backward ------------------------------------------------------------------------------
-// Sums of one splat, accumulated over the pixels and kept until k_preprocess_bwd: with g = dL/dpower and
-// d = mean2d - pixel, sum g, g dx, g dy, g dx^2, g dx dy, g dy^2 (which give the gradients of opacity, mean2d
-// and conic), then sum alpha T dL/dpixel per colour channel, each group of KG colour sets on a 16-byte
-// boundary.
+// Sums of one splat, accumulated over the pixels and kept until k_preprocess_bwd: with g = dL/dpower, K the conic
+// and (u, v) = K (mean2d - pixel), sum g, g u, g v, g u^2, g u v, g v^2, then sum alpha T dL/dpixel per colour
+// channel, each group of KG colour sets on a 16-byte boundary. Power is -(K d).d / 2, so dL/dmean2d = -sum g (u, v)
+// and dL/dcov = sum g (u, v)(u, v)^T / 2. Of sums of g d and g d d^T, in which a needle's long axis is large, both
+// gradients would be what is left after it cancels: with scales that differ by e^1.4 at random (900 splats, 160 x 90,
+// geometric mean of six scenes, one colour set) the errors against 64 bits of means, scales and rotations were 1.6e-3,
+// 1.6e-3 and 3.0e-3 that way, 1.1e-3, 1.2e-3 and 2.2e-3 with K d and d d^T summed pixel by pixel, and are 8e-5, 1.2e-4
+// and 1.4e-4 like this.
 constexpr int kMoments = 8;  // six sums, padded
 static int bwd_group(int k) { return k <= 1 ? 1 : (k <= 4 ? 4 : 8); }
 static int bwd_stride(int k) { return kMoments + color_floats(bwd_group(k)) * ((k + bwd_group(k) - 1) / bwd_group(k)); }
@@ -641,12 +645,13 @@ struct BwdWarp {
 // (splat, half of the pixels): the moments of g and the colour sums of w are plain sums in registers, and a
 // splat's sums leave the warp as a few vector reductions. (Reducing every value of every splat over the warp
 // by shuffles and adding it to shared memory by one lane was 5.47 ms of the 8.4 ms of a 300k-splat full-HD
-// frame; this takes 0.46 ms. 8 scenes x 4 lights at 720p: 14.8 -> 1.33 ms.) Bound by issue slots. The registers are the
-// compiler's choice (56 and 64 for one set; 80 for groups of four, 96 of eight, which spill 12 and 56 bytes).
+// frame; this takes 0.46 ms. 8 scenes x 4 lights at 720p: 14.8 -> 1.33 ms.) Bound by issue slots. The bounds
+// leave 56 registers for one set (its own choice), 80 for groups of four and 96 of eight, which spill 12 and 28 bytes: 3 sets
+// of 300k splats 688 us a call with 6 blocks, 708 with 5, 732 with 7; 8 sets 1,089 with 5, 1,245 with 6, 1,122 unbounded.
 // The colours enter dL/dalpha through the scalar c . dL/dpixel only, whose blended remainder follows the same
 // recursion as the colours'.
 template <int KG, class V>
-__global__ void __launch_bounds__(kCompThreads) k_composite_bwd(
+__global__ void __launch_bounds__(kCompThreads, KG == 1 ? 0 : KG == 4 ? 6 : 5) k_composite_bwd(
     V v, const uint32_t* __restrict__ ranges, const int32_t* __restrict__ ids, const float* __restrict__ mean2d,
     const float4* __restrict__ conic_op, const float* __restrict__ colors, int64_t n, int k,
     const float* __restrict__ bg, const float* __restrict__ final_T, const int32_t* __restrict__ n_contrib,
@@ -745,33 +750,46 @@ __global__ void __launch_bounds__(kCompThreads) k_composite_bwd(
       }
       __syncwarp();
       const int i = lane & (kBwdChunk - 1), half = lane >> 4;
-      float m0 = 0.f, mx = 0.f, my = 0.f, mxx = 0.f, mxy = 0.f, myy = 0.f;
+      float m0 = 0.f, mx = 0.f, my = 0.f, mxx = 0.f, mxy = 0.f, myy = 0.f;  // of u and v
       float cs[CF];
 #pragma unroll
       for (int e = 0; e < CF; ++e) cs[e] = 0.f;
       if (i < cnt) {
-        const float4 q = sm.xy[c0 + i];
+        const float4 q = sm.xy[c0 + i], o = sm.co[c0 + i];
         const float x0 = q.x - (float)bx, y0 = q.y - (float)(by + 2 * half);
+        // along a row v = rho u + tau, so that the sums with v follow from the row's sums with u
+        const float rho = __fdividef(o.y, o.x), dv = fmaf(-rho, o.y, o.z);
+        float u0 = fmaf(o.x, x0, o.y * y0), tau = dv * y0;  // at the half's first pixel
 #pragma unroll
-        for (int r = 0; r < 16; ++r) {
-          const int at = 16 * half + r;
-          const float g = sm.g[i][at], w = sm.w[i][at];
-          const float dx = x0 - (float)(r & 7), dy = y0 - (float)(r >> 3);
-          const float gx = g * dx, gy = g * dy;
-          m0 += g;
-          mx += gx;
-          my += gy;
-          mxx = fmaf(gx, dx, mxx);
-          mxy = fmaf(gx, dy, mxy);
-          myy = fmaf(gy, dy, myy);
+        for (int row = 0; row < 2; ++row) {
+          float s0 = 0.f, su = 0.f, suu = 0.f;
 #pragma unroll
-          for (int e = 0; e < CF; e += 4) {
-            const float4 d = *reinterpret_cast<const float4*>(&sm.dpix[at][e]);
-            cs[e] = fmaf(w, d.x, cs[e]);
-            cs[e + 1] = fmaf(w, d.y, cs[e + 1]);
-            cs[e + 2] = fmaf(w, d.z, cs[e + 2]);
-            if (e + 3 < 3 * KG) cs[e + 3] = fmaf(w, d.w, cs[e + 3]);
+          for (int r = 0; r < 8; ++r) {
+            const int at = 16 * half + 8 * row + r;
+            const float g = sm.g[i][at], w = sm.w[i][at];
+            const float u = fmaf(-(float)r, o.x, u0);
+            const float gu = g * u;
+            s0 += g;
+            su += gu;
+            suu = fmaf(gu, u, suu);
+#pragma unroll
+            for (int e = 0; e < CF; e += 4) {
+              const float4 d = *reinterpret_cast<const float4*>(&sm.dpix[at][e]);
+              cs[e] = fmaf(w, d.x, cs[e]);
+              cs[e + 1] = fmaf(w, d.y, cs[e + 1]);
+              cs[e + 2] = fmaf(w, d.z, cs[e + 2]);
+              if (e + 3 < 3 * KG) cs[e + 3] = fmaf(w, d.w, cs[e + 3]);
+            }
           }
+          const float sv = fmaf(rho, su, tau * s0), suv = fmaf(rho, suu, tau * su);
+          m0 += s0;
+          mx += su;
+          my += sv;
+          mxx += suu;
+          mxy += suv;
+          myy += fmaf(rho, suv, tau * sv);
+          u0 -= o.y;
+          tau -= dv;
         }
       }
       m0 += __shfl_xor_sync(0xffffffffu, m0, 16);
@@ -821,15 +839,9 @@ __global__ void k_preprocess_bwd(int64_t n, const float* __restrict__ means, con
     out[1] = cs[1];
     out[2] = cs[2];
   }
-  // dL/dmean2d = -(conic d) g, dL/dconic = -(dx^2, 2 dx dy, dy^2) g / 2, dL/dopacity = g / opacity
   const float4 ma = *reinterpret_cast<const float4*>(sums), mb = *reinterpret_cast<const float4*>(sums + 4);
-  float gmx = 0.f, gmy = 0.f, gop = 0.f;
-  if (radius[i] > 0 && (ma.x != 0.f || ma.y != 0.f || ma.z != 0.f)) {
-    const float4 co = conic_op[i];
-    gmx = -(co.x * ma.y + co.y * ma.z);
-    gmy = -(co.z * ma.z + co.y * ma.y);
-    gop = ma.x / co.w;
-  }
+  const float gmx = -ma.y, gmy = -ma.z;
+  const float gop = radius[i] > 0 && ma.x != 0.f ? ma.x / conic_op[i].w : 0.f;  // dL/dopacity = sum g / opacity
   d_opacity[i] = gop;
   float gm[3] = {0.f, 0.f, 0.f}, gs[3] = {0.f, 0.f, 0.f}, gq[4] = {0.f, 0.f, 0.f, 0.f};
   if (radius[i] > 0) {
@@ -856,33 +868,8 @@ __global__ void k_preprocess_bwd(int64_t n, const float* __restrict__ means, con
     float M[2][3];
     for (int a = 0; a < 2; ++a)
       for (int k2 = 0; k2 < 3; ++k2) M[a][k2] = J[a][0] * W[0][k2] + J[a][1] * W[1][k2] + J[a][2] * W[2][k2];
-    float cov[2][2];
-    for (int a = 0; a < 2; ++a)
-      for (int b = 0; b < 2; ++b) {
-        float acc = 0.f;
-        for (int p = 0; p < 3; ++p)
-          for (int q = 0; q < 3; ++q) acc += M[a][p] * Sm[p][q] * M[b][q];
-        cov[a][b] = acc;
-      }
-    const float A = cov[0][0] + kDilation, B = cov[0][1], Cc = cov[1][1] + kDilation;
-    const float det = A * Cc - B * B;
-    const float id2 = 1.0f / (det * det);
-    const float gA = -0.5f * ma.w, gB = -mb.x, gC = -0.5f * mb.y;
-    // conic = (C/det, -B/det, A/det)
-    const float dA = id2 * (-Cc * Cc * gA + B * Cc * gB - B * B * gC);
-    const float dC = id2 * (-B * B * gA + A * B * gB - A * A * gC);
-    const float dB = id2 * (2.f * B * Cc * gA - (det + 2.f * B * B) * gB + 2.f * A * B * gC);
-    // symmetric gradient of cov2 (B is read from the 01 entry once)
-    const float G2[2][2] = {{dA, 0.5f * dB}, {0.5f * dB, dC}};
-    // dSigma = M^T G2 M
-    float dS[3][3];
-    for (int p = 0; p < 3; ++p)
-      for (int q = 0; q < 3; ++q) {
-        float acc = 0.f;
-        for (int a = 0; a < 2; ++a)
-          for (int b = 0; b < 2; ++b) acc += M[a][p] * G2[a][b] * M[b][q];
-        dS[p][q] = acc;
-      }
+    // dL/dcov2
+    const float G2[2][2] = {{0.5f * ma.w, 0.5f * mb.x}, {0.5f * mb.x, 0.5f * mb.y}};
     // dM = 2 G2 M Sigma ; dJ = dM W^T
     float dM[2][3];
     for (int a = 0; a < 2; ++a)
@@ -915,18 +902,16 @@ __global__ void k_preprocess_bwd(int64_t n, const float* __restrict__ means, con
     }
     // world-space: p = W mu + t
     for (int k2 = 0; k2 < 3; ++k2) gm[k2] = W[0][k2] * gx + W[1][k2] * gy + W[2][k2] * gz;
-    // Sigma = R diag(s^2) R^T. With G = R^T dSigma R: dL/ds_k = 2 s_k G_kk, and a rotation by theta about the
-    // local axes, R exp([theta]x), changes L by tau . theta, tau_1 = 2 G_23 (s_2^2 - s_3^2) and cyclic (exactly 0
-    // for equal scales, where the chain through dL/dR leaves its rounding). On the unit quaternion that is
+    // cov2 = N diag(s^2) N^T with N = M R. With G = N^T G2 N (= R^T dSigma R): dL/ds_k = 2 s_k G_kk, and a rotation by
+    // theta about the local axes, R exp([theta]x), changes L by tau . theta, tau_1 = 2 G_23 (s_2^2 - s_3^2) and cyclic
+    // (exactly 0 for equal scales, where the chain through dL/dR leaves its rounding). On the unit quaternion that is
     // 2 (tau_1 q i + tau_2 q j + tau_3 q k).
-    float G[3][3];
+    float N[2][3], G[3][3];
+    for (int a = 0; a < 2; ++a)
+      for (int k2 = 0; k2 < 3; ++k2) N[a][k2] = M[a][0] * R[0][k2] + M[a][1] * R[1][k2] + M[a][2] * R[2][k2];
     for (int a = 0; a < 3; ++a)
-      for (int k2 = 0; k2 < 3; ++k2) {
-        float acc = 0.f;
-        for (int p = 0; p < 3; ++p)
-          for (int q = 0; q < 3; ++q) acc += R[p][a] * dS[p][q] * R[q][k2];
-        G[a][k2] = acc;
-      }
+      for (int k2 = 0; k2 < 3; ++k2)
+        G[a][k2] = N[0][a] * (G2[0][0] * N[0][k2] + G2[0][1] * N[1][k2]) + N[1][a] * (G2[1][0] * N[0][k2] + G2[1][1] * N[1][k2]);
     for (int k2 = 0; k2 < 3; ++k2) gs[k2] = 2.f * s[k2] * G[k2][k2];
     const float t1 = 2.f * (G[1][2] + G[2][1]) * ((s[1] - s[2]) * (s[1] + s[2])) / qn;
     const float t2 = 2.f * (G[0][2] + G[2][0]) * ((s[2] - s[0]) * (s[2] + s[0])) / qn;

@@ -131,3 +131,16 @@ def test_color_groups_and_rows_agree(w, h, k):
     assert st.read() == 0 and torch.equal(tight, img)
     _, normal, _ = api.render_geometry(g, cam, max_pairs=400_000)
     assert torch.equal(normal, img[1])
+
+
+@pytest.mark.parametrize("seed", [0, 1, 2])
+@pytest.mark.parametrize("k", [1, 3])
+def test_needle_gradients(seed, k):
+    """Scales that differ by e^1.4 at random, in any direction: along a needle's long axis the offsets of its pixels
+    are large and what they add to the gradients small."""
+    sc, rng = S.isotropic_scene(900, 10 + seed), np.random.default_rng(seed)
+    sc.scales = (1.6 * sc.scales * np.exp(rng.normal(0, 1.4, sc.scales.shape))).astype(np.float32)
+    q = rng.normal(size=(sc.n, 4))
+    sc.quats = (q / np.linalg.norm(q, axis=1, keepdims=True)).astype(np.float32)
+    sc.opacity = np.clip(sc.opacity * (1 + seed), 0, 0.99).astype(np.float32)
+    _check(sc, S.look_at_camera((0, -4.0, 1.5), (0, 0, 0), 50, 160, 90), k, (0.2, 0.2, 0.2))
