@@ -239,7 +239,7 @@ int prtgs_precompute_transfer(const prtgs_gaussians* g, const prtgs_bvh* bvh, co
  *                overwritten; accumulated with float atomics, so the last bits vary run to run)
  * p->flags must be PRTGS_SHADOW or 0 (unshadowed: only d_normals is non-zero); PRTGS_BOUNCE or
  * PRTGS_GLOSSY -> PRTGS_ERR_UNSUPPORTED. The bvh must have been built from the same g.
- * Errors: as prtgs_precompute_transfer. The workspace (up to 0.56 GB and 80 bytes a Gaussian: two floats per
+ * Errors: as prtgs_precompute_transfer. The workspace (up to 0.56 GB and 96 bytes a Gaussian: two floats per
  * ray of at most 2^26 at a time, the sums, and the lists of the packets in flight) depends on n, the directions
  * and the order alone.
  */

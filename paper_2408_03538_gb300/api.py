@@ -178,7 +178,7 @@ def precompute_transfer_backward(g: GaussianTensors, bvh: Bvh, dirs: torch.Tenso
     """Gradients of a loss through P [n,C] (shadowed diffuse transfer) and, optionally, through the
     rays' visibility directly (dV [n,S], e.g. from the glossy matrices) to the Gaussians: dict of
     d_means [n,3], d_scales [n,3], d_quats [n,4], d_opacity [n], d_normals [n,3], and the scratch
-    (up to 0.56 GB and 80 bytes a splat) as "_ws"."""
+    (up to 0.56 GB and 96 bytes a splat) as "_ws"."""
     lib = L.load()
     dev = g.means.device
     n = g.n

@@ -407,7 +407,7 @@ int precompute_transfer_backward(const prtgs_gaussians* gs, const prtgs_bvh* bvh
   a.status = status;
   a.work = work;
   a.stats = p->stats;
-  return launch_packet_bwd(a, gs->quats, dP, dV, d_means, d_scales, d_quats, d_opacity, d_normals,
+  return launch_packet_bwd(a, gs->scales, gs->quats, dP, dV, d_means, d_scales, d_quats, d_opacity, d_normals,
                            static_cast<char*>(ws) + c.off, device_sms(), stream);
 }
 

@@ -107,3 +107,23 @@ def test_second_batch_of_receivers():
     for f in ("means", "scales", "opacity", "normals"):  # (round splats: the rotation gradient is 0 but for rounding)
         ref = 0.5 * (parts[0]["d_" + f].double() + parts[1]["d_" + f].double())
         assert float((whole["d_" + f].double() - ref).norm()) <= 1e-5 * float(ref.norm()), f
+
+
+@pytest.mark.parametrize("seed", [0, 1, 2])
+def test_normal_gradient_of_many_directions(seed):
+    """512 directions of few hits each: a term g V w_s has some six roundings of 2^-25 on average, 2^-23 at most in
+    all but rare terms, and sums over the directions keep that: 2^-23 norm-wise. A sum in 32 bits adds twice as much."""
+    from oracle import transfer_torch as TT
+
+    rng, n, dirs = np.random.default_rng(seed), 500, 512
+    sc = S.isotropic_scene(n, 20 + seed)
+    sc.means *= np.float32(3.0)
+    sc.scales = (0.6 * sc.scales * np.exp(rng.normal(0, 0.3, sc.scales.shape))).astype(np.float32)
+    d, w = S.direction_set(dirs, 3), rng.standard_normal((n, 9)).astype(np.float32)
+    g = api.GaussianTensors.from_scene(sc)
+    got = api.precompute_transfer_backward(g, api.build_bvh(g), torch.from_numpy(d).cuda(), 2,
+                                           torch.from_numpy(w).cuda(), t_min=0.0)["d_normals"].cpu().double()
+    f64 = [torch.tensor(np.asarray(getattr(sc, f), np.float64)) for f in FIELDS]
+    V = TT.transfer_V(*f64, d).numpy()
+    ref = torch.tensor((4 * np.pi / dirs * (w.astype(np.float64) @ oracle.sh(2, d).T) * V) @ d.astype(np.float64))
+    assert float((got - ref).norm()) <= 2.0 ** -23 * float(ref.norm())

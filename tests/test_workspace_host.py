@@ -17,4 +17,4 @@ def test_transfer_backward_size_does_not_depend_on_the_device(n, S):
     got = L.load().prtgs_transfer_backward_workspace_size(n, ctypes.byref(p))
     batch = min(n, max(2**26 // S // 64 * 64, 64))
     blocks = min(152 * 4, max(1, (8 * -(-batch // 256) * S + 3) // 4))  # 4 per SM, or a warp per packet
-    assert got == 256 + 2 * _up(4 * batch * S) + _up(80 * n) + _up(4 * blocks * 4 * 2048)
+    assert got == 256 + 2 * _up(4 * batch * S) + _up(96 * n) + _up(4 * blocks * 4 * 2048)
