@@ -56,8 +56,9 @@ struct TraceArgs;
 int launch_packet(const TraceArgs& a, float* V, bool bounce, int sms, cudaStream_t stream);
 size_t packet_search_bytes(int64_t batch, int S);
 size_t packet_bwd_workspace(int64_t n, int S);
-int launch_packet_bwd(TraceArgs a, const float* scales, const float* quats, const float* dP, const float* dV, float* d_means, float* d_scales,
-                      float* d_quats, float* d_opacity, float* d_normals, void* ws, int sms, cudaStream_t stream);
+int launch_packet_bwd(TraceArgs a, const float* scales, const float* quats, const float* dP, const float* dV,
+                      float* d_means, float* d_scales, float* d_quats, float* d_opacity, float* d_normals, void* ws, int sms,
+                      cudaStream_t stream);
 
 size_t transfer_backward_workspace(int64_t n, const prtgs_transfer_params* p);
 // dP [n,C] and dV [n,S] (extra dLoss/dV per ray, e.g. from the glossy matrices) are both nullable

@@ -1345,8 +1345,9 @@ size_t packet_bwd_workspace(int64_t n, int S) {
          align_up(sizeof(int) * (size_t)bwd_blocks(n, S) * kPacketWarps * kBwdList);
 }
 
-int launch_packet_bwd(TraceArgs a, const float* scales, const float* quats, const float* dP, const float* dV, float* d_means, float* d_scales,
-                      float* d_quats, float* d_opacity, float* d_normals, void* ws, int sms, cudaStream_t stream) {
+int launch_packet_bwd(TraceArgs a, const float* scales, const float* quats, const float* dP, const float* dV,
+                      float* d_means, float* d_scales, float* d_quats, float* d_opacity, float* d_normals, void* ws, int sms,
+                      cudaStream_t stream) {
   if (!(a.flags & PRTGS_SHADOW)) {
     cudaMemsetAsync(d_means, 0, sizeof(float) * 3 * a.n, stream);
     cudaMemsetAsync(d_scales, 0, sizeof(float) * 3 * a.n, stream);

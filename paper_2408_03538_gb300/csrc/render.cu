@@ -758,7 +758,7 @@ __global__ void __launch_bounds__(kCompThreads, KG == 1 ? 0 : KG == 4 ? 6 : 5) k
         const float4 q = sm.xy[c0 + i], o = sm.co[c0 + i];
         const float x0 = q.x - (float)bx, y0 = q.y - (float)(by + 2 * half);
         // along a row v = rho u + tau, so that the sums with v follow from the row's sums with u
-        const float rho = __fdividef(o.y, o.x), dv = fmaf(-rho, o.y, o.z);
+        const float rho = o.x > 0.f ? __fdividef(o.y, o.x) : 0.f, dv = fmaf(-rho, o.y, o.z);  // (0: a form that underflowed)
         float u0 = fmaf(o.x, x0, o.y * y0), tau = dv * y0;  // at the half's first pixel
 #pragma unroll
         for (int row = 0; row < 2; ++row) {
