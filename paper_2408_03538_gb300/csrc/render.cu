@@ -19,9 +19,9 @@ namespace prtgs {
 constexpr int kTile = 16;
 constexpr int kTileThreads = kTile * kTile;
 // Blocks of a tile's eight warps: its warps end at different times, and a block keeps its place until the last
-// has. Composite of 300k splats at 1080p, forward and backward, at 1, 2, 4 and 8: 261, 235, 236, 242 and 470, 459, 469,
-// 474 us; of 8 scenes x 4 lights 658, 589, 598, 607 and 1,394, 1,325, 1,273, 1,509.
-// (One split for both directions and every size: four would be 2 % worse on the one backward and 4 % better on the other.)
+// has. Composite of 300k splats at 1080p, forward and backward, at 1, 2, 4 and 8: 228, 221, 224, 239 and 463, 449, 457,
+// 466 us; of 8 scenes x 4 lights 596, 570, 579, 594 and 2,150, 1,244, 1,535, 1,612 (the backward's register bounds being
+// those for two).
 constexpr int kSplit = 2;
 constexpr int kCompThreads = kTileThreads / kSplit;
 constexpr float kNear = 0.2f;
@@ -645,7 +645,7 @@ struct BwdWarp {
 // (splat, half of the pixels): the moments of g and the colour sums of w are plain sums in registers, and a
 // splat's sums leave the warp as a few vector reductions. (Reducing every value of every splat over the warp
 // by shuffles and adding it to shared memory by one lane was 5.47 ms of the 8.4 ms of a 300k-splat full-HD
-// frame; this takes 0.46 ms. 8 scenes x 4 lights at 720p: 14.8 -> 1.33 ms.) Bound by issue slots. The bounds
+// frame; this takes 0.45 ms. 8 scenes x 4 lights at 720p: 14.8 -> 1.24 ms.) Bound by issue slots. The bounds
 // leave 56 registers for one set (its own choice), 80 for groups of four and 96 of eight, which spill 12 and 28 bytes: 3 sets
 // of 300k splats 688 us a call with 6 blocks, 708 with 5, 732 with 7; 8 sets 1,089 with 5, 1,245 with 6, 1,122 unbounded.
 // The colours enter dL/dalpha through the scalar c . dL/dpixel only, whose blended remainder follows the same
