@@ -352,7 +352,7 @@ def run_surface(args):
     if hits_per_ray is not None:
         flops = traced * (hits_per_ray * 40.0 + 2.0 * C)
         achieved = flops / (transfer_ms / args.steps / 1e3) / 1e12
-        roof = {"bound": "alu", "kernel": "transfer call: k_packet<true>, k_project, k_bounce", "achieved": achieved,
+        roof = {"bound": "alu", "kernel": "transfer call: k_packet<true>, k_search, k_project, k_bounce", "achieved": achieved,
                 "peak": alu_peak, "unit": "TFLOP/s", "frac": achieved / alu_peak,
                 "traffic": transfer_traffic_bytes(SURFACE, traced),
                 "peak_source": f"{sms} SMs x 128 FP32 lanes x 2 flop x {sm_max:.0f} MHz ({pk_kind} max clock)",
@@ -1157,7 +1157,7 @@ def run_tiled(args):
     if hits_per_ray is not None:
         flops = traced * (hits_per_ray * 40.0 + 2.0 * C)
         achieved = flops / (walk_ms / 1e3) / 1e12
-        roof = {"bound": "alu", "kernel": "k_packet<true> (visibility walk + index matrix; with k_project and "
+        roof = {"bound": "alu", "kernel": "k_packet<true> and k_search (visibility walk, index matrix; with k_project and "
                                           "k_bounce, one transfer call without the glossy matrices)",
                 "achieved": achieved, "peak": alu_peak, "unit": "TFLOP/s", "frac": achieved / alu_peak,
                 "traffic": transfer_traffic_bytes(WORKLOAD, traced),
